@@ -12,6 +12,7 @@
 #include <cuda_bf16.h>
 
 #include "common.cuh"
+#include "softf64.cuh"
 
 namespace hwfv1 {
 
@@ -1358,7 +1359,7 @@ struct Phys {
 template <typename T>
 __device__ __forceinline__ void velocity(const Cell<T>& c, T tol, T& u, T& v) {
     if (ge_nonneg(c.h, tol)) {                         // h >= tol (tol > 0)
-        const T rh = T(1) / c.h;
+        const T rh = recip(c.h);
         u = c.qx * rh;
         v = c.qy * rh;
     } else {
@@ -1391,7 +1392,7 @@ __device__ __forceinline__ void hll_face(T g, T hg, T tol, T hL, T zL, T unL, T 
         F[0] = F[1] = F[2] = T(0);
         return;
     }
-    const T aL = sqrt(g * hLs), aR = sqrt(g * hRs);
+    const T aL = root(g * hLs), aR = root(g * hRs);
     T SL, SR;
     if (!is_zero(hLs) && !is_zero(hRs)) {
         const T us = half(unL + unR) + aL - aR;
@@ -1416,7 +1417,7 @@ __device__ __forceinline__ void hll_face(T g, T hg, T tol, T hL, T zL, T unL, T 
     } else if (le_zero(SR)) {
         F[0] = FR0; F[1] = FR1; F[2] = FR2;
     } else {
-        const T inv = T(1) / (SR - SL);
+        const T inv = recip(SR - SL);
         F[0] = (SR * FL0 - SL * FR0 + SL * SR * (hRs - hLs)) * inv;
         F[1] = (SR * FL1 - SL * FR1 + SL * SR * (qnR - qnL)) * inv;
         F[2] = (SR * FL2 - SL * FR2 + SL * SR * (qtR - qtL)) * inv;
@@ -1516,12 +1517,12 @@ __device__ __forceinline__ void cell_update_faces_sq(const Phys<T>& P, T rx, T r
         qx = T(0);
         qy = T(0);
     } else if (P.nM > T(0)) {
-        const T rh = T(1) / h;
+        const T rh = recip(h);
         if (rh_out) *rh_out = rh;
         const T u = qx * rh, v = qy * rh;
-        const T speed = sqrt(u * u + v * v);
+        const T speed = root(u * u + v * v);
         const T D = T(1) + friction_term(fk * speed, h, rh);
-        const T rD = T(1) / D;
+        const T rD = recip(D);
         qx = qx * rD;
         qy = qy * rD;
     }
@@ -1545,9 +1546,9 @@ __device__ __forceinline__ void cell_update_faces(const Phys<T>& P, T rx, T ry, 
 template <typename T>
 __device__ __forceinline__ T cfl_bound(const Phys<T>& P, T h, T qx, T qy) {
     if (!ge_nonneg(h, P.tol)) return T(INFINITY);      // h < tol (tol > 0)
-    const T rh = T(1) / h;
+    const T rh = recip(h);
     const T u = absval(qx * rh), v = absval(qy * rh);
-    const T a = sqrt(P.g * h);
+    const T a = root(P.g * h);
     const T rx = P.dxL / (u + a), ry = P.dyL / (v + a);
     return sel_min(rx, ry);
 }
@@ -1786,9 +1787,9 @@ __device__ __forceinline__ void wet_leaf_store(const StepArgs<T>& a, DevState* s
         // per step from their maxima, finish_body); the same operations as
         // cfl_bound up to the division, reusing the friction step's 1/h
         if (ge_nonneg(out[0], a.P.tol)) {
-            const T rh = is_zero(rh_known) ? T(1) / out[0] : rh_known;
+            const T rh = is_zero(rh_known) ? recip(out[0]) : rh_known;
             const T u = absval(out[1] * rh), v = absval(out[2] * rh);
-            const T aa = sqrt(a.P.g * out[0]);
+            const T aa = root(a.P.g * out[0]);
             const unsigned long long bx = abs_obits(u + aa), by = abs_obits(v + aa);
             spd[0] = bx > spd[0] ? bx : spd[0];
             spd[1] = by > spd[1] ? by : spd[1];
