@@ -119,11 +119,10 @@ static __global__ void __launch_bounds__(256) kb_fv1_dry(const DomainPlan<T>* P,
     fv1_dry_body<T>(a, domain_blk(base, d));
 }
 
-// the shared-face pair of the single-domain path (float64; float32 domains
-// have no face buffer and take the one-pass update inside kb_fv1_update),
-// launched, as there, in 64-thread blocks
+// the shared-face pair of the single-domain path (float64), and the one-pass
+// update of the leaves it leaves out (float32: all of them)
 template <typename T>
-static __global__ void __launch_bounds__(64) kb_fv1_faces(const DomainPlan<T>* P, const uint32_t* base, int D) {
+static __global__ void __launch_bounds__(128) kb_fv1_faces(const DomainPlan<T>* P, const uint32_t* base, int D) {
     const int d = find_domain(base, D, blockIdx.x);
     const StepArgs<T> a = P[d].step;
     fv1_faces_body<T>(a, domain_blk(base, d));
@@ -134,6 +133,13 @@ static __global__ void __launch_bounds__(64) kb_fv1_update(const DomainPlan<T>* 
     const int d = find_domain(base, D, blockIdx.x);
     const StepArgs<T> a = P[d].step;
     fv1_update_body<T>(a, domain_blk(base, d));
+}
+
+template <typename T>
+static __global__ void __launch_bounds__(64) kb_fv1_wet(const DomainPlan<T>* P, const uint32_t* base, int D) {
+    const int d = find_domain(base, D, blockIdx.x);
+    const StepArgs<T> a = P[d].step;
+    fv1_wet_body<T>(a, domain_blk(base, d));
 }
 
 template <typename T>
@@ -312,10 +318,17 @@ class BatchT final : public Batch {
         cudaMemcpyAsync(d_bases_, bases.data(), sizeof(uint32_t) * bases.size(), cudaMemcpyHostToDevice, stream_);
         launches_ = 0;
         for (int k = 0; k < BK_KINDS; ++k) launches_ += total_[k] > 0 ? 1 : 0;
-        if (total_[BK_WET] > 0) launches_ += 1;        // the wet update is two kernels
+        // the wet update: the face pair (float64), the one-pass kernel where needed
+        if (total_[BK_WET] > 0) launches_ += (sizeof(T) == 8 ? 2 : 0) + (one_pass() ? 1 : 0) - 1;
         return check("batch plan", true);
     }
 
+    // some member's queue can outgrow its face buffer (float32 has none)
+    bool one_pass() const {
+        for (const auto* e : doms_)
+            if (e->outgrows_faces()) return true;
+        return false;
+    }
     const uint32_t* base(int kind) const { return d_bases_ + (size_t)kind * (doms_.size() + 1); }
 
     void launch_step() {
@@ -329,8 +342,11 @@ class BatchT final : public Batch {
         kb_trav_scan<T><<<total_[BK_TSCAN], 1024, 0, stream_>>>(d_plans_, base(BK_TSCAN), D);
         kb_trav_write<T><<<total_[BK_TWRITE], 256, 0, stream_>>>(d_plans_, base(BK_TWRITE), D);
         kb_fv1_dry<T><<<total_[BK_DRY], 256, 0, stream_>>>(d_plans_, base(BK_DRY), D);
-        kb_fv1_faces<T><<<total_[BK_WET], 64, 0, stream_>>>(d_plans_, base(BK_WET), D);
-        kb_fv1_update<T><<<total_[BK_WET], 64, 0, stream_>>>(d_plans_, base(BK_WET), D);
+        if constexpr (sizeof(T) == 8) {
+            kb_fv1_faces<T><<<total_[BK_WET], 128, 0, stream_>>>(d_plans_, base(BK_WET), D);
+            kb_fv1_update<T><<<total_[BK_WET], 64, 0, stream_>>>(d_plans_, base(BK_WET), D);
+        }
+        if (one_pass()) kb_fv1_wet<T><<<total_[BK_WET], 64, 0, stream_>>>(d_plans_, base(BK_WET), D);
         kb_decode<T><<<total_[BK_DEC], 256, 0, stream_>>>(d_plans_, base(BK_DEC), D);
         kb_finish<T><<<D, 64, 0, stream_>>>(d_plans_, D);
     }

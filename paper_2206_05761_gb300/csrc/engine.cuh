@@ -159,13 +159,12 @@ class EngineT final : public Engine {
         if (!alloc(&counts_, ((size_t)ntiles_ * 3 + 1) * sizeof(uint32_t))) return oom();
         offs_ = counts_ + ntiles_;
         dlist_ = counts_ + 2 * ntiles_ + 1;
-        // shared faces of the wet-leaf update: 10 values per queued leaf and
-        // its two velocities, a stamp per hierarchy cell.  Float64 only: in
+        // shared faces of the wet-leaf update and a stamp per hierarchy cell.  Float64 only: in
         // float32 the arithmetic saved costs less than the extra launch and
         // face traffic.
         if (sizeof(T) == 8) {
             fcap_ = (uint32_t)std::min<uint64_t>(N_, 1ull << 22);
-            if (!alloc(&face_, (size_t)fcap_ * 12 * sizeof(T))) return oom();
+            if (!alloc(&face_, (size_t)fcap_ * kFaceArrays * sizeof(T))) return oom();
             if (!alloc(&mark_, H_ * sizeof(unsigned long long))) return oom();
             cudaMemsetAsync(mark_, 0, H_ * sizeof(unsigned long long), stream_);
         }
@@ -800,6 +799,7 @@ class EngineT final : public Engine {
     // Everything a batched step needs for this domain (see batch.cuh):
     // encode passes of at most enc_k levels, FV1 work of about fv1_cells
     // finest cells per thread (the block count is set by the batch).
+    bool outgrows_faces() const { return N_ > fcap_; }   // (float32: no face buffer)
     template <class Plan>
     void fill_plan(Plan& p, int enc_k, int /*fv1_cells*/) const {
         for (int b = 0; b < 2; ++b)
@@ -863,6 +863,10 @@ class EngineT final : public Engine {
     int wet_grid() const {
         const uint64_t g = (N_ + 63) / 64, cap = (uint64_t)nsm_ * 16;
         return (int)(g < cap ? (g < 1 ? 1 : g) : cap);
+    }
+    int faces_grid() const {
+        const uint64_t g = (N_ + 63) / 64, cap = (uint64_t)nsm_ * 16;
+        return (int)(g < cap ? g : cap);
     }
     // Blocks of `threads` that one launch of kern keeps resident on the GPU.
     // A grid-stride loop over more blocks than that runs its last ones as a
@@ -1110,26 +1114,25 @@ class EngineT final : public Engine {
         mark("k_fv1_dry");
         launch_wet(a);
     }
-    // the full update of the queued leaves (after k_fv1_dry)
+    // the full update of the queued leaves (after k_fv1_dry): the face pair,
+    // then, where the queue can outgrow the face buffer, one pass over the rest
     void launch_wet(const StepArgs<T>& a) {
-        if (a.fm && face_) {
-            // matched fluxes with shared faces: a face toward a refined
-            // neighbour takes the walk over its halves in either phase
-            lk(k_fv1_faces<T, true>, grid_res(k_fv1_faces<T, true>, wet_grid(), 64), 64, a);
-            mark("k_fv1_faces");
-            lk(k_fv1_update<T, true>, grid_res(k_fv1_update<T, true>, wet_grid(), 64), 64, a);
-            mark("k_fv1_update");
-        } else if (a.fm) {
-            lk(k_fv1_match<T>, grid_res(k_fv1_match<T>, wet_grid(), 64), 64, a);
-            mark("k_fv1_match");
-        } else if (face_) {
-            // 64-thread blocks: a short queue spreads over every SM's FP64 units
+        if (face_) {
+            // blocks of 128 threads form the faces of 64 leaves.  The update
+            // runs in 64-thread blocks: a short queue spreads over every SM
             // (one warp-wide FP64 instruction holds a sub-partition's unit for
             // tens of cycles, so few warps per unit means a shorter chain)
-            lk(k_fv1_faces<T>, grid_res(k_fv1_faces<T>, wet_grid(), 64), 64, a);
+            const int gf = faces_grid();
+            if (a.fm) lk(k_fv1_faces<T, true>, grid_res(k_fv1_faces<T, true>, gf, 128), 128, a);
+            else lk(k_fv1_faces<T>, grid_res(k_fv1_faces<T>, gf, 128), 128, a);
             mark("k_fv1_faces");
             lk(k_fv1_update<T>, grid_res(k_fv1_update<T>, wet_grid(), 64), 64, a);
             mark("k_fv1_update");
+            if (N_ <= fcap_) return;
+        }
+        if (a.fm) {
+            lk(k_fv1_match<T>, grid_res(k_fv1_match<T>, wet_grid(), 64), 64, a);
+            mark("k_fv1_match");
         } else {
             lk(k_fv1_wet<T>, grid_res(k_fv1_wet<T>, wet_grid(), 64), 64, a);
             mark("k_fv1_wet");
@@ -1557,7 +1560,7 @@ class EngineT final : public Engine {
     uint32_t *counts_ = nullptr, *offs_ = nullptr, *dlist_ = nullptr;
     uint8_t* tilebytes_ = nullptr;      // per tile: zf of buffer 0, zf of buffer 1, inlet, act
     bool batched_ = false;
-    T* face_ = nullptr;                 // shared faces and velocities (12 x fcap_)
+    T* face_ = nullptr;                 // shared faces and velocities (kFaceArrays x fcap_)
     std::unordered_map<const void*, int> occ_;   // resident blocks per kernel
     uint32_t fcap_ = 0;
     unsigned long long* mark_ = nullptr;   // per hierarchy cell: (epoch + 1) << 32 | queue slot

@@ -96,18 +96,23 @@ __device__ __forceinline__ float absval(float x) { return __int_as_float(__float
 // operation returns (NaN inputs aside, which the state checks report).
 // ---------------------------------------------------------------------------
 // x * 2^k for k in {-2, -1, 1}: an exponent step when input and result are
-// normal numbers; otherwise the IEEE product (inline PTX, so that it is not
-// executed when the integer path applies).
+// normal numbers, x itself for a zero; otherwise the IEEE product, in a
+// function of its own (an FP64 instruction the compiler predicates would
+// hold the pipe even where no lane needs it).
+template <int K>
+static __device__ __noinline__ double pow2_rare(double x) {
+    return x * (K == -2 ? 0.25 : (K == -1 ? 0.5 : 2.0));
+}
 template <int K>
 __device__ __forceinline__ double pow2_scale(double x) {
-    const long long b = dbits(x);
-    const int e = (int)((b >> 52) & 0x7FF);
-    if (e + K >= 1 && e + K <= 0x7FE && e >= 1 && e <= 0x7FE) return dval(b + ((long long)K << 52));
-    double r;
-    if (K == -2) asm volatile("mul.rn.f64 %0, %1, 0d3FD0000000000000;" : "=d"(r) : "d"(x));
-    else if (K == -1) asm volatile("mul.rn.f64 %0, %1, 0d3FE0000000000000;" : "=d"(r) : "d"(x));
-    else asm volatile("mul.rn.f64 %0, %1, 0d4000000000000000;" : "=d"(r) : "d"(x));
-    return r;
+    uint32_t lo, hi;
+    d_split(x, lo, hi);
+    const uint32_t m = hi & 0x7FFFFFFFu;
+    // exponents e and e + K in [1, 2046]
+    constexpr uint32_t e0 = (uint32_t)(K < 0 ? 1 - K : 1), e1 = (uint32_t)(K > 0 ? 2046 - K : 2046);
+    if (m - (e0 << 20) < ((e1 - e0 + 1u) << 20)) return d_join((uint64_t)(hi + ((uint32_t)K << 20)) << 32 | lo);
+    if ((m | lo) == 0u) return x;
+    return pow2_rare<K>(x);
 }
 template <int K>
 __device__ __forceinline__ float pow2_scale(float x) {
@@ -122,11 +127,12 @@ __device__ __forceinline__ float pow2_scale(float x) {
 }
 // x * 2^n for 0 <= n <= 30: an exponent step when x and the result are
 // normal numbers, otherwise the IEEE product (the same bits either way).
+static __device__ __noinline__ double mul_pow2_rare(double x, int n) { return x * (double)(1u << n); }
 __device__ __forceinline__ double mul_pow2(double x, int n) {
     const long long b = dbits(x);
     const int e = (int)((b >> 52) & 0x7FF);
     if (e >= 1 && e + n <= 0x7FE) return dval(b + ((long long)n << 52));
-    return x * (double)(1u << n);
+    return mul_pow2_rare(x, n);
 }
 __device__ __forceinline__ float mul_pow2(float x, int n) {
     const int b = __float_as_int(x);
@@ -1360,38 +1366,23 @@ template <typename T>
 __device__ __forceinline__ void velocity(const Cell<T>& c, T tol, T& u, T& v) {
     if (ge_nonneg(c.h, tol)) {                         // h >= tol (tol > 0)
         const T rh = recip(c.h);
-        u = c.qx * rh;
-        v = c.qy * rh;
+        u = prod(c.qx, rh);
+        v = prod(c.qy, rh);
     } else {
         u = T(0);
         v = T(0);
     }
 }
 
-// HLL flux across a face with normal from L to R; F = (mass, normal
-// momentum, tangential momentum), hLs/hRs the reconstructed depths.
+// HLL flux across a face with normal from L to R, from the reconstructed
+// depths (not both 0): F = (mass, normal momentum, tangential momentum).
 //
 // Every comparison, selection and power-of-two scaling below is done on the
 // bit patterns (is_zero, ge_nonneg, sel_min/sel_max, ge_zero/le_zero,
 // half/quarter/twice): the same results as the IEEE operations the oracle
 // performs, without occupying the FP64 pipe.
 template <typename T>
-__device__ __forceinline__ void hll_face(T g, T hg, T tol, T hL, T zL, T unL, T utL, T hR, T zR, T unR,
-                                         T utR, T F[3], T& hLs_o, T& hRs_o) {
-    const T zf = sel_max(zR, zL);                       // zL > zR ? zL : zR
-    // on a +0 bed both sides are exact: (h + 0) - 0 = h for h != -0, and a
-    // -0 depth gives +0 where the shortcut gives -0, both below tol
-    const bool bed0 = pos_zero(zL) && pos_zero(zR);
-    const T dL = bed0 ? hL : (hL + zL) - zf;
-    const T dR = bed0 ? hR : (hR + zR) - zf;
-    const T hLs = ge_nonneg(dL, tol) ? dL : T(0);        // tol > 0
-    const T hRs = ge_nonneg(dR, tol) ? dR : T(0);
-    hLs_o = hLs;
-    hRs_o = hRs;
-    if (is_zero(hLs) && is_zero(hRs)) {
-        F[0] = F[1] = F[2] = T(0);
-        return;
-    }
+__device__ __forceinline__ void hll_flux(T g, T hg, T hLs, T unL, T utL, T hRs, T unR, T utR, T F[3]) {
     const T aL = root(g * hLs), aR = root(g * hRs);
     T SL, SR;
     if (!is_zero(hLs) && !is_zero(hRs)) {
@@ -1424,6 +1415,115 @@ __device__ __forceinline__ void hll_face(T g, T hg, T tol, T hL, T zL, T unL, T 
     }
 }
 
+// The same operations in float64 with the products formed in integer
+// instructions beside the FP64 pipe, which is left with the sums (22 of the
+// face's 49 operations besides its roots and reciprocal).  That needs the
+// operands' exponents in a window, checked once per cell: depths and g below
+// 2^100, the wet tolerance and g above 2^-100, velocities 0 or within
+// 2^-300..2^100, beds below 2^99.  Every product below is then zero, or normal
+// by a wide margin: the smallest magnitudes are 2^-102 for SL and SR (a sum
+// that cancels), 2^-400 for q, 2^-700 for q u, 2^-656 for SL SR d and 2^-955
+// for the last product, the largest 2^700.  Out of the window, hll_flux.
+__device__ __forceinline__ bool speed_window(double u) {
+    uint32_t lo, hi;
+    d_split(u, lo, hi);
+    hi &= 0x7FFFFFFFu;
+    return hi - (723u << 20) < (400u << 20) || (hi | lo) == 0u;
+}
+__device__ __forceinline__ bool below_window(double x) { return ((uint32_t)(dbits(x) >> 32) & 0x7FFFFFFFu) < (1122u << 20); }
+__device__ __forceinline__ bool cell_window(double h, double z, double u, double v) {
+    return below_window(h) && below_window(z) && speed_window(u) && speed_window(v);
+}
+__device__ __forceinline__ bool const_window(double g, double tol) {
+    const uint32_t gh = (uint32_t)(dbits(g) >> 32), th = (uint32_t)(dbits(tol) >> 32);
+    return gh - (923u << 20) < (200u << 20) && th - (923u << 20) < (200u << 20);
+}
+__device__ __forceinline__ bool cell_window(float, float, float, float) { return true; }
+__device__ __forceinline__ bool const_window(float, float) { return true; }
+// x 2^K for an x that is zero or whose result is normal
+template <int K>
+__device__ __forceinline__ double scale_z(double x) {
+    uint32_t lo, hi;
+    d_split(x, lo, hi);
+    const uint32_t e = hi & 0x7FF00000u, k = (uint32_t)(K < 0 ? -K : K) << 20;
+    const uint32_t d = e < k ? e : k;
+    return d_join((uint64_t)(K < 0 ? hi - d : hi + d) << 32 | lo);
+}
+// a < b, -0 before +0 (no NaN)
+__device__ __forceinline__ bool less_ord(double a, double b) {
+    const long long x = dbits(a), y = dbits(b);
+    const long long kx = x ^ ((x >> 63) & 0x7FFFFFFFFFFFFFFFll), ky = y ^ ((y >> 63) & 0x7FFFFFFFFFFFFFFFll);
+    return kx < ky;
+}
+static __device__ __noinline__ void hll_flux_rare(double g, double hg, double hLs, double unL, double utL, double hRs,
+                                                  double unR, double utR, double* F) {
+    hll_flux<double>(g, hg, hLs, unL, utL, hRs, unR, utR, F);
+}
+__device__ __forceinline__ void hll_flux_mixed(double g, double hg, double hL, double unL, double utL, double hR,
+                                               double unR, double utR, bool safe, double F[3]) {
+    if (!safe) {
+        double f[3];
+        hll_flux_rare(g, hg, hL, unL, utL, hR, unR, utR, f);
+        F[0] = f[0];
+        F[1] = f[1];
+        F[2] = f[2];
+        return;
+    }
+    const double gL = prod_z(g, hL), gR = prod_z(g, hR);
+    const double aL = root(gL), aR = root(gR);
+    const double us = scale_z<-1>(unL + unR) + aL - aR;
+    const double as = scale_z<-1>(aL + aR) + scale_z<-2>(unL - unR);
+    // a dry side replaces one estimate: SL = unR - 2 aR, SR = unL + 2 aL
+    const bool dryL = is_zero(hL), dryR = is_zero(hR);
+    const double a1 = unL - aL, a2 = (dryL ? unR : us) - (dryL ? scale_z<1>(aR) : as);
+    const double b1 = unR + aR, b2 = (dryR ? unL : us) + (dryR ? scale_z<1>(aL) : as);
+    const double SL = dryL || (!dryR && less_ord(a2, a1)) ? a2 : a1;
+    const double SR = dryR || (!dryL && less_ord(b1, b2)) ? b2 : b1;
+    const double qnL = prod_z(hL, unL), qtL = prod_z(hL, utL);
+    const double qnR = prod_z(hR, unR), qtR = prod_z(hR, utR);
+    // hg h = half(g h) exactly
+    const double FL1 = prod_z(qnL, unL) + prod_z(scale_z<-1>(gL), hL), FL2 = prod_z(qnL, utL);
+    const double FR1 = prod_z(qnR, unR) + prod_z(scale_z<-1>(gR), hR), FR2 = prod_z(qnR, utR);
+    // a sum that cancels is +0, so neither S is ever -0
+    if (dbits(SL) >= 0) {
+        F[0] = qnL; F[1] = FL1; F[2] = FL2;
+    } else if (dbits(SR) <= 0) {
+        F[0] = qnR; F[1] = FR1; F[2] = FR2;
+    } else {
+        const double inv = recip(SR - SL);
+        const double P = prod_nz(SL, SR);
+        F[0] = prod_z(prod_z(SR, qnL) - prod_z(SL, qnR) + prod_z(P, hR - hL), inv);
+        F[1] = prod_z(prod_z(SR, FL1) - prod_z(SL, FR1) + prod_z(P, qnR - qnL), inv);
+        F[2] = prod_z(prod_z(SR, FL2) - prod_z(SL, FR2) + prod_z(P, qtR - qtL), inv);
+    }
+}
+__device__ __forceinline__ void hll_flux_mixed(float g, float hg, float hL, float unL, float utL, float hR, float unR,
+                                               float utR, bool, float F[3]) {
+    hll_flux<float>(g, hg, hL, unL, utL, hR, unR, utR, F);
+}
+
+// HLL flux across a face with normal from L to R, from the two sides' free
+// surfaces eta = h + z and beds; hLs/hRs the reconstructed depths.  safe: both
+// sides and the constants are in the window of hll_flux_mixed.
+template <typename T>
+__device__ __forceinline__ void hll_face(T g, T hg, T tol, T eL, T zL, T unL, T utL, T eR, T zR, T unR, T utR,
+                                         bool safe, T F[3], T& hLs_o, T& hRs_o) {
+    const T zf = sel_max(zR, zL);                       // zL > zR ? zL : zR
+    // on a +0 bed x - 0 = x
+    const bool bed0 = pos_zero(zL) && pos_zero(zR);
+    const T dL = bed0 ? eL : eL - zf;
+    const T dR = bed0 ? eR : eR - zf;
+    const T hLs = ge_nonneg(dL, tol) ? dL : T(0);        // tol > 0
+    const T hRs = ge_nonneg(dR, tol) ? dR : T(0);
+    hLs_o = hLs;
+    hRs_o = hRs;
+    if (is_zero(hLs) && is_zero(hRs)) {
+        F[0] = F[1] = F[2] = T(0);
+        return;
+    }
+    hll_flux_mixed(g, hg, hLs, unL, utL, hRs, unR, utR, safe, F);
+}
+
 template <typename T>
 __device__ __forceinline__ void cell_update_faces(const Phys<T>& P, T rx, T ry, T fk, const Cell<T>& C,
                                                   const T FW[3], const T FE[3], const T GS[3], const T GN[3],
@@ -1451,10 +1551,16 @@ __device__ __forceinline__ void cell_update(const Phys<T>& P, T rx, T ry, T fk, 
         velocity(E, tol, uE, vE);
         velocity(S, tol, uS, vS);
         velocity(N, tol, uN, vN);
-        hll_face(g, hg, tol, W.h, W.z, uW, vW, C.h, C.z, uC, vC, FW, dummy, hW_R);
-        hll_face(g, hg, tol, C.h, C.z, uC, vC, E.h, E.z, uE, vE, FE, hE_L, dummy);
-        hll_face(g, hg, tol, S.h, S.z, vS, uS, C.h, C.z, vC, uC, GS, dummy, hS_R);
-        hll_face(g, hg, tol, C.h, C.z, vC, uC, N.h, N.z, vN, uN, GN, hN_L, dummy);
+        const T eC = eta_of(C.h, C.z);
+        const bool ok = const_window(g, tol) && cell_window(C.h, C.z, uC, vC);
+        hll_face(g, hg, tol, eta_of(W.h, W.z), W.z, uW, vW, eC, C.z, uC, vC, ok && cell_window(W.h, W.z, uW, vW), FW,
+                 dummy, hW_R);
+        hll_face(g, hg, tol, eC, C.z, uC, vC, eta_of(E.h, E.z), E.z, uE, vE, ok && cell_window(E.h, E.z, uE, vE), FE,
+                 hE_L, dummy);
+        hll_face(g, hg, tol, eta_of(S.h, S.z), S.z, vS, uS, eC, C.z, vC, uC, ok && cell_window(S.h, S.z, uS, vS), GS,
+                 dummy, hS_R);
+        hll_face(g, hg, tol, eC, C.z, vC, uC, eta_of(N.h, N.z), N.z, vN, uN, ok && cell_window(N.h, N.z, uN, vN), GN,
+                 hN_L, dummy);
     }
     cell_update_faces(P, rx, ry, fk, C, FW, FE, GS, GN, hW_R, hE_L, hS_R, hN_L, inlet, dh, out);
 }
@@ -1477,9 +1583,9 @@ __device__ __forceinline__ double rcbrt_newton(float hf, double h) {
     const uint32_t b = (uint32_t)__float_as_int(rf);
     const long long e = (long long)((b >> 23) & 0xFFu) - 127 + 1023;
     const double r = dval((e << 52) | ((long long)(b & 0x7FFFFFu) << 29));
-    const double r3 = (r * r) * r;
+    const double r3 = prod(prod(r, r), r);
     const double d = __fma_rn(-h, r3, 1.0);
-    return __fma_rn(r * d, 1.0 / 3.0, r);
+    return __fma_rn(prod(r, d), 1.0 / 3.0, r);
 }
 
 // x / (h cbrt(h)) = x h^(-4/3) of Manning's friction term for a wet cell
@@ -1490,7 +1596,7 @@ __device__ __forceinline__ double rcbrt_newton(float hf, double h) {
 __device__ __forceinline__ double friction_term(double x, double h, double rh) {
     const float hf = trunc_float(h);
     const uint32_t eb = ((uint32_t)__float_as_int(hf) >> 23) & 0xFFu;
-    if (eb != 0u && eb != 0xFFu) return (x * rh) * rcbrt_newton(hf, h);
+    if (eb != 0u && eb != 0xFFu) return prod(prod(x, rh), rcbrt_newton(hf, h));
     return x / (h * cbrt(h));
 }
 __device__ __forceinline__ float friction_term(float x, float h, float /*rh*/) { return x / (h * cbrtf(h)); }
@@ -1506,25 +1612,25 @@ __device__ __forceinline__ void cell_update_faces_sq(const Phys<T>& P, T rx, T r
                                                      T* rh_out = nullptr) {
     if (rh_out) *rh_out = T(0);
     const T hg = P.hg, tol = P.tol;
-    const T bx = hg * (hW2 - hE2);
-    const T by = hg * (hS2 - hN2);
-    T h = C.h - rx * (FE[0] - FW[0]) - ry * (GN[0] - GS[0]);
-    T qx = C.qx - rx * ((FE[1] - FW[1]) + bx) - ry * (GN[2] - GS[2]);
-    T qy = C.qy - rx * (FE[2] - FW[2]) - ry * ((GN[1] - GS[1]) + by);
+    const T bx = prod(hg, hW2 - hE2);
+    const T by = prod(hg, hS2 - hN2);
+    T h = C.h - prod(rx, FE[0] - FW[0]) - prod(ry, GN[0] - GS[0]);
+    T qx = C.qx - prod(rx, (FE[1] - FW[1]) + bx) - prod(ry, GN[2] - GS[2]);
+    T qy = C.qy - prod(rx, FE[2] - FW[2]) - prod(ry, (GN[1] - GS[1]) + by);
     if (inlet) h = h + dh;
     h = gt_zero(h) ? h : T(0);
     if (!ge_nonneg(h, tol)) {                           // h < tol (tol > 0)
         qx = T(0);
         qy = T(0);
-    } else if (P.nM > T(0)) {
+    } else if (gt_zero(P.nM)) {
         const T rh = recip(h);
         if (rh_out) *rh_out = rh;
-        const T u = qx * rh, v = qy * rh;
-        const T speed = root(u * u + v * v);
-        const T D = T(1) + friction_term(fk * speed, h, rh);
+        const T u = prod(qx, rh), v = prod(qy, rh);
+        const T speed = root(prod(u, u) + prod(v, v));
+        const T D = T(1) + friction_term(prod(fk, speed), h, rh);
         const T rD = recip(D);
-        qx = qx * rD;
-        qy = qy * rD;
+        qx = prod(qx, rD);
+        qy = prod(qy, rD);
     }
     out[0] = h;
     out[1] = qx;
@@ -1538,7 +1644,8 @@ __device__ __forceinline__ void cell_update_faces(const Phys<T>& P, T rx, T ry, 
                                                   const T FW[3], const T FE[3], const T GS[3], const T GN[3],
                                                   T hW_R, T hE_L, T hS_R, T hN_L, bool inlet, T dh, T out[3],
                                                   T* rh_out) {
-    cell_update_faces_sq(P, rx, ry, fk, C, FW, FE, GS, GN, hW_R * hW_R, hE_L * hE_L, hS_R * hS_R, hN_L * hN_L,
+    cell_update_faces_sq(P, rx, ry, fk, C, FW, FE, GS, GN, prod(hW_R, hW_R), prod(hE_L, hE_L),
+                         prod(hS_R, hS_R), prod(hN_L, hN_L),
                          inlet, dh, out, rh_out);
 }
 
@@ -1547,10 +1654,40 @@ template <typename T>
 __device__ __forceinline__ T cfl_bound(const Phys<T>& P, T h, T qx, T qy) {
     if (!ge_nonneg(h, P.tol)) return T(INFINITY);      // h < tol (tol > 0)
     const T rh = recip(h);
-    const T u = absval(qx * rh), v = absval(qy * rh);
-    const T a = root(P.g * h);
+    const T u = absval(prod(qx, rh)), v = absval(prod(qy, rh));
+    const T a = root(prod(P.g, h));
     const T rx = P.dxL / (u + a), ry = P.dyL / (v + a);
     return sel_min(rx, ry);
+}
+
+// The face buffer: per queued leaf, in units of fcap values (pairs are stored
+// as pairs, so a leaf's pair is one 128-bit access in float64).
+enum : int {
+    kLeafUV = 0,         // u, v
+    kLeafEZ = 2,         // free surface h + z, bed z  (these two written by k_fv1_dry)
+    kFaceE = 4,          // east face: F0, F1 | F2, left depth squared | right depth squared
+    kFaceN = 9,          // north face, as the east one
+    kFaceW = 14,         // west face where it is not shared: F0, F1 | F2, its own depth squared
+    kFaceS = 18,         // south face, as the west one
+    kFaceArrays = 22
+};
+// A leaf's stamp: (epoch + 1) << 32 | queue slot, with kUnsafe set where the
+// leaf is out of the window of hll_flux_mixed.
+constexpr uint32_t kUnsafe = 0x80000000u;
+
+template <typename T> struct Pair2;
+template <> struct Pair2<double> { typedef double2 V; };
+template <> struct Pair2<float> { typedef float2 V; };
+template <typename T>
+__device__ __forceinline__ typename Pair2<T>::V* pair_at(T* face, size_t cap, int k, uint32_t w) {
+    return reinterpret_cast<typename Pair2<T>::V*>(face + k * cap) + w;
+}
+template <typename T>
+__device__ __forceinline__ typename Pair2<T>::V make_pair2(T a, T b) {
+    typename Pair2<T>::V v;
+    v.x = a;
+    v.y = b;
+    return v;
 }
 
 template <typename T>
@@ -1566,10 +1703,8 @@ struct StepArgs {
     int bc_ref[4];           // 1: the side reflects (closed or inflow)
     int inflow_side;         // -1: none
     int a0, a1;
-    // shared faces (k_fv1_faces / k_fv1_update): 12 arrays of fcap values
-    // (east face F0..F2, h*_L, h*_R, then the north face's, then the
-    // leaf's velocities u, v, written by k_fv1_dry), and a stamp per
-    // hierarchy cell ((epoch + 1) << 32 | queue slot)
+    // shared faces (k_fv1_faces / k_fv1_update): kFaceArrays arrays of fcap
+    // values, and a stamp per hierarchy cell
     T* face = nullptr;
     uint32_t fcap = 0;
     unsigned long long* mark = nullptr;
@@ -1715,20 +1850,20 @@ __device__ __forceinline__ void dry_finish(const StepArgs<T>& a, DevState* st, T
         base_pos = __shfl_sync(m, base_pos, leader);
         const uint32_t w = base_pos + __popc(m & ((1u << lane) - 1u));
         a.wet[w] = pk;                                            // the packed leaf
-        // float64 with shared faces: the leaf's velocities (the operations
-        // of velocity() in k_fv1_faces, which reads them here instead of
-        // forming them for the leaf and for the two neighbours whose west
-        // and south faces it is) and its stamp, once per queued leaf
-        if (sizeof(T) == 8 && a.face != nullptr && !a.fm && w < a.fcap) {
+        // float64 with shared faces: what the faces read of the leaf (its
+        // velocities, with the operations of velocity(), its free surface and
+        // bed) and its stamp, once per queued leaf
+        if (sizeof(T) == 8 && a.face != nullptr && w < a.fcap) {
             Cell<T> C;
             C.h = __ldg(src.h + d.iC);
             C.qx = __ldg(src.qx + d.iC);
             C.qy = __ldg(src.qy + d.iC);
+            C.z = __ldg(src.z + d.iC);
             T u, v;
             velocity(C, a.P.tol, u, v);
-            a.face[10 * (size_t)a.fcap + w] = u;
-            a.face[11 * (size_t)a.fcap + w] = v;
-            a.mark[d.iC] = stamp | w;
+            *pair_at(a.face, a.fcap, kLeafUV, w) = make_pair2(u, v);
+            *pair_at(a.face, a.fcap, kLeafEZ, w) = make_pair2(eta_of(C.h, C.z), C.z);
+            a.mark[d.iC] = stamp | w | (cell_window(C.h, C.z, u, v) ? 0u : kUnsafe);
         }
     }
 }
@@ -1788,8 +1923,8 @@ __device__ __forceinline__ void wet_leaf_store(const StepArgs<T>& a, DevState* s
         // cfl_bound up to the division, reusing the friction step's 1/h
         if (ge_nonneg(out[0], a.P.tol)) {
             const T rh = is_zero(rh_known) ? recip(out[0]) : rh_known;
-            const T u = absval(out[1] * rh), v = absval(out[2] * rh);
-            const T aa = root(a.P.g * out[0]);
+            const T u = absval(prod(out[1], rh)), v = absval(prod(out[2], rh));
+            const T aa = root(prod(a.P.g, out[0]));
             const unsigned long long bx = abs_obits(u + aa), by = abs_obits(v + aa);
             spd[0] = bx > spd[0] ? bx : spd[0];
             spd[1] = by > spd[1] ? by : spd[1];
@@ -1817,7 +1952,7 @@ __device__ __forceinline__ void wet_leaf_store(const StepArgs<T>& a, DevState* s
         const uint32_t cnt = 1u << (2 * (a.L - n));
         const T hl = out[0];
         const bool restore = ge_nonneg(hl, a.P.tol);
-        const T eta = restore ? eta_of(hl, C.z) : T(0);
+        const T eta = restore ? eta_of(hl, __ldg(z + iC)) : T(0);
         for (uint32_t e = 0; e < cnt; e += 4) {
             T hf[4];
             if (restore) {
@@ -1845,14 +1980,15 @@ __device__ __forceinline__ void wet_leaf_store(const StepArgs<T>& a, DevState* s
         atomicOr(&st->err, kErrNonFinite);
 }
 
-// FV1, second kernel: the full update (Eq. 2 with the L_c reading) of every
-// queued leaf, with the CFL and s_max reductions.
+// FV1 in one pass: the full update (Eq. 2 with the L_c reading) of the queued
+// leaves from fcap on, with the CFL and s_max reductions (float32: every
+// queued leaf; float64: those that outgrow the face buffer).
 template <typename T>
 __device__ __forceinline__ void fv1_wet_body(const StepArgs<T>& a, Blk B) {
     DevState* st = a.st;
     if (!st->active) return;
     const uint32_t nq = st->nwet;
-    if (B.id * blockDim.x >= nq) return;          // whole block idle
+    if (a.fcap + B.id * blockDim.x >= nq) return; // whole block idle
     const int par = (int)st->cur, nxt = par ^ 1;
     const T fk = fric_k_of<T>(st);
     const T rx0 = rx0_of<T>(st), ry0 = ry0_of<T>(st);
@@ -1866,7 +2002,7 @@ __device__ __forceinline__ void fv1_wet_body(const StepArgs<T>& a, Blk B) {
     T* const oqx = nxt ? a.f[1][1] : a.f[0][1];
     T* const oqy = nxt ? a.f[1][2] : a.f[0][2];
     unsigned long long rmin = kInfBits, mh = 0, mqx = 0, mqy = 0, spd[2] = {0ull, 0ull};
-    for (uint32_t w = B.id * blockDim.x + threadIdx.x; w < nq; w += B.n * blockDim.x) {
+    for (uint32_t w = a.fcap + B.id * blockDim.x + threadIdx.x; w < nq; w += B.n * blockDim.x) {
         const uint32_t pk = a.wet[w];            // the queue holds packed leaves
         const int n = (int)(pk >> kLeafShift);
         const uint32_t code = pk & kCodeMask;
@@ -1925,19 +2061,13 @@ __device__ __forceinline__ void face_of(const Phys<T>& P, int s, const Cell<T>& 
     T uC, vC, uX, vX, hl, hr;
     velocity(C, P.tol, uC, vC);
     velocity(X, P.tol, uX, vX);
-    if (s == 0) {
-        hll_face(P.g, P.hg, P.tol, X.h, X.z, uX, vX, C.h, C.z, uC, vC, F, hl, hr);
-        own2 = hr * hr;
-    } else if (s == 1) {
-        hll_face(P.g, P.hg, P.tol, C.h, C.z, uC, vC, X.h, X.z, uX, vX, F, hl, hr);
-        own2 = hl * hl;
-    } else if (s == 2) {
-        hll_face(P.g, P.hg, P.tol, X.h, X.z, vX, uX, C.h, C.z, vC, uC, F, hl, hr);
-        own2 = hr * hr;
-    } else {
-        hll_face(P.g, P.hg, P.tol, C.h, C.z, vC, uC, X.h, X.z, vX, uX, F, hl, hr);
-        own2 = hl * hl;
-    }
+    const bool right = s == 0 || s == 2, yf = s >= 2;       // right: the cell is the right side
+    const T eC = eta_of(C.h, C.z), eX = eta_of(X.h, X.z);
+    const T nC = yf ? vC : uC, tC = yf ? uC : vC, nX = yf ? vX : uX, tX = yf ? uX : vX;
+    const bool safe = const_window(P.g, P.tol) && cell_window(C.h, C.z, uC, vC) && cell_window(X.h, X.z, uX, vX);
+    hll_face(P.g, P.hg, P.tol, right ? eX : eC, right ? X.z : C.z, right ? nX : nC, right ? tX : tC,
+             right ? eC : eX, right ? C.z : X.z, right ? nC : nX, right ? tC : tX, safe, F, hl, hr);
+    own2 = right ? prod(hr, hr) : prod(hl, hl);
 }
 
 // The face on side s of the leaf (n, i, j) whose same-level neighbour is
@@ -2021,7 +2151,7 @@ __device__ __forceinline__ void fv1_match_body(const StepArgs<T>& a, Blk B) {
     DevState* st = a.st;
     if (!st->active) return;
     const uint32_t nq = st->nwet;
-    if (B.id * blockDim.x >= nq) return;          // whole block idle
+    if (a.fcap + B.id * blockDim.x >= nq) return; // whole block idle
     const int par = (int)st->cur, nxt = par ^ 1;
     const T fk = fric_k_of<T>(st);
     const T rx0 = rx0_of<T>(st), ry0 = ry0_of<T>(st);
@@ -2035,7 +2165,7 @@ __device__ __forceinline__ void fv1_match_body(const StepArgs<T>& a, Blk B) {
     T* const oqx = nxt ? a.f[1][1] : a.f[0][1];
     T* const oqy = nxt ? a.f[1][2] : a.f[0][2];
     unsigned long long rmin = kInfBits, mh = 0, mqx = 0, mqy = 0, spd[2] = {0ull, 0ull};
-    for (uint32_t w = B.id * blockDim.x + threadIdx.x; w < nq; w += B.n * blockDim.x) {
+    for (uint32_t w = a.fcap + B.id * blockDim.x + threadIdx.x; w < nq; w += B.n * blockDim.x) {
         const uint32_t pk = a.wet[w];
         const int n = (int)(pk >> kLeafShift);
         const uint32_t code = pk & kCodeMask;
@@ -2074,119 +2204,160 @@ static __global__ void __launch_bounds__(256) k_fv1_match(StepArgs<T> a) {
 }
 
 // The same update in two kernels that compute every face between two queued
-// leaves of one level once.  Phase 1: each queued leaf computes its east and
-// north faces (it is their left side) and stamps its cell.  Phase 2: a
-// queued leaf whose west (south) same-level neighbour carries this step's
-// stamp takes that neighbour's east (north) face -- the same call with the
-// same operands, so the same bits -- and computes only its other faces.
-// The velocities k_fv1_dry formed for the queued leaf at hierarchy index
-// idx, if that cell holds one this step (its stamp is this step's).
-template <typename T>
-__device__ __forceinline__ bool queued_velocity(const StepArgs<T>& a, unsigned long long stamp, uint64_t idx,
-                                                T& u, T& v) {
-    const unsigned long long m = __ldg(a.mark + idx);
-    if ((m >> 32) != (stamp >> 32)) return false;
-    const uint32_t wn = (uint32_t)m;
-    u = a.face[10 * (size_t)a.fcap + wn];
-    v = a.face[11 * (size_t)a.fcap + wn];
-    return true;
+// leaves of one level once.  Phase 1 (k_fv1_faces): each queued leaf's east
+// and north faces (it is their left side), and its west or south face where
+// the same-level neighbour is not queued (its stamp is not this step's), so
+// that phase 2 (k_fv1_update) only reads faces: a west (south) face is the
+// queued west (south) neighbour's east (north) face -- the same call with the
+// same operands, so the same bits -- or the leaf's own.
+//
+// The cells next to a leaf along one axis (y: north and south, else east and
+// west): hierarchy indices (below 2^32 up to L = 14), and whether the domain
+// ends there.
+struct AxisProbe {
+    uint32_t iC, iM, iP, code;
+    int n;
+    bool endM, endP;
+};
+__device__ __forceinline__ AxisProbe axis_probe(uint32_t pk, bool y) {
+    AxisProbe d;
+    d.n = (int)(pk >> kLeafShift);
+    d.code = pk & kCodeMask;
+    const uint32_t base = (uint32_t)lvl_off(d.n), lm = (1u << (2 * d.n)) - 1u;
+    const uint32_t A = y ? kYBits : kXBits, one = y ? 2u : 1u;
+    const uint32_t own = d.code & A, rest = d.code & ~A;
+    d.iC = base + d.code;
+    d.iP = base + ((((d.code | ~A) + one) & A) | rest);
+    d.iM = base + (((own - one) & A) | rest);
+    d.endP = own == (A & lm);
+    d.endM = own == 0u;
+    return d;
 }
 
+// Face s (0 W, 1 E, 2 S, 3 N) of queued leaf w into the face buffer.
+template <typename T, bool FM>
+__device__ __forceinline__ void queued_face(const StepArgs<T>& a, const CellSrc<T>& src, uint32_t tag, bool ok,
+                                            uint32_t w, int s, const AxisProbe& d) {
+    const size_t cap = a.fcap;
+    const bool yface = s >= 2, right = (s & 1) == 0;      // right: the leaf is the right side
+    const bool edge = right ? d.endM : d.endP;
+    const uint32_t iX = edge ? d.iC : (right ? d.iM : d.iP);
+    T F[3], own2, other2 = T(0);
+    if (FM && !edge && d.n < a.L && sig_bit(a.Sb, d.n, iX - (uint32_t)lvl_off(d.n))) {
+        // toward a refined neighbour: the walk over the finer halves (the
+        // face's other side belongs to no leaf)
+        matched_face(a, src, s, d.n, compact16(d.code), compact16(d.code >> 1), F, own2);
+    } else {
+        const unsigned long long m = __ldg(a.mark + iX), mc = __ldg(a.mark + d.iC);
+        const typename Pair2<T>::V uv = *pair_at(a.face, cap, kLeafUV, w), ez = *pair_at(a.face, cap, kLeafEZ, w);
+        typename Pair2<T>::V xuv, xez;
+        bool safe = ok && !((uint32_t)mc & kUnsafe);
+        if ((uint32_t)(m >> 32) == tag) {                 // queued too (at an edge: the leaf itself)
+            const uint32_t wx = (uint32_t)m & ~kUnsafe;
+            xuv = *pair_at(a.face, cap, kLeafUV, wx);
+            xez = *pair_at(a.face, cap, kLeafEZ, wx);
+            safe = safe && !((uint32_t)m & kUnsafe);
+        } else {
+            Cell<T> X = fetch(src, iX);
+            T u, v;
+            velocity(X, a.P.tol, u, v);
+            safe = safe && cell_window(X.h, X.z, u, v);
+            xuv = make_pair2(u, v);
+            xez = make_pair2(eta_of(X.h, X.z), X.z);
+        }
+        T un = yface ? uv.y : uv.x, ut = yface ? uv.x : uv.y;
+        T xn = yface ? xuv.y : xuv.x, xt = yface ? xuv.x : xuv.y;
+        if (edge) {
+            // the ghost's velocity is the leaf's, the normal part reversed at
+            // a wall (a dry leaf's is +0 either way)
+            const int wall = s == 0 ? a.bc_ref[0] : (s == 1 ? a.bc_ref[1] : (s == 2 ? a.bc_ref[2] : a.bc_ref[3]));
+            if (wall && ge_nonneg(__ldg(src.h + d.iC), a.P.tol)) xn = -xn;
+        }
+        T hl, hr;
+        hll_face(a.P.g, a.P.hg, a.P.tol, right ? xez.x : ez.x, right ? xez.y : ez.y, right ? xn : un, right ? xt : ut,
+                 right ? ez.x : xez.x, right ? ez.y : xez.y, right ? un : xn, right ? ut : xt, safe, F, hl, hr);
+        const T own = right ? hr : hl, other = right ? hl : hr;
+        own2 = prod(own, own);
+        if (!right) other2 = prod(other, other);
+    }
+    const int k = s == 0 ? kFaceW : (s == 1 ? kFaceE : (s == 2 ? kFaceS : kFaceN));
+    *pair_at(a.face, cap, k, w) = make_pair2(F[0], F[1]);
+    *pair_at(a.face, cap, k + 2, w) = make_pair2(F[2], own2);
+    if (!right) a.face[(k + 4) * cap + w] = other2;
+}
+
+// A block takes as many leaves as half its threads: the first half forms their
+// east faces, the second half their north faces.  The west and south faces
+// that no neighbour shares are gathered in shared memory meanwhile and formed
+// in a second round by as few warps as they fill: resolution changes and
+// shorelines would otherwise have every warp that holds one such leaf run
+// two more faces.  One face per thread and one copy of the face's code (some
+// 1200 instructions) for all four sides also halves the latency of a short
+// queue and keeps the loop in the instruction cache.
+//
+// Bound by the FP64 pipe and the integer pipe together: 1 M leaves (uniform
+// FV1, L=10) take 148 us, in which the FP64 pipe's 24 sums a face fill 71 % of
+// the cycles and 790 integer instructions 61 %; 321 us with every operation on
+// the FP64 pipe and two faces per thread.
 template <typename T, bool FM = false>
 __device__ __forceinline__ void fv1_faces_body(const StepArgs<T>& a, Blk B) {
     DevState* st = a.st;
     if (!st->active) return;
-    const uint32_t nq = st->nwet;
-    if (nq > a.fcap || B.id * blockDim.x >= nq) return;
+    const uint32_t nw = st->nwet, nq = nw < a.fcap ? nw : a.fcap;
+    const uint32_t hb = blockDim.x >> 1, tid = threadIdx.x;
+    if (B.id * hb >= nq) return;                  // whole block idle
     const int par = (int)st->cur;
     CellSrc<T> src;
     src.h = par ? a.f[1][0] : a.f[0][0];
     src.qx = par ? a.f[1][1] : a.f[0][1];
     src.qy = par ? a.f[1][2] : a.f[0][2];
     src.z = a.z;
-    const T g = a.P.g, hg = a.P.hg, tol = a.P.tol;
-    const unsigned long long stamp = (unsigned long long)(st->epoch + 1u) << 32;
-    const uint32_t cap = a.fcap;
-    for (uint32_t w = B.id * blockDim.x + threadIdx.x; w < nq; w += B.n * blockDim.x) {
-        const uint32_t pk = a.wet[w];
-        const int n = (int)(pk >> kLeafShift);
-        const uint32_t code = pk & kCodeMask;
-        const uint32_t i = compact16(code), j = compact16(code >> 1);
-        const uint32_t last = (1u << n) - 1u;
-        const uint64_t base = lvl_off(n);
-        const uint64_t iC = base + code;
-        const Cell<T> C = fetch(src, iC);
-        T FE[3], GN[3], hEL2, hER2 = T(0), hNL2, hNR2 = T(0);
-        // with matched fluxes, a face toward a refined neighbour is the walk
-        // over its finer halves (its other side belongs to no leaf)
-        const bool mE = FM && i < last && n < a.L && sig_bit(a.Sb, n, morton2(i + 1, j));
-        const bool mN = FM && j < last && n < a.L && sig_bit(a.Sb, n, morton2(i, j + 1));
-        if (FM && (mE || mN)) {
-            if (mE) matched_face(a, src, 1, n, i, j, FE, hEL2);
-            if (mN) matched_face(a, src, 3, n, i, j, GN, hNL2);
+    const uint32_t tag = st->epoch + 1u;
+    const bool ok = const_window(a.P.g, a.P.tol);
+    __shared__ uint32_t nlist;
+    __shared__ uint16_t list[256];
+    const bool first = tid < hb;
+    const uint32_t l0 = first ? tid : tid - hb;
+    for (uint32_t base = B.id * hb; base < nq; base += B.n * hb) {
+        if (tid == 0) nlist = 0u;
+        __syncthreads();
+        uint32_t l = l0;
+        int s = first ? 1 : 3;
+        bool on = base + l < nq;
+        AxisProbe d = {};
+        if (on) {
+            // the face opposite to this thread's: shared by a queued neighbour?
+            d = axis_probe(a.wet[base + l], !first);
+            if (d.endM || (uint32_t)(__ldg(a.mark + d.iM) >> 32) != tag)
+                list[atomicAdd(&nlist, 1u)] = (uint16_t)(first ? l : l | 0x8000u);
         }
-        if (!(mE && mN)) {
-            const Cell<T> E = i < last ? fetch(src, base + morton2(i + 1, j)) : ghost(C, a.bc_ref[1], true);
-            const Cell<T> N = j < last ? fetch(src, base + morton2(i, j + 1)) : ghost(C, a.bc_ref[3], false);
-            T uC, vC, uE, vE, uN, vN;
-            // velocities formed by k_fv1_dry for every queued leaf (the
-            // leaf's own, and a same-level neighbour's when it is queued:
-            // its stamp is this step's), else formed here
-            if (!FM) {
-                uC = a.face[10 * (size_t)cap + w];
-                vC = a.face[11 * (size_t)cap + w];
-            } else {
-                velocity(C, tol, uC, vC);
-            }
-            if (!mE) {
-                if (!(!FM && i < last && queued_velocity(a, stamp, base + morton2(i + 1, j), uE, vE)))
-                    velocity(E, tol, uE, vE);
-                T hEL, hER;
-                hll_face(g, hg, tol, C.h, C.z, uC, vC, E.h, E.z, uE, vE, FE, hEL, hER);
-                hEL2 = hEL * hEL;
-                hER2 = hER * hER;
-            }
-            if (!mN) {
-                if (!(!FM && j < last && queued_velocity(a, stamp, base + morton2(i, j + 1), uN, vN)))
-                    velocity(N, tol, uN, vN);
-                T hNL, hNR;
-                hll_face(g, hg, tol, C.h, C.z, vC, uC, N.h, N.z, vN, uN, GN, hNL, hNR);
-                hNL2 = hNL * hNL;
-                hNR2 = hNR * hNR;
+#pragma unroll 1
+        for (int round = 0; round < 2; ++round) {
+            if (on) queued_face<T, FM>(a, src, tag, ok, base + l, s, d);
+            if (round == 1) break;
+            __syncthreads();
+            on = tid < nlist;
+            if (on) {
+                const uint32_t e = list[tid];
+                l = e & 0x7FFFu;
+                s = (e & 0x8000u) ? 2 : 0;
+                d = axis_probe(a.wet[base + l], s == 2);
             }
         }
-        // the face of both sides: flux, then the squares of the two
-        // reconstructed depths (the bed source terms of the two cells)
-        T* f = a.face + w;
-        f[0 * (size_t)cap] = FE[0];
-        f[1 * (size_t)cap] = FE[1];
-        f[2 * (size_t)cap] = FE[2];
-        f[3 * (size_t)cap] = hEL2;
-        f[4 * (size_t)cap] = hER2;
-        f[5 * (size_t)cap] = GN[0];
-        f[6 * (size_t)cap] = GN[1];
-        f[7 * (size_t)cap] = GN[2];
-        f[8 * (size_t)cap] = hNL2;
-        f[9 * (size_t)cap] = hNR2;
-        if (FM) a.mark[iC] = stamp | w;      // (k_fv1_dry stamped the leaf otherwise)
+        __syncthreads();                          // the list is read before the next chunk's
     }
 }
 template <typename T, bool FM = false>
-static __global__ void __launch_bounds__(256) k_fv1_faces(StepArgs<T> a) {
+static __global__ void __launch_bounds__(128) k_fv1_faces(StepArgs<T> a) {
     pdl_wait();
     fv1_faces_body<T, FM>(a, this_blk());
 }
 
-template <typename T, bool FM = false>
+template <typename T>
 __device__ __forceinline__ void fv1_update_body(const StepArgs<T>& a, Blk B) {
     DevState* st = a.st;
     if (!st->active) return;
-    const uint32_t nq = st->nwet;
-    if (nq > a.fcap) {                            // no room for the faces: one pass
-        if (FM) fv1_match_body<T>(a, B);
-        else fv1_wet_body<T>(a, B);
-        return;
-    }
+    const uint32_t nw = st->nwet, nq = nw < a.fcap ? nw : a.fcap;
     if (B.id * blockDim.x >= nq) return;          // whole block idle
     const int par = (int)st->cur, nxt = par ^ 1;
     const T fk = fric_k_of<T>(st);
@@ -2200,82 +2371,37 @@ __device__ __forceinline__ void fv1_update_body(const StepArgs<T>& a, Blk B) {
     T* const oh = nxt ? a.f[1][0] : a.f[0][0];
     T* const oqx = nxt ? a.f[1][1] : a.f[0][1];
     T* const oqy = nxt ? a.f[1][2] : a.f[0][2];
-    const T g = a.P.g, hg = a.P.hg, tol = a.P.tol;
     const uint32_t tag = st->epoch + 1u;
-    const uint32_t cap = a.fcap;
-    const T* F = a.face;
+    const size_t cap = a.fcap;
     unsigned long long rmin = kInfBits, mh = 0, mqx = 0, mqy = 0, spd[2] = {0ull, 0ull};
     for (uint32_t w = B.id * blockDim.x + threadIdx.x; w < nq; w += B.n * blockDim.x) {
-        const uint32_t pk = a.wet[w];
-        const int n = (int)(pk >> kLeafShift);
-        const uint32_t code = pk & kCodeMask;
-        const uint32_t i = compact16(code), j = compact16(code >> 1);
-        const uint32_t last = (1u << n) - 1u;
-        const uint64_t base = lvl_off(n);
-        const uint64_t iC = base + code;
-        const Cell<T> C = fetch(src, iC);
+        const DryProbe d = dry_probe(a.wet[w]);
+        const int n = d.n;
+        // the west and south faces: the queued neighbour's, or the leaf's own
+        const unsigned long long mW = __ldg(a.mark + d.iW), mS = __ldg(a.mark + d.iS);
+        const bool sW = d.iW != d.iC && (uint32_t)(mW >> 32) == tag, sS = d.iS != d.iC && (uint32_t)(mS >> 32) == tag;
+        const uint32_t wW = sW ? (uint32_t)mW & ~kUnsafe : w, wS = sS ? (uint32_t)mS & ~kUnsafe : w;
+        const typename Pair2<T>::V e0 = *pair_at(a.face, cap, kFaceE, w), e1 = *pair_at(a.face, cap, kFaceE + 2, w);
+        const typename Pair2<T>::V n0 = *pair_at(a.face, cap, kFaceN, w), n1 = *pair_at(a.face, cap, kFaceN + 2, w);
+        const int kW = sW ? kFaceE : kFaceW, kS = sS ? kFaceN : kFaceS;
+        const typename Pair2<T>::V w0 = *pair_at(a.face, cap, kW, wW), w1 = *pair_at(a.face, cap, kW + 2, wW);
+        const typename Pair2<T>::V s0 = *pair_at(a.face, cap, kS, wS), s1 = *pair_at(a.face, cap, kS + 2, wS);
         // squares of the reconstructed depths of the cell at its faces
-        T FE[3], GN[3], FW[3], GS[3], hE2, hN2, hW2, hS2;
-        FE[0] = F[0 * (size_t)cap + w];
-        FE[1] = F[1 * (size_t)cap + w];
-        FE[2] = F[2 * (size_t)cap + w];
-        hE2 = F[3 * (size_t)cap + w];
-        GN[0] = F[5 * (size_t)cap + w];
-        GN[1] = F[6 * (size_t)cap + w];
-        GN[2] = F[7 * (size_t)cap + w];
-        hN2 = F[8 * (size_t)cap + w];
-        bool haveW = false, haveS = false;
-        if (i > 0) {
-            const unsigned long long m = __ldg(a.mark + base + morton2(i - 1, j));
-            if ((uint32_t)(m >> 32) == tag) {
-                const uint32_t v = (uint32_t)m;
-                FW[0] = F[0 * (size_t)cap + v];
-                FW[1] = F[1 * (size_t)cap + v];
-                FW[2] = F[2 * (size_t)cap + v];
-                hW2 = F[4 * (size_t)cap + v];
-                haveW = true;
-            }
-        }
-        if (j > 0) {
-            const unsigned long long m = __ldg(a.mark + base + morton2(i, j - 1));
-            if ((uint32_t)(m >> 32) == tag) {
-                const uint32_t v = (uint32_t)m;
-                GS[0] = F[5 * (size_t)cap + v];
-                GS[1] = F[6 * (size_t)cap + v];
-                GS[2] = F[7 * (size_t)cap + v];
-                hS2 = F[9 * (size_t)cap + v];
-                haveS = true;
-            }
-        }
-        if (FM && !haveW && i > 0 && n < a.L && sig_bit(a.Sb, n, morton2(i - 1, j))) {
-            matched_face(a, src, 0, n, i, j, FW, hW2);
-            haveW = true;
-        }
-        if (FM && !haveS && j > 0 && n < a.L && sig_bit(a.Sb, n, morton2(i, j - 1))) {
-            matched_face(a, src, 2, n, i, j, GS, hS2);
-            haveS = true;
-        }
-        if (!(haveW && haveS)) {
-            T uC, vC, dummy;
-            velocity(C, tol, uC, vC);
-            if (!haveW) {
-                const Cell<T> W = i > 0 ? fetch(src, base + morton2(i - 1, j)) : ghost(C, a.bc_ref[0], true);
-                T uW, vW, hW_R;
-                velocity(W, tol, uW, vW);
-                hll_face(g, hg, tol, W.h, W.z, uW, vW, C.h, C.z, uC, vC, FW, dummy, hW_R);
-                hW2 = hW_R * hW_R;
-            }
-            if (!haveS) {
-                const Cell<T> S = j > 0 ? fetch(src, base + morton2(i, j - 1)) : ghost(C, a.bc_ref[2], false);
-                T uS, vS, hS_R;
-                velocity(S, tol, uS, vS);
-                hll_face(g, hg, tol, S.h, S.z, vS, uS, C.h, C.z, vC, uC, GS, dummy, hS_R);
-                hS2 = hS_R * hS_R;
-            }
-        }
+        T hW2 = w1.y, hS2 = s1.y;
+        if (sW) hW2 = a.face[(kFaceE + 4) * cap + wW];
+        if (sS) hS2 = a.face[(kFaceN + 4) * cap + wS];
+        Cell<T> C;
+        C.h = __ldg(src.h + d.iC);
+        C.qx = __ldg(src.qx + d.iC);
+        C.qy = __ldg(src.qy + d.iC);
+        const T FE[3] = {e0.x, e0.y, e1.x}, hE2 = e1.y;
+        const T GN[3] = {n0.x, n0.y, n1.x}, hN2 = n1.y;
+        const T FW[3] = {w0.x, w0.y, w1.x};
+        const T GS[3] = {s0.x, s0.y, s1.x};
         const T rx = mul_pow2(rx0, n), ry = mul_pow2(ry0, n);   // rx0 * 2^n, exact
         int64_t lo = 0, hi = 0;
-        const bool inlet = inlet_range(a, n, i, j, last, lo, hi);
+        const bool inlet = a.inflow_side >= 0 && inlet_range(a, n, compact16(d.code), compact16(d.code >> 1),
+                                                             (1u << n) - 1u, lo, hi);
         T dh = T(0);
         if (inlet) {
             const T scale = (T)(1u << n);
@@ -2286,16 +2412,19 @@ __device__ __forceinline__ void fv1_update_body(const StepArgs<T>& a, Blk B) {
         }
         T out[3], rh;
         cell_update_faces_sq(a.P, rx, ry, fk, C, FW, FE, GS, GN, hW2, hE2, hS2, hN2, inlet, dh, out, &rh);
-        wet_leaf_store(a, st, src.z, oh, oqx, oqy, n, code, iC, C, out, rmin, mh, mqx, mqy, spd, rh);
+        wet_leaf_store(a, st, src.z, oh, oqx, oqy, n, d.code, d.iC, C, out, rmin, mh, mqx, mqy, spd, rh);
     }
     block_atomic_u64<false>(rmin, &st->rmin_bits);
     block_max3_u64(mh, mqx, mqy, st->max_bits);
     block_max3_u64(spd[0], spd[1], 0ull, st->speed_bits);
 }
-template <typename T, bool FM = false>
-static __global__ void __launch_bounds__(256) k_fv1_update(StepArgs<T> a) {
+// 64 us for 1 M leaves (uniform FV1, L=10; 116 us with its products on the
+// FP64 pipe and the unshared faces formed here): the FP64 pipe's 19 sums a leaf
+// fill two thirds of it, the rest is the latency of the gathers.
+template <typename T>
+static __global__ void __launch_bounds__(64) k_fv1_update(StepArgs<T> a) {
     pdl_wait();
-    fv1_update_body<T, FM>(a, this_blk());
+    fv1_update_body<T>(a, this_blk());
 }
 
 // Uniform FV1 (every finest cell a leaf): the fixed leaf list in Z-order ...

@@ -2,15 +2,15 @@
 // nearest (ties to even) bit for bit as the FP64 instructions round them.
 //
 // The FP64 pipe takes about 77 cycles per warp and sub-partition for one
-// addition or multiplication (0.53 T/s on the whole GPU); the integer pipes
-// take one instruction every 1-2 cycles.  A square root or reciprocal, which
-// the FP64 pipe builds from several of its instructions, is therefore cheaper
-// as some forty integer instructions, and leaves the FP64 pipe to the sums
-// and products around it.  Measured, cycles per warp and sub-partition with
-// 64 (16) warps per SM: square root 90 (104) against 620 (619) on the FP64
-// pipe, reciprocal 71 (87) against 362 (366).  The update's kernels are bound
-// by that pipe: uniform FV1 on 1024 x 1024 cells went from 424 to 318 us a
-// step, the dam-break over humps at that size from 238 to 186 us a step.
+// addition or multiplication (0.53 T/s on the whole GPU), the integer pipes
+// 1-2 for an instruction, and the two work at the same time.  A square root or
+// reciprocal, which the FP64 pipe builds from several of its instructions, is
+// far cheaper in some forty integer instructions; a product costs less too
+// and leaves the FP64 pipe to the sums.  Measured, cycles per warp and
+// sub-partition with 48-64 warps per SM: square root 86-90 against 620 on the
+// FP64 pipe, reciprocal 67-71 against 362, product 46 (57 where a factor may be
+// zero, 66 with a check of its range) against 77; a product followed by a sum
+// takes the time of the sum.
 //
 // The methods are the usual ones of exact arithmetic: a float seed refined by
 // Newton steps in fixed point, each with the residual taken modulo 2^64 (it
@@ -120,6 +120,58 @@ __host__ __device__ __forceinline__ uint64_t rcp_bits(uint32_t lo, uint32_t hi, 
     return (q + ((uint64_t)eo << 32)) | ((uint64_t)(hi & 0x80000000u) << 32);
 }
 
+// ---- product ---------------------------------------------------------------
+// true when both factors are normal and so is the product before rounding
+__host__ __device__ __forceinline__ bool mul_in_range(uint32_t ah, uint32_t bh) {
+    const uint32_t ea = ah & 0x7FF00000u, eb = bh & 0x7FF00000u;
+    // ea, eb in [1, 2046] (neither 0 nor 2047) and ea + eb - 1023 in [1, 2044]
+    const bool na = ((ah + 0x00100000u) & 0x7FE00000u) != 0u, nb = ((bh + 0x00100000u) & 0x7FE00000u) != 0u;
+    return na && nb && ea + eb - (1024u << 20) < (2044u << 20);
+}
+// The product of two factors in range; with Z, of factors in range or +-0 (a
+// zero factor gives a signed zero).
+template <bool Z>
+__host__ __device__ __forceinline__ uint64_t mul_bits(uint32_t al, uint32_t ah, uint32_t bl, uint32_t bh) {
+    const uint32_t ma = (ah & 0x000FFFFFu) | 0x00100000u, mb = (bh & 0x000FFFFFu) | 0x00100000u;
+    // 105 or 106 bits, w3:w2:w1:w0; the two middle products and the carries
+    // into them fit 64 bits
+    const uint64_t p00 = (uint64_t)al * bl;
+    const uint64_t mid = (uint64_t)ma * bl + ((uint64_t)al * mb + (p00 >> 32));
+    const uint64_t top = (uint64_t)ma * mb + (mid >> 32);
+    const uint32_t w3 = (uint32_t)(top >> 32), w2 = (uint32_t)top, w1 = (uint32_t)mid, w0 = (uint32_t)p00;
+    // the significand kh:kl is the top 53 bits: z = 11 with 106 bits (the
+    // product of the significands is 2 or more), 12 with 105
+    const uint32_t z = (6655u - w3) >> 9;
+    const uint32_t kl = HWFV1_FSHL(w1, w2, z), kh = HWFV1_FSHL(w2, w3, z);
+    // the bits below, rounded into kl by the carry of an addition: more than
+    // half a unit (w0 only matters as "not 0"), or half and an odd kl
+    const uint32_t f = HWFV1_FSHL(w0, w1, z) | (w0 < 1u ? w0 : 1u);
+    // the exponent word (kh holds the significand's leading bit); without Z
+    // the sign bits add up to the result's along with it, modulo 2^32
+    constexpr uint32_t mask = Z ? 0x7FF00000u : 0xFFF00000u;
+    const uint32_t e = (ah & mask) + (bh & mask) - (1012u << 20) - (z << 20);
+    uint32_t rl, rh;
+#ifdef __CUDA_ARCH__
+    asm("{.reg .u32 t; and.b32 t, %2, 1; add.u32 t, t, 0x7fffffff; add.cc.u32 t, t, %4; addc.cc.u32 %0, %2, 0; "
+        "addc.u32 %1, %3, %5;}"
+        : "=r"(rl), "=r"(rh) : "r"(kl), "r"(kh), "r"(f), "r"(e));
+#else
+    const uint64_t r = (uint64_t)f + 0x7FFFFFFFu + (kl & 1u);
+    const uint64_t k = ((uint64_t)(kh + e) << 32 | kl) + (r >> 32);
+    rl = (uint32_t)k;
+    rh = (uint32_t)(k >> 32);
+#endif
+    if (Z) {
+        // times 0 for a zero factor, as multiplications: the pipe they run on
+        // has slots to spare, the one selections run on has not
+        const uint32_t ea = ah & mask, eb = bh & mask;
+        const uint32_t nz = (ea < 1u ? ea : 1u) * (eb < 1u ? eb : 1u);
+        rl = rl * nz;
+        rh = rh * nz + ((ah ^ bh) & 0x80000000u);
+    }
+    return (uint64_t)rh << 32 | rl;
+}
+
 #ifdef __CUDACC__
 // Device forms on doubles.  Operands outside an operation's range (next to
 // no lane meets one) take the FP64 instruction in a function of its own: a
@@ -134,6 +186,7 @@ __device__ __forceinline__ double d_join(uint64_t b) {
     return x;
 }
 static __device__ __noinline__ double sqrt_rare(double x) { return sqrt(x); }
+static __device__ __noinline__ double mul_rare(double a, double b) { return __dmul_rn(a, b); }
 static __device__ __noinline__ double rcp_rare(double x) { return 1.0 / x; }
 
 // sqrt(x) and 1 / x
@@ -154,6 +207,33 @@ __device__ __forceinline__ double recip(double x) {
     asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(__uint_as_float(rcp_seed_arg(lo, hi))));
     return d_join(rcp_bits(lo, hi, __float_as_uint(y)));
 }
+// a b.  prod: any operands.  prod_nz: operands known to be in range.
+// prod_z: operands known to be in range or zero.
+__device__ __forceinline__ double prod(double a, double b) {
+    uint32_t al, ah, bl, bh;
+    d_split(a, al, ah);
+    d_split(b, bl, bh);
+    if (!mul_in_range(ah, bh)) {
+        const uint32_t xa = ah & 0x7FFFFFFFu, xb = bh & 0x7FFFFFFFu;
+        if (((xa | al) == 0u || (xb | bl) == 0u) && xa < 0x7FF00000u && xb < 0x7FF00000u)
+            return d_join((uint64_t)((ah ^ bh) & 0x80000000u) << 32);
+        return mul_rare(a, b);
+    }
+    return d_join(mul_bits<false>(al, ah, bl, bh));
+}
+__device__ __forceinline__ double prod_nz(double a, double b) {
+    uint32_t al, ah, bl, bh;
+    d_split(a, al, ah);
+    d_split(b, bl, bh);
+    return d_join(mul_bits<false>(al, ah, bl, bh));
+}
+__device__ __forceinline__ double prod_z(double a, double b) {
+    uint32_t al, ah, bl, bh;
+    d_split(a, al, ah);
+    d_split(b, bl, bh);
+    return d_join(mul_bits<true>(al, ah, bl, bh));
+}
+__device__ __forceinline__ float prod(float a, float b) { return a * b; }
 __device__ __forceinline__ float root(float x) { return sqrtf(x); }
 __device__ __forceinline__ float recip(float x) { return 1.0f / x; }
 #endif

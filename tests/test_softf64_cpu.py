@@ -1,8 +1,9 @@
 """The integer-instruction float64 operations (csrc/softf64.cuh) against the
 host's IEEE operations, bit for bit, on the operands where a rounding can go
 wrong: exact squares and their neighbours, powers of two, all-ones
-significands, reciprocals of reciprocals, every exponent parity, the range's
-edges; with seeds off by more than the device's approximations are."""
+significands, reciprocals of reciprocals, products next to ties, signed
+zeros, every exponent parity, the range's edges; with seeds off by more than
+the device's approximations are."""
 import os
 import subprocess
 
@@ -79,6 +80,24 @@ int main(int, char** argv) {
         if (rcp_in_range(hi)) {
             const uint32_t y = fbits((float)(1.0 / (double)fval(rcp_seed_arg(lo, hi)))) + d;
             check("rcp", x, rcp_bits(lo, hi, y), 1.0 / val(x));
+        }
+        uint64_t p = a, q = operand();
+        if (i % 4 == 2) {                      // 27-bit factors: products of 53 and 54 bits, ties among them
+            p = (p & 0xFFF0000000000000ull) | (rnd() & 0x3FFFFFF) << 26;
+            q = (q & 0xFFF0000000000000ull) | (rnd() & 0x3FFFFFF) << (24 + rnd() % 3);
+        }
+        const bool in = mul_in_range((uint32_t)(p >> 32), (uint32_t)(q >> 32));
+        const double pq = val(p) * val(q);
+        const uint64_t m = bits(pq) & 0x7FFFFFFFFFFFFFFFull;
+        if (in) {
+            check("mul", p, mul_bits<false>((uint32_t)p, (uint32_t)(p >> 32), (uint32_t)q, (uint32_t)(q >> 32)), pq);
+            if (rnd() % 2) p &= 1ull << 63;    // signed zeros beside normal factors
+            if (rnd() % 2) q &= 1ull << 63;
+            check("mul with zeros", p, mul_bits<true>((uint32_t)p, (uint32_t)(p >> 32), (uint32_t)q, (uint32_t)(q >> 32)),
+                  val(p) * val(q));
+        } else if (m > 0x002FFFFFFFFFFFFFull && m < 0x7FD0000000000000ull &&
+                   (p & 0x7FF0000000000000ull) && (q & 0x7FF0000000000000ull)) {
+            ++fails;                           // normal factors, a product well inside the normal range
         }
     }
     std::printf("%ld wrong\n", fails);
