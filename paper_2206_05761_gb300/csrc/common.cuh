@@ -263,6 +263,8 @@ struct DevState {
     uint32_t epoch;                   // completed steps (never reset; tags the face stamps)
     uint32_t enc_ticket;              // finished CTAs of the fused last encode passes
     uint32_t dec_ticket;              // finished CTAs of the fused decode + finish
+    unsigned long long in_bits[3];    // max |h|, |qx|, |qy| of fields coming in (set_fields; 0 between calls)
+    uint32_t in_ticket;               // finished CTAs of the fields-in kernel
     uint32_t ntodo;                   // tiles the first encode pass works on (listed by the
                                       // clear kernel, reset by the encode's last CTA)
 };

@@ -1,6 +1,6 @@
 // engine.cuh -- host side of one HWFV1 simulation: device buffers, the
 // launch sequence of a timestep, CUDA-graph replay, checkpoints, host field
-// transfers (and k_quiet_tiles, a kernel only the initialisation launches).
+// transfers.
 #pragma once
 #include <algorithm>
 #include <cmath>
@@ -16,24 +16,6 @@
 #include "skipnet.h"
 
 namespace hwfv1 {
-
-// Quiescence marks of an initial state, one field at a time: zf[t] (set to
-// 1 beforehand) is cleared where the finest values of field x in tile t
-// (4^kt consecutive Morton codes) are not all +0.  The tiles' coarser levels
-// were cleared beforehand, so a mark left at 1 holds for them too.  One warp
-// per tile.
-template <typename T>
-static __global__ void k_quiet_tiles(const T* __restrict__ x, uint8_t* __restrict__ zf, uint32_t ntiles, int kt) {
-    const uint32_t lane = threadIdx.x & 31u, cells = 1u << (2 * kt);
-    const uint32_t nw = (gridDim.x * blockDim.x) >> 5;
-    for (uint32_t t = (blockIdx.x * blockDim.x + threadIdx.x) >> 5; t < ntiles; t += nw) {   // warp-uniform
-        const uint64_t b = (uint64_t)t * cells;
-        bool nz = false;
-        for (uint32_t i = lane; i < cells; i += 32u) nz |= !pos_zero(x[b + i]);
-        nz = __any_sync(0xffffffffu, nz);
-        if (lane == 0u && nz) zf[t] = 0;
-    }
-}
 
 // Kernel nodes of a captured graph (memset and copy nodes are not counted).
 inline int64_t count_kernel_nodes(cudaGraph_t g) {
@@ -175,8 +157,8 @@ class EngineT final : public Engine {
         quiet_on_ = !(spec_.flags & HWFV1_FULL_SWEEP) && spec_.eps >= 1e-30;
         // With quiescent tiles on, the first step starts from marks as a
         // later step does: both buffers are cleared (buffer 0 below its
-        // finest level, which the fields fill) and the tiles of +0 marked
-        // once the fields are in (k_quiet_tiles), so that the first encode,
+        // finest level, which the fields fill) and the tiles of +0 stay marked
+        // as the fields come in (k_fields_in), so that the first encode,
         // traversal and decode skip them as well.
         if (quiet_on_)
             for (int q = 0; q < 3; ++q) {
@@ -217,17 +199,16 @@ class EngineT final : public Engine {
             cudaMemcpyAsync(st_, &s0, sizeof s0, cudaMemcpyHostToDevice, stream_);
             cudaStreamSynchronize(stream_);
         }
-        // finest fields into the Morton hierarchy, the bed's first
+        // finest fields into the Morton hierarchy, the bed's first (with its
+        // s_max), then its thresholds, one-off encode and static flags
         const int g = grid_for(N_);
-        k_rm_to_morton<T><<<g, 256, 0, stream_>>>(field(0), z_ + lvl_off(L_), L_);
-        converted(0);
-        if (!copy_in(2)) return fail(HWFV1_ERR_CUDA, "init: copy of a host field");
-        // bed: s_max, thresholds, one-off encode and its static flags
         unsigned long long* zmax = reinterpret_cast<unsigned long long*>(zaux_);
         double* smax_z = reinterpret_cast<double*>(zaux_ + 8);
         double* thr_zd = reinterpret_cast<double*>(zaux_ + kZThrD);
         float* thr_zf = reinterpret_cast<float*>(zaux_ + kZThrF);
-        k_maxabs<T><<<g, 256, 0, stream_>>>(z_ + lvl_off(L_), N_, zmax);
+        field_in(field(0), z_ + lvl_off(L_), zmax, nullptr);
+        converted(0);
+        if (!copy_in(2)) return fail(HWFV1_ERR_CUDA, "init: copy of a host field");
         k_z_thresholds<<<1, 32, 0, stream_>>>(zmax, thr_zd, thr_zf, reinterpret_cast<double*>(zaux_ + kZThr4D),
                                               reinterpret_cast<float*>(zaux_ + kZThr4F), smax_z, L_, spec_.eps,
                                               st_);
@@ -254,13 +235,9 @@ class EngineT final : public Engine {
         if (quiet_on_) cudaMemsetAsync(tilebytes_, 1, (size_t)ntiles_ * 2, stream_);   // both buffers +0 so far
         k_reset_red<<<1, 32, 0, stream_>>>(st_);
         for (int q = 0; q < 3; ++q) {
-            T* const x = f_[0][q] + lvl_off(L_);
-            k_rm_to_morton<T><<<g, 256, 0, stream_>>>(field(1 + q), x, L_);
+            field_in(field(1 + q), f_[0][q] + lvl_off(L_), &st_->max_bits[q], quiet_on_ ? tilebytes_ : nullptr);
             converted(1 + q);
             if (q == 0 && !copy_in(3)) return fail(HWFV1_ERR_CUDA, "init: copy of a host field");
-            k_maxabs_cur<T><<<g, 256, 0, stream_>>>(x, f_[1][q] + lvl_off(L_), st_, N_, q);
-            if (quiet_on_)
-                k_quiet_tiles<T><<<grid_for((uint64_t)ntiles_ * 32), 256, 0, stream_>>>(x, tilebytes_, ntiles_, kt_);
         }
         // initial state scalars: the CFL step over the three fields
         k_cfl_cur<T><<<g, 256, 0, stream_>>>(f_[0][0] + lvl_off(L_), f_[1][0] + lvl_off(L_), f_[0][1] + lvl_off(L_),
@@ -510,24 +487,23 @@ class EngineT final : public Engine {
             if (hwfv1_status r = stage_alloc(&stg.p); r != HWFV1_OK) return r;
         }
         double* const stage = stg.p;
+        // device outputs in one pass
+        double* dev[3];
+        for (int q = 0; q < 3; ++q) dev[q] = hostp[q] ? nullptr : out[q];
+        if (dev[0] || dev[1] || dev[2]) fields_out(dev, other);
         int j = 0;
         for (int q = 0; q < 3; ++q) {
-            if (!out[q]) continue;
-            double* dst = out[q];
-            if (hostp[q]) {
-                if (j >= 2) cudaStreamWaitEvent(stream_, hev_[j - 2], 0);
-                dst = stage + (size_t)(j & 1) * N_;
-            }
-            k_morton_to_rm<T><<<grid_for(N_), 256, 0, stream_>>>(
-                f_[other ? 1 : 0][q] + lvl_off(L_), f_[other ? 0 : 1][q] + lvl_off(L_), st_, dst, L_);
-            if (hostp[q]) {
-                cudaEventRecord(hev_[4 + j], stream_);
-                cudaStreamWaitEvent(cstream_, hev_[4 + j], 0);
-                if (cudaMemcpyAsync(out[q], dst, N_ * sizeof(double), cudaMemcpyDeviceToHost, cstream_) != cudaSuccess ||
-                    cudaEventRecord(hev_[j], cstream_) != cudaSuccess)
-                    return fail(HWFV1_ERR_CUDA, "get_fields: copy to a host field");
-                ++j;
-            }
+            if (!hostp[q]) continue;
+            double* one[3] = {nullptr, nullptr, nullptr};
+            if (j >= 2) cudaStreamWaitEvent(stream_, hev_[j - 2], 0);
+            one[q] = stage + (size_t)(j & 1) * N_;
+            fields_out(one, other);
+            cudaEventRecord(hev_[4 + j], stream_);
+            cudaStreamWaitEvent(cstream_, hev_[4 + j], 0);
+            if (cudaMemcpyAsync(out[q], one[q], N_ * sizeof(double), cudaMemcpyDeviceToHost, cstream_) != cudaSuccess ||
+                cudaEventRecord(hev_[j], cstream_) != cudaSuccess)
+                return fail(HWFV1_ERR_CUDA, "get_fields: copy to a host field");
+            ++j;
         }
         if (!any_host) return check("get_fields");
         for (int k = 0; k < j; ++k) cudaStreamWaitEvent(stream_, hev_[k], 0);
@@ -536,14 +512,34 @@ class EngineT final : public Engine {
 
     hwfv1_status set_fields(const double* h, const double* qx, const double* qy) override {
         const double* in[3] = {h, qx, qy};
+        FieldsIn<T, 3> a;
+        bool v16 = true;
         for (int q = 0; q < 3; ++q) {
             if (!in[q]) return fail(HWFV1_ERR_INVALID_SPEC, "set_fields: NULL field");
-            k_rm_to_morton_cur<T><<<grid_for(N_), 256, 0, stream_>>>(
-                in[q], f_[0][q] + lvl_off(L_), f_[1][q] + lvl_off(L_), st_, L_);
+            v16 = v16 && aligned16(in[q]);
+            a.src[q] = in[q];
+            for (int b = 0; b < 2; ++b) a.dst[b][q] = f_[b][q] + lvl_off(L_);
         }
-        forget_quiet();
+        // the current buffer's marks survive where the new values are +0 too,
+        // the other buffer's all do (it keeps what it holds); the skip modes
+        // keep no marks
+        if (skipmode_) {
+            forget_quiet();
+        } else if (quiet_on_) {
+            a.zf[0] = tilebytes_;
+            a.zf[1] = tilebytes_ + ntiles_;
+            a.keep = 1;
+        }
         stored_at_finest();
-        reduce_state(/*set_dt=*/0);
+        a.max_bits = st_->in_bits;
+        a.st = st_;
+        a.ticket = &st_->in_ticket;
+        a.fin = fin_args();
+        a.ntiles = ntiles_;
+        a.L = L_;
+        a.kt = kt_;
+        if (v16) k_fields_in<T, 3, true><<<tile_grid(), 256, 0, stream_>>>(a);
+        else k_fields_in<T, 3, false><<<tile_grid(), 256, 0, stream_>>>(a);
         return check("set_fields");
     }
 
@@ -896,6 +892,46 @@ class EngineT final : public Engine {
         const uint64_t cap = (uint64_t)nsm_ * 8;
         if (g > cap) g = cap;
         return g < 1 ? 1 : (int)g;
+    }
+    // one CTA per tile, at most 8 per SM
+    int tile_grid() const { return (int)std::min<uint32_t>(ntiles_, (uint32_t)nsm_ * 8u); }
+    static bool aligned16(const void* p) { return (reinterpret_cast<uintptr_t>(p) & 15u) == 0; }
+    // one field (the bed, or at init h, qx or qy) into buffer 0
+    void field_in(const double* src, T* dst, unsigned long long* max_bits, uint8_t* zf) {
+        FieldsIn<T, 1> a;
+        a.src[0] = src;
+        a.dst[0][0] = a.dst[1][0] = dst;
+        a.zf[0] = a.zf[1] = zf;
+        a.max_bits = max_bits;
+        a.st = st_;
+        a.fin = FinishArgs();
+        a.ntiles = ntiles_;
+        a.L = L_;
+        a.kt = kt_;
+        if (aligned16(src)) k_fields_in<T, 1, true><<<tile_grid(), 256, 0, stream_>>>(a);
+        else k_fields_in<T, 1, false><<<tile_grid(), 256, 0, stream_>>>(a);
+    }
+    // the finest fields to row-major device arrays (NULL: not wanted); other:
+    // from the buffer that is not current (marks unknown there)
+    void fields_out(double* const dst[3], bool other) {
+        FieldsOut<T> a;
+        bool v16 = true;
+        for (int q = 0; q < 3; ++q) {
+            a.dst[q] = dst[q];
+            v16 = v16 && aligned16(dst[q]);
+            for (int b = 0; b < 2; ++b) a.src[b][q] = f_[b][q] + lvl_off(L_);
+        }
+        if (quiet_on_ && !other) {
+            a.zf[0] = tilebytes_;
+            a.zf[1] = tilebytes_ + ntiles_;
+        }
+        a.st = st_;
+        a.ntiles = ntiles_;
+        a.L = L_;
+        a.kt = kt_;
+        a.other = other ? 1 : 0;
+        if (v16) k_fields_out<T, true><<<tile_grid(), 256, 0, stream_>>>(a);
+        else k_fields_out<T, false><<<tile_grid(), 256, 0, stream_>>>(a);
     }
     int predict() const { return (spec_.flags & HWFV1_REG_PREDICT) ? 1 : 0; }
     int close() const { return (spec_.flags & HWFV1_REG_CLOSE) ? 1 : 0; }

@@ -2715,11 +2715,12 @@ static __global__ void k_set_tend(DevState* st, FinishArgs a, double t_end) {
     set_tend_body(st, a, t_end);
 }
 
-// State from the reductions of the initial (or reloaded) fields:
-// s_max from max_bits[0..2], and, if set_dt, dt from rmin_bits.
-static __global__ void k_init_state(DevState* st, FinishArgs a, int set_dt) {
+// State from the reductions of the initial (or reloaded) fields: s_max from
+// their maxima, and, if set_dt, dt from rmin_bits.
+__device__ __forceinline__ void init_state_body(DevState* st, const FinishArgs& a, const unsigned long long* max_bits,
+                                                int set_dt) {
     if (threadIdx.x == 0) {
-        for (int q = 0; q < 3; ++q) st->smax[q] = smax_of(st->max_bits[q]);
+        for (int q = 0; q < 3; ++q) st->smax[q] = smax_of(__ldcg(max_bits + q));
         // a NaN or inf anywhere in the fields shows up in its maximum
         for (int q = 0; q < 3; ++q)
             if (!isfinite(st->smax[q])) st->err |= kErrNonFinite;
@@ -2727,6 +2728,9 @@ static __global__ void k_init_state(DevState* st, FinishArgs a, int set_dt) {
     }
     __syncthreads();
     prepare_step(st, a);
+}
+static __global__ void k_init_state(DevState* st, FinishArgs a, int set_dt) {
+    init_state_body(st, a, st->max_bits, set_dt);
 }
 
 // z thresholds for the one-off bed encode
@@ -2748,18 +2752,6 @@ static __global__ void k_z_thresholds(const unsigned long long* zmax_bits, doubl
 // ---------------------------------------------------------------------------
 // Reductions over the finest grid (initial state)
 // ---------------------------------------------------------------------------
-template <typename T>
-static __global__ void __launch_bounds__(256) k_maxabs(const T* __restrict__ x, uint64_t n,
-                                                unsigned long long* dst) {
-    unsigned long long m = 0;
-    for (uint64_t i = blockIdx.x * (uint64_t)blockDim.x + threadIdx.x; i < n;
-         i += (uint64_t)gridDim.x * blockDim.x) {
-        const unsigned long long b = abs_obits(x[i]);
-        m = b > m ? b : m;
-    }
-    block_atomic_u64<true>(m, dst);
-}
-
 template <typename T>
 static __global__ void __launch_bounds__(256) k_cfl_finest(const T* __restrict__ h, const T* __restrict__ qx,
                                                     const T* __restrict__ qy, uint64_t n, Phys<T> P,
@@ -2813,29 +2805,160 @@ static __global__ void __launch_bounds__(256) k_cfl_cur(const T* h0, const T* h1
 }
 
 // ---------------------------------------------------------------------------
-// Layout conversion: row-major (j*2^L + i, float64) <-> Morton (type T)
+// Layout conversion: row-major (j*2^L + i, float64) <-> Morton (type T), one
+// CTA per traversal tile, one thread per 2 x 2 cells: four consecutive Morton
+// codes, two neighbours in each of two rows.  A warp covers 16 x 8 cells, rows
+// of 128 bytes.  V16: the row-major pointers are 16-byte aligned.
 // ---------------------------------------------------------------------------
-template <typename T>
-static __global__ void k_rm_to_morton(const double* __restrict__ src, T* __restrict__ dst, int L) {
-    const uint64_t N = 1ull << (2 * L);
-    for (uint64_t m = blockIdx.x * (uint64_t)blockDim.x + threadIdx.x; m < N;
-         m += (uint64_t)gridDim.x * blockDim.x) {
-        const uint32_t i = compact16((uint32_t)m), j = compact16((uint32_t)(m >> 1));
-        dst[m] = (T)src[((uint64_t)j << L) + i];
+struct QuadPos {
+    uint64_t rm;        // row-major index of the quad's first cell
+    uint32_t m;         // Morton code of it
+    bool on;
+};
+__device__ __forceinline__ QuadPos quad_pos(int L, int kt, uint32_t tile) {
+    const uint32_t t = threadIdx.x;
+    QuadPos p;
+    p.on = t < (1u << (2 * (kt - 1)));
+    const uint32_t i = (compact16(tile) << kt) + 2u * compact16(t);
+    const uint32_t j = (compact16(tile >> 1) << kt) + 2u * compact16(t >> 1);
+    p.rm = ((uint64_t)j << L) + i;
+    p.m = (tile << (2 * kt)) + 4u * t;
+    return p;
+}
+template <bool V16>
+__device__ __forceinline__ double2 load_rm(const double* p) {
+    return V16 ? __ldcs(reinterpret_cast<const double2*>(p)) : make_double2(__ldcs(p), __ldcs(p + 1));
+}
+template <bool V16>
+__device__ __forceinline__ void store_rm(double* p, double a, double b) {
+    if (V16) {
+        __stcs(reinterpret_cast<double2*>(p), make_double2(a, b));
+    } else {
+        __stcs(p, a);
+        __stcs(p + 1, b);
     }
 }
 
-// dst_rm[j*2^L+i] = src[Morton(i,j)]; src chosen by the current buffer when
-// `src2` is given (src = buffer 0, src2 = buffer 1)
+// Fields in: NF fields into the finest level (of the current buffer where dst
+// names two), with their maxima of |x| and the tiles' quiescence marks in the
+// same pass: a mark survives where the new values are all +0 (the tile's
+// coarser levels, which it covers too, are left as they are).  keep: what a
+// marked tile holds is +0 already, so its new +0 values are not written.  With
+// a ticket, the last CTA sets the step's scalars from the maxima (set_fields).
+//
+// Bound by HBM: L=12, three fields: 805 MB, 403 MB where everything is +0.  One
+// pass instead of a conversion and a reduction per field (51 + 31 us each) took
+// the MRA of the terrain flood at L=12 (new fields, encode, leaves) from 678 to
+// 239 us together with the kept marks, which spare its encode the dry tiles.
+template <typename T, int NF>
+struct FieldsIn {
+    const double* src[NF];
+    T* dst[2][NF];
+    uint8_t* zf[2] = {nullptr, nullptr};   // NULL: no marks
+    unsigned long long* max_bits;          // NF words, max-reduced
+    DevState* st;
+    uint32_t* ticket = nullptr;
+    FinishArgs fin;
+    uint32_t ntiles;
+    int L, kt, keep = 0;
+};
+template <typename T, int NF, bool V16>
+static __global__ void __launch_bounds__(256) k_fields_in(FieldsIn<T, NF> a) {
+    const bool c = a.st->cur != 0u;
+    uint8_t* const zf = c ? a.zf[1] : a.zf[0];
+    unsigned long long mx[NF];
+#pragma unroll
+    for (int q = 0; q < NF; ++q) mx[q] = 0ull;
+    for (uint32_t tile = blockIdx.x; tile < a.ntiles; tile += gridDim.x) {
+        const QuadPos p = quad_pos(a.L, a.kt, tile);
+        const bool old = zf != nullptr && zf[tile] != 0;
+        double2 u[NF], v[NF];
+        if (p.on) {
+#pragma unroll
+            for (int q = 0; q < NF; ++q) {
+                u[q] = load_rm<V16>(a.src[q] + p.rm);
+                v[q] = load_rm<V16>(a.src[q] + p.rm + (1ull << a.L));
+            }
+        }
+        bool nz = false;
+        T x[NF][4];
+        if (p.on) {
+#pragma unroll
+            for (int q = 0; q < NF; ++q) {
+                x[q][0] = (T)u[q].x;
+                x[q][1] = (T)u[q].y;
+                x[q][2] = (T)v[q].x;
+                x[q][3] = (T)v[q].y;
+#pragma unroll
+                for (int e = 0; e < 4; ++e) {
+                    const unsigned long long b = abs_obits(x[q][e]);
+                    mx[q] = b > mx[q] ? b : mx[q];
+                    nz = nz || !pos_zero(x[q][e]);
+                }
+            }
+        }
+        if (old) {
+            // (uniform over the CTA)
+            const bool any = __syncthreads_or(nz ? 1 : 0) != 0;
+            if (any && threadIdx.x == 0) zf[tile] = 0;
+            if (!any && a.keep) continue;
+        }
+        if (p.on) {
+#pragma unroll
+            for (int q = 0; q < NF; ++q)
+                Vec4<T>::store((c ? a.dst[1][q] : a.dst[0][q]) + p.m, x[q][0], x[q][1], x[q][2], x[q][3]);
+        }
+    }
+#pragma unroll
+    for (int q = 0; q < NF; ++q) block_atomic_u64<true>(mx[q], a.max_bits + q);
+    if (a.ticket == nullptr) return;
+    __threadfence();
+    __syncthreads();
+    __shared__ bool last;
+    if (threadIdx.x == 0) last = atomicAdd(a.ticket, 1u) == gridDim.x - 1u;
+    __syncthreads();
+    if (!last) return;
+    __threadfence();
+    init_state_body(a.st, a.fin, a.max_bits, 0);
+    __syncthreads();
+    if (threadIdx.x == 0) *a.ticket = 0u;
+    if (threadIdx.x < NF) a.max_bits[threadIdx.x] = 0ull;
+}
+
+// Fields out: the finest level of the current buffer (other: of the one that
+// is not) to row-major arrays (NULL: not wanted).  A marked tile (zf given) is
+// +0 and is not read.  Bound by HBM: L=12, three fields: 805 MB, 403 MB where
+// everything is marked.
 template <typename T>
-static __global__ void k_morton_to_rm(const T* __restrict__ src, const T* __restrict__ src2,
-                               const DevState* st, double* __restrict__ dst, int L) {
-    const T* s = (src2 && st && st->cur) ? src2 : src;
-    const uint64_t N = 1ull << (2 * L);
-    for (uint64_t r = blockIdx.x * (uint64_t)blockDim.x + threadIdx.x; r < N;
-         r += (uint64_t)gridDim.x * blockDim.x) {
-        const uint32_t i = (uint32_t)(r & ((1ull << L) - 1)), j = (uint32_t)(r >> L);
-        dst[r] = (double)s[morton2(i, j)];
+struct FieldsOut {
+    const T* src[2][3];
+    double* dst[3];
+    const uint8_t* zf[2] = {nullptr, nullptr};
+    const DevState* st;
+    uint32_t ntiles;
+    int L, kt, other;
+};
+template <typename T, bool V16>
+static __global__ void __launch_bounds__(256) k_fields_out(FieldsOut<T> a) {
+    const bool c = (a.st->cur != 0u) != (a.other != 0);
+    const uint8_t* const zf = c ? a.zf[1] : a.zf[0];
+    for (uint32_t tile = blockIdx.x; tile < a.ntiles; tile += gridDim.x) {
+        const QuadPos p = quad_pos(a.L, a.kt, tile);
+        if (!p.on) continue;
+        const bool zero = zf != nullptr && zf[tile] != 0;
+        T x[3][4];
+#pragma unroll
+        for (int q = 0; q < 3; ++q) {
+            x[q][0] = x[q][1] = x[q][2] = x[q][3] = T(0);
+            if (a.dst[q] && !zero)
+                Vec4<T>::load((c ? a.src[1][q] : a.src[0][q]) + p.m, x[q][0], x[q][1], x[q][2], x[q][3]);
+        }
+#pragma unroll
+        for (int q = 0; q < 3; ++q) {
+            if (!a.dst[q]) continue;
+            store_rm<V16>(a.dst[q] + p.rm, (double)x[q][0], (double)x[q][1]);
+            store_rm<V16>(a.dst[q] + p.rm + (1ull << a.L), (double)x[q][2], (double)x[q][3]);
+        }
     }
 }
 
@@ -2847,20 +2970,6 @@ static __global__ void k_copy_level(const T* __restrict__ src, const T* __restri
          i += (uint64_t)gridDim.x * blockDim.x)
         dst[i] = (double)s[i];
 }
-
-// into the current buffer (set_fields / load)
-template <typename T>
-static __global__ void k_rm_to_morton_cur(const double* __restrict__ src, T* dst0, T* dst1,
-                                   const DevState* st, int L) {
-    T* dst = st->cur ? dst1 : dst0;
-    const uint64_t N = 1ull << (2 * L);
-    for (uint64_t m = blockIdx.x * (uint64_t)blockDim.x + threadIdx.x; m < N;
-         m += (uint64_t)gridDim.x * blockDim.x) {
-        const uint32_t i = compact16((uint32_t)m), j = compact16((uint32_t)(m >> 1));
-        dst[m] = (T)src[((uint64_t)j << L) + i];
-    }
-}
-
 
 // ---------------------------------------------------------------------------
 // Learned look-ahead (subtree CNN).  A subtree is one cell of level
