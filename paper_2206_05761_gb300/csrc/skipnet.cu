@@ -3,8 +3,9 @@
 // operands staged in shared memory, FP32 accumulators in TMEM).
 //
 //   forward       Z[p][o]  = b[o] + sum_k Xcol[p][k] W[o][k]      M=128 pixels, N=16, K=48|144
-//   grad input    dXcol    = dZ W  -> scattered back (col2im)      M=128 pixels, N=K, K=16
-//   grad weights  dW[k][o] = sum_p Xcol[p][k] dZ[p][o]            M=128 k-rows, N=16, K=128 pixels
+//   grad input    dX[p][c] = sum_k dZcol[p][k] W'[c][k]           the same convolution of dZ with
+//                            the taps reversed and W transposed over its channels
+//   grad weights  dW[k][o] = sum_p Xcol[p][k] dZ[p][o]            M=128 k-rows, N=16, K=pixels
 //
 // k = tap * cin + c with tap = 3*(di+1) + (dj+1): the im2col of a 3x3 window
 // with zero padding over channels-last images.  Parameters are kept in FP32
@@ -39,25 +40,15 @@ __constant__ Layer c_layers[3] = {
 };
 constexpr uint32_t kWaitLimit = 1u << 24;   // polls of an mbarrier before giving up
 
-__device__ __forceinline__ void put_bf16(uint8_t* base, uint32_t off, bf16 v) {
-    *reinterpret_cast<bf16*>(base + off) = v;
-}
-
-__device__ __forceinline__ uint32_t tmem_cols_for(int n) {
-    uint32_t c = 32;
-    while ((int)c < n) c <<= 1;
-    return c;
-}
-
 // ---------------------------------------------------------------------------
-// Weight packing: FP32 [cout][cin][3][3] -> the B tiles of the forward GEMM
-// (N = 16 rows of cout, K = kpad) and of the input-gradient GEMM (N = kpad
-// rows, K = 16 cout), both in the core-matrix layout.
+// Weight packing: FP32 [cout][cin][3][3] -> the B tiles (N = 16 rows, K =
+// kpad, core-matrix layout) of the forward GEMM (rows cout) and, where cin is
+// 16, of the input gradient (rows cin, k = tap' * 16 + cout with tap' = 8 - tap).
 // ---------------------------------------------------------------------------
 __global__ void k_pack(const float* __restrict__ params, bf16* __restrict__ wf, bf16* __restrict__ wt) {
     const Layer ly = c_layers[blockIdx.y];
     bf16* f = wf + blockIdx.y * (16 * 144);
-    bf16* t = wt + blockIdx.y * (144 * 16);
+    bf16* t = wt + blockIdx.y * (16 * 144);
     for (int idx = threadIdx.x; idx < 16 * ly.kpad; idx += blockDim.x) {
         const int o = idx / ly.kpad, k = idx % ly.kpad;
         float v = 0.f;
@@ -65,62 +56,64 @@ __global__ void k_pack(const float* __restrict__ params, bf16* __restrict__ wf, 
             const int tap = k / ly.cin, c = k % ly.cin;
             v = params[ly.offw + (o * ly.cin + c) * 9 + tap];
         }
-        const bf16 b = __float2bfloat16(v);
-        f[tc::core_off(o, k, ly.kpad / 8) / 2] = b;
-        t[tc::core_off(k, o, 2) / 2] = b;
+        f[tc::core_off(o, k, ly.kpad / 8) / 2] = __float2bfloat16(v);
+    }
+    if (ly.cin != 16) return;
+    for (int idx = threadIdx.x; idx < 16 * 144; idx += blockDim.x) {
+        const int c = idx / 144, k = idx % 144, tap = 8 - k / 16, o = k % 16;
+        const float v = o < ly.cout ? params[ly.offw + (o * ly.cin + c) * 9 + tap] : 0.f;
+        t[tc::core_off(c, k, 18) / 2] = __float2bfloat16(v);
     }
 }
 
-// im2col value (pixel p, k) of a channels-last image batch
 struct Img {
     int B, H, W, cin;
 };
-__device__ __forceinline__ bf16 xcol(const bf16* __restrict__ X, const Img& g, int p, int k) {
-    const int npix = g.B * g.H * g.W;
-    if (p >= npix || k >= 9 * g.cin) return __float2bfloat16(0.f);
-    const int tap = k / g.cin, c = k % g.cin;
-    const int b = p / (g.H * g.W), rem = p % (g.H * g.W);
-    const int y = rem / g.W + tap / 3 - 1, x = rem % g.W + tap % 3 - 1;
-    if (y < 0 || y >= g.H || x < 0 || x >= g.W) return __float2bfloat16(0.f);
-    return X[((size_t)(b * g.H + y) * g.W + x) * g.cin + c];
-}
 
-// The im2col row of pixel p (k = tap * cin + c over the 3x3 taps, zero
-// outside the image and for k >= 9 cin) written to row `row` of the
-// core-matrix operand: the pixel's position is formed once, and each tap's
-// channels move as one 16-byte (cin % 8 == 0) or 8-byte (cin == 4) vector.
+// Which of the 9 taps of pixel p fall inside its image (none past the last
+// pixel).  Tap t of pixel p is pixel p + tap_shift(t, W).
+__device__ __forceinline__ uint32_t tap_mask(const Img& g, int p) {
+    if (p >= g.B * g.H * g.W) return 0u;
+    const int rem = p % (g.H * g.W), y = rem / g.W, x = rem % g.W;
+    const uint32_t row = (x > 0 ? 1u : 0u) | 2u | (x + 1 < g.W ? 4u : 0u);
+    return (y > 0 ? row : 0u) | (row << 3) | (y + 1 < g.H ? row << 6 : 0u);
+}
+__device__ __forceinline__ int tap_shift(int tap, int W) { return (tap / 3 - 1) * W + tap % 3 - 1; }
+
+// The im2col row of pixel p (k = tap * CIN + c over the 3x3 taps, zero
+// outside the image and for k >= 9 CIN) written to row `row` of the
+// core-matrix operand: every load first (16 bytes a piece, 8 for CIN = 4),
+// then the stores.
+template <int CIN>
 __device__ __forceinline__ void im2col_row(const bf16* __restrict__ X, const Img& g, int p, uint32_t row,
-                                           uint8_t* sA, int kpad) {
-    const uint32_t kb = (uint32_t)kpad / 8u;
-    const int npix = g.B * g.H * g.W;
-    if (g.cin % 8 != 0 && g.cin != 4) {
-        for (int k = 0; k < kpad; ++k) put_bf16(sA, tc::core_off(row, k, kb), xcol(X, g, p, k));
-        return;
-    }
-    const bool inside = p < npix;
-    int b = 0, y = 0, x = 0;
-    if (inside) {
-        b = p / (g.H * g.W);
-        const int rem = p % (g.H * g.W);
-        y = rem / g.W;
-        x = rem % g.W;
-    }
+                                           uint8_t* sA) {
+    const uint32_t m = tap_mask(g, p);
+    if constexpr (CIN == 16) {
+        uint4 v[9][2];
 #pragma unroll
-    for (int tap = 0; tap < 9; ++tap) {
-        const int yy = y + tap / 3 - 1, xx = x + tap % 3 - 1;
-        const bool ok = inside && yy >= 0 && yy < g.H && xx >= 0 && xx < g.W;
-        const size_t at = ok ? ((size_t)(b * g.H + yy) * g.W + xx) * g.cin : 0;
-        if (g.cin == 4) {
-            const uint2 v = ok ? __ldg(reinterpret_cast<const uint2*>(X + at)) : make_uint2(0u, 0u);
-            *reinterpret_cast<uint2*>(sA + tc::core_off(row, tap * 4, kb)) = v;
-        } else {
-            for (int cb = 0; cb < g.cin / 8; ++cb) {
-                const uint4 v = ok ? __ldg(reinterpret_cast<const uint4*>(X + at) + cb) : make_uint4(0u, 0u, 0u, 0u);
-                *reinterpret_cast<uint4*>(sA + tc::core_off(row, tap * g.cin + cb * 8, kb)) = v;
-            }
+        for (int tap = 0; tap < 9; ++tap) {
+            const uint4* src = reinterpret_cast<const uint4*>(X + ((int64_t)p + tap_shift(tap, g.W)) * 16);
+            const bool ok = (m >> tap) & 1u;
+            v[tap][0] = ok ? __ldg(src) : make_uint4(0u, 0u, 0u, 0u);
+            v[tap][1] = ok ? __ldg(src + 1) : make_uint4(0u, 0u, 0u, 0u);
         }
+#pragma unroll
+        for (int tap = 0; tap < 9; ++tap)
+#pragma unroll
+            for (int cb = 0; cb < 2; ++cb)
+                *reinterpret_cast<uint4*>(sA + tc::core_off(row, tap * 16 + cb * 8, 18)) = v[tap][cb];
+    } else {
+        uint2 v[12];
+#pragma unroll
+        for (int tap = 0; tap < 12; ++tap) {
+            const bool ok = tap < 9 && ((m >> tap) & 1u);
+            v[tap] = ok ? __ldg(reinterpret_cast<const uint2*>(X + ((int64_t)p + tap_shift(tap, g.W)) * 4))
+                        : make_uint2(0u, 0u);
+        }
+#pragma unroll
+        for (int tap = 0; tap < 12; ++tap)
+            *reinterpret_cast<uint2*>(sA + tc::core_off(row, tap * 4, 6)) = v[tap];
     }
-    for (int k = 9 * g.cin; k < kpad; ++k) put_bf16(sA, tc::core_off(row, k, kb), __float2bfloat16(0.f));
 }
 
 // Shared TMEM/mbarrier bookkeeping of one CTA (128 threads).
@@ -146,12 +139,14 @@ __device__ __forceinline__ void tc_begin(TcCta& s, uint32_t ncols) {
 
 // Wait for the committed MMAs (bounded); on timeout flag the error and wait
 // once more (bounded) so that TMEM is not freed under a running MMA.
-__device__ __forceinline__ void tc_wait(TcCta& s, int* err) {
-    if (!tc::mbar_wait_bounded(&s.bar, 0, kWaitLimit)) {
+__device__ __forceinline__ bool tc_wait(TcCta& s, uint32_t phase, int* err) {
+    const bool ok = tc::mbar_wait_bounded(&s.bar, phase, kWaitLimit);
+    if (!ok) {
         if (threadIdx.x == 0) atomicOr(err, 1);
-        tc::mbar_wait_bounded(&s.bar, 0, kWaitLimit);
+        tc::mbar_wait_bounded(&s.bar, phase, kWaitLimit);
     }
     tc::fence_after_sync();
+    return ok;
 }
 
 __device__ __forceinline__ void tc_end(TcCta& s, uint32_t ncols) {
@@ -164,22 +159,59 @@ __device__ __forceinline__ void tc_end(TcCta& s, uint32_t ncols) {
 }
 
 // ---------------------------------------------------------------------------
-// Forward convolution: 128 pixels per CTA.
+// One convolution, 128 pixels per CTA, its epilogue in registers (thread t
+// holds pixel t's 16 outputs).
+//   kActivate  A = relu(Z + b), bf16
+//   kLogits    Z + b, float (16 a pixel, zero from cout on)
+//   kLoss      softmax cross-entropy of the logits: the summed loss and
+//              dZ = (softmax - onehot) / npix, bf16
+//   kInputGrad dZ of the layer below: the outputs where its activation is
+//              positive (relu'), else 0, bf16
 // ---------------------------------------------------------------------------
-__global__ void __launch_bounds__(128) k_conv_fwd(const bf16* __restrict__ X, Img g,
-                                                  const bf16* __restrict__ wf, int kpad,
-                                                  const float* __restrict__ bias, int cout,
-                                                  float* __restrict__ Z, bf16* __restrict__ A, int relu,
-                                                  int* err) {
+enum ConvOut { kActivate, kLogits, kLoss, kInputGrad };
+struct ConvArgs {
+    const bf16* X;                  // [npix][CIN]
+    Img g;
+    const bf16* w;                  // packed B tile, 16 x kpad
+    const float* bias;              // (not kInputGrad)
+    int cout;
+    bf16* A;                        // bf16 output [npix][16]
+    float* Z;                       // kLogits: output [npix][16]
+    const uint8_t* labels;          // kLoss
+    float inv_npix;
+    double* loss;
+    const bf16* act;                // kInputGrad: the layer below's activations [npix][16]
+    int* err;
+};
+
+__device__ __forceinline__ uint32_t pack2(float a, float b) {
+    const __nv_bfloat162 v = __floats2bfloat162_rn(a, b);
+    return *reinterpret_cast<const uint32_t*>(&v);
+}
+__device__ __forceinline__ void store_bf16x16(bf16* dst, const float (&v)[16]) {
+    uint4* d = reinterpret_cast<uint4*>(dst);
+    d[0] = make_uint4(pack2(v[0], v[1]), pack2(v[2], v[3]), pack2(v[4], v[5]), pack2(v[6], v[7]));
+    d[1] = make_uint4(pack2(v[8], v[9]), pack2(v[10], v[11]), pack2(v[12], v[13]), pack2(v[14], v[15]));
+}
+
+// Bound by the latency of its three parts (im2col gather, one MMA chain,
+// epilogue), not by bytes or the tensor cores: 18-20 us for 131,072 pixels
+// (8 images of 128 x 128) with 16 channels in.  What a pixel needs moves as
+// 128-bit accesses (41 us with element-wise stores), and the input gradient is
+// the same convolution with relu' in its epilogue (96 us for its columns, 43 to
+// add them up and 12 for relu' as kernels of their own).
+template <int CIN, int OUT>
+__global__ void __launch_bounds__(128) k_conv(ConvArgs a) {
+    constexpr int kpad = CIN == 16 ? 144 : 48, kb = kpad / 8;
     extern __shared__ __align__(1024) uint8_t smem[];
     __shared__ TcCta s;
     uint8_t* sA = smem;                        // 128 x kpad
     uint8_t* sB = smem + 256 * kpad;           // 16 x kpad
-    const int kb = kpad / 8;
     const int t = threadIdx.x;
     const int p = blockIdx.x * 128 + t;
-    im2col_row(X, g, p, (uint32_t)t, sA, kpad);
-    const uint4* src = reinterpret_cast<const uint4*>(wf);
+    const int npix = a.g.B * a.g.H * a.g.W;
+    im2col_row<CIN>(a.X, a.g, p, (uint32_t)t, sA);
+    const uint4* src = reinterpret_cast<const uint4*>(a.w);
     for (int i = t; i < 2 * kpad; i += 128) reinterpret_cast<uint4*>(sB)[i] = src[i];
     tc_begin(s, 32);
     if (t == 0) {
@@ -189,195 +221,206 @@ __global__ void __launch_bounds__(128) k_conv_fwd(const bf16* __restrict__ X, Im
                          tc::idesc_bf16(128, 16), kk > 0);
         tc::mma_commit(&s.bar);
     }
-    tc_wait(s, err);
+    tc_wait(s, 0, a.err);
     float v[16];
     tc::tmem_ld16(s.tmem + ((uint32_t)(32 * (t >> 5)) << 16), v);
-    const int npix = g.B * g.H * g.W;
-    if (p < npix) {
+    if constexpr (OUT == kInputGrad) {
+        if (p < npix) {
+            const uint4* m = reinterpret_cast<const uint4*>(a.act + (size_t)p * 16);
+            const uint4 m0 = __ldg(m), m1 = __ldg(m + 1);
+            const uint32_t w[8] = {m0.x, m0.y, m0.z, m0.w, m1.x, m1.y, m1.z, m1.w};
 #pragma unroll
-        for (int o = 0; o < 16; ++o) {
-            const float z = o < cout ? v[o] + bias[o] : 0.f;
-            Z[(size_t)p * 16 + o] = z;
-            if (A) A[(size_t)p * 16 + o] = __float2bfloat16(relu ? fmaxf(z, 0.f) : z);
+            for (int o = 0; o < 16; ++o) {
+                // activations are never negative: positive = not 0
+                const uint32_t h = (o & 1) ? w[o / 2] >> 16 : w[o / 2] & 0xFFFFu;
+                if ((h & 0x7FFFu) == 0u) v[o] = 0.f;
+            }
+            store_bf16x16(a.A + (size_t)p * 16, v);
         }
-    }
-    tc_end(s, 32);
-}
-
-// ---------------------------------------------------------------------------
-// Input gradient: dXcol = dZ W (K = 16 output channels) into dcol [pix][kpad];
-// k_col2im then sums each input cell's nine taps in a fixed order (no float
-// atomics: the same gradients on every run).
-// ---------------------------------------------------------------------------
-__global__ void __launch_bounds__(128) k_conv_bwd_data(const bf16* __restrict__ dZ, Img g,
-                                                       const bf16* __restrict__ wt, int kpad,
-                                                       float* __restrict__ dcol, int* err) {
-    extern __shared__ __align__(1024) uint8_t smem[];
-    __shared__ TcCta s;
-    uint8_t* sA = smem;                        // 128 x 16
-    uint8_t* sB = smem + 4096;                 // kpad x 16
-    const int t = threadIdx.x;
-    const int p = blockIdx.x * 128 + t;
-    const int npix = g.B * g.H * g.W;
-    for (int o = 0; o < 16; ++o)
-        put_bf16(sA, tc::core_off(t, o, 2), p < npix ? dZ[(size_t)p * 16 + o] : __float2bfloat16(0.f));
-    const uint4* src = reinterpret_cast<const uint4*>(wt);
-    for (int i = t; i < 2 * kpad; i += 128) reinterpret_cast<uint4*>(sB)[i] = src[i];
-    const uint32_t ncols = tmem_cols_for(kpad);
-    tc_begin(s, ncols);
-    if (t == 0) {
-        tc::mma_bf16(s.tmem, tc::sdesc(tc::smem_addr(sA), 128, 256), tc::sdesc(tc::smem_addr(sB), 128, 256),
-                     tc::idesc_bf16(128, kpad), 0);
-        tc::mma_commit(&s.bar);
-    }
-    tc_wait(s, err);
-    for (int c0 = 0; c0 < kpad; c0 += 16) {
-        float v[16];
-        tc::tmem_ld16(s.tmem + ((uint32_t)(32 * (t >> 5)) << 16) + c0, v);
+    } else {
         if (p < npix) {
 #pragma unroll
-            for (int j = 0; j < 16; ++j) dcol[(size_t)p * kpad + c0 + j] = v[j];
+            for (int o = 0; o < 16; ++o) v[o] = o < a.cout ? v[o] + __ldg(a.bias + o) : 0.f;
+        }
+        if constexpr (OUT == kActivate) {
+            if (p < npix) {
+#pragma unroll
+                for (int o = 0; o < 16; ++o) v[o] = fmaxf(v[o], 0.f);
+                store_bf16x16(a.A + (size_t)p * 16, v);
+            }
+        } else if constexpr (OUT == kLogits) {
+            if (p < npix) {
+                float4* z = reinterpret_cast<float4*>(a.Z + (size_t)p * 16);
+#pragma unroll
+                for (int j = 0; j < 4; ++j) z[j] = make_float4(v[4 * j], v[4 * j + 1], v[4 * j + 2], v[4 * j + 3]);
+            }
+        } else {
+            double l = 0.0;
+            if (p < npix) {
+                float m = -INFINITY, se = 0.f;
+#pragma unroll
+                for (int o = 0; o < kSkipCls; ++o) m = fmaxf(m, v[o]);
+                float e[kSkipCls];
+#pragma unroll
+                for (int o = 0; o < kSkipCls; ++o) {
+                    e[o] = expf(v[o] - m);
+                    se += e[o];
+                }
+                const int y = a.labels[p];
+                float zy = v[0], d[16];
+#pragma unroll
+                for (int o = 0; o < 16; ++o) {
+                    d[o] = o < kSkipCls ? (e[o < kSkipCls ? o : 0] / se - (o == y ? 1.f : 0.f)) * a.inv_npix : 0.f;
+                    if (o < kSkipCls && o == y) zy = v[o];
+                }
+                store_bf16x16(a.A + (size_t)p * 16, d);
+                l = (double)(logf(se) + m - zy);
+            }
+            for (int off = 16; off; off >>= 1) l += __shfl_xor_sync(0xffffffffu, l, off);
+            if ((t & 31) == 0) atomicAdd(a.loss, l);
         }
     }
-    tc_end(s, ncols);
-}
-
-// dX[b][y][x][c] = sum over the taps (0..8, in order) of the column entry of
-// the output cell that the tap maps onto (b, y, x): the transpose of the
-// forward's im2col.
-__global__ void k_col2im(const float* __restrict__ dcol, Img g, int kpad, float* __restrict__ dX) {
-    const int64_t n = (int64_t)g.B * g.H * g.W * g.cin;
-    for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
-        const int c = (int)(i % g.cin);
-        const int64_t q = i / g.cin;
-        const int x = (int)(q % g.W), y = (int)((q / g.W) % g.H), b = (int)(q / ((int64_t)g.W * g.H));
-        float acc = 0.f;
-        for (int tap = 0; tap < 9; ++tap) {
-            const int ys = y - (tap / 3 - 1), xs = x - (tap % 3 - 1);     // the output cell of this tap
-            if (ys < 0 || ys >= g.H || xs < 0 || xs >= g.W) continue;
-            acc += dcol[((size_t)(b * g.H + ys) * g.W + xs) * kpad + tap * g.cin + c];
-        }
-        dX[i] = acc;
-    }
-}
-
-// ---------------------------------------------------------------------------
-// Weight gradient of 128 pixels: D[k][o] = sum_p Xcol[p][k] dZ[p][o] and
-// sum_p dZ[p][o], this block's part (part + blockIdx.x * (16 kpad + 16):
-// [o][k] then [o]); k_sum_parts adds the blocks' parts in block order.
-// ---------------------------------------------------------------------------
-__global__ void __launch_bounds__(128) k_conv_bwd_weight(const bf16* __restrict__ X, Img g,
-                                                         const bf16* __restrict__ dZ, int kpad, int cout,
-                                                         float* __restrict__ part, int* err) {
-    extern __shared__ __align__(1024) uint8_t smem[];
-    __shared__ TcCta s;
-    const int mt = (kpad + 127) / 128;         // 128-row tiles of k
-    uint8_t* sA = smem;                        // mt*128 x 128 (rows k, K = pixels)
-    uint8_t* sB = smem + mt * 32768;           // 16 x 128 (rows o)
-    const int t = threadIdx.x;
-    const int p = blockIdx.x * 128 + t;
-    const int npix = g.B * g.H * g.W;
-    for (int k = 0; k < mt * 128; ++k) put_bf16(sA, tc::core_off(k, t, 16), xcol(X, g, p, k));
-    float dzv[16];
-#pragma unroll
-    for (int o = 0; o < 16; ++o) {
-        const bf16 d = p < npix ? dZ[(size_t)p * 16 + o] : __float2bfloat16(0.f);
-        dzv[o] = __bfloat162float(d);
-        put_bf16(sB, tc::core_off(o, t, 16), d);
-    }
-    tc_begin(s, 32);
-    if (t == 0) {
-        const uint32_t a0 = tc::smem_addr(sA), b0 = tc::smem_addr(sB);
-        for (int m = 0; m < mt; ++m)
-            for (int kk = 0; kk < 8; ++kk)
-                tc::mma_bf16(s.tmem + 16 * m, tc::sdesc(a0 + m * 32768 + kk * 256, 128, 2048),
-                             tc::sdesc(b0 + kk * 256, 128, 2048), tc::idesc_bf16(128, 16), kk > 0);
-        tc::mma_commit(&s.bar);
-    }
-    tc_wait(s, err);
-    float* const pw = part + (size_t)blockIdx.x * (16 * kpad + 16);
-    for (int m = 0; m < mt; ++m) {
-        float v[16];
-        tc::tmem_ld16(s.tmem + ((uint32_t)(32 * (t >> 5)) << 16) + 16 * m, v);
-        const int k = m * 128 + t;
-        if (k < kpad) {
-#pragma unroll
-            for (int o = 0; o < 16; ++o) pw[(size_t)o * kpad + k] = (o < cout && k < 9 * g.cin) ? v[o] : 0.f;
-        }
-    }
-    // bias gradient: warp sums, then the four warps' sums in order
-    __shared__ float sdb[4][16];
-#pragma unroll
-    for (int o = 0; o < 16; ++o) {
-        float x = dzv[o];
-        for (int off = 16; off; off >>= 1) x += __shfl_xor_sync(0xffffffffu, x, off);
-        if ((t & 31) == 0) sdb[t >> 5][o] = x;
-    }
-    __syncthreads();
-    if (t < 16) pw[16 * kpad + t] = t < cout ? ((sdb[0][t] + sdb[1][t]) + sdb[2][t]) + sdb[3][t] : 0.f;
     tc_end(s, 32);
 }
 
-// dW[o][k] and db[o]: the nb blocks' parts added in a fixed order, one warp
-// per entry (lane l adds blocks l, l + 32, ... in turn, then a fixed
-// shuffle tree adds the lanes' sums).
-__global__ void k_sum_parts(const float* __restrict__ part, int nb, int kpad, float* __restrict__ dW,
-                            float* __restrict__ db) {
-    const int per = 16 * kpad + 16;
-    const int lane = threadIdx.x & 31;
-    const int nw = (gridDim.x * blockDim.x) >> 5;
-    for (int e = (blockIdx.x * blockDim.x + threadIdx.x) >> 5; e < per; e += nw) {
-        float acc = 0.f;
-        for (int b = lane; b < nb; b += 32) acc += part[(size_t)b * per + e];
-        for (int off = 16; off; off >>= 1) acc += __shfl_down_sync(0xffffffffu, acc, off);
-        if (lane == 0) {
-            if (e < 16 * kpad) dW[e] = acc;
-            else db[e - 16 * kpad] = acc;
-        }
-    }
+// ---------------------------------------------------------------------------
+// Weight gradient: D[k][o] = sum_p Xcol[p][k] dZ[p][o], and with a row of ones
+// under the kpad rows of k the bias gradient sum_p dZ[p][o].  A CTA takes
+// 128-pixel chunks b, b + grid, ... and adds them up in TMEM; its part goes to
+// part + blockIdx.x * (16 kpad + 16) ([o][k], then [o]), and k_sum_grads adds
+// the parts in block order (no float atomics: the same gradients on every
+// run).
+//
+// Both operands have the pixels along K, while the images have the channels
+// contiguous: a warp gathers 8 pixels x 8 channels (4 bytes a lane) and stores
+// them transposed with stmatrix, four core matrices (512 contiguous bytes) at
+// a time: 20 us for 131,072 pixels with 16 channels; 205 us element by
+// element, with two divisions each.
+// ---------------------------------------------------------------------------
+__device__ __forceinline__ void stmatrix_x4_trans(uint32_t addr, const uint32_t (&r)[4]) {
+    asm volatile("stmatrix.sync.aligned.m8n8.x4.trans.shared.b16 [%0], {%1, %2, %3, %4};" ::"r"(addr), "r"(r[0]),
+                 "r"(r[1]), "r"(r[2]), "r"(r[3])
+                 : "memory");
 }
 
-// softmax cross-entropy over the 5 classes of every pixel
-__global__ void k_xent(const float* __restrict__ Z3, const uint8_t* __restrict__ labels, int npix,
-                       float inv_npix, bf16* __restrict__ dZ3, double* loss) {
-    const int p = blockIdx.x * blockDim.x + threadIdx.x;
-    double l = 0.0;
-    if (p < npix) {
-        float z[kSkipCls], m = -INFINITY;
-        for (int o = 0; o < kSkipCls; ++o) {
-            z[o] = Z3[(size_t)p * 16 + o];
-            m = fmaxf(m, z[o]);
+template <int CIN>
+__global__ void __launch_bounds__(256) k_conv_bwd_weight(const bf16* __restrict__ X, Img g,
+                                                         const bf16* __restrict__ dZ, int cout,
+                                                         float* __restrict__ part, int* err) {
+    constexpr int kpad = CIN == 16 ? 144 : 48, kb = kpad / 8;
+    constexpr int mt = (kpad + 16 + 127) / 128;        // 128-row tiles of k and the row of ones
+    extern __shared__ __align__(1024) uint8_t smem[];
+    __shared__ TcCta s;
+    __shared__ uint16_t taps[128];
+    uint8_t* sA = smem;                        // mt*128 x 128 (rows k, K = pixels)
+    uint8_t* sB = smem + mt * 32768;           // 16 x 128 (rows o)
+    const int t = threadIdx.x, lane = t & 31, warp = t >> 5;
+    const int npix = g.B * g.H * g.W, nchunk = (npix + 127) / 128;
+    tc_begin(s, 32);
+    const uint32_t a0 = tc::smem_addr(sA), b0 = tc::smem_addr(sB);
+    // rows of k past the ones' core row are never written: their D rows are
+    // not read
+    uint32_t phase = 0;
+    bool ok = true;
+    for (int ch = blockIdx.x; ch < nchunk && ok; ch += gridDim.x) {
+        const int base = ch * 128;
+        if (t < 128) taps[t] = (uint16_t)tap_mask(g, base + t);
+        __syncthreads();
+        // core row blocks: kb of X, one of ones, two of dZ; each is 16 pixel
+        // groups, four per store
+        for (int q = warp; q < 4 * (kb + 3); q += 8) {
+            const int r = q >> 2, pg = (q & 3) * 4;
+            const uint32_t c2 = 2u * (lane & 3);          // the lane's channel pair in the block
+            uint32_t v[4];
+            if (r < kb) {
+                const int k = r * 8 + c2, tap = k / CIN, c = k % CIN;
+                const int64_t sh = tap_shift(tap, g.W);
+#pragma unroll
+                for (int m = 0; m < 4; ++m) {
+                    const int i = (pg + m) * 8 + (lane >> 2);
+                    const bool in = tap < 9 && ((taps[i] >> tap) & 1u);
+                    v[m] = in ? __ldg(reinterpret_cast<const uint32_t*>(X + (base + i + sh) * CIN + c)) : 0u;
+                }
+            } else if (r == kb) {
+#pragma unroll
+                for (int m = 0; m < 4; ++m) v[m] = c2 == 0u ? 0x3F80u : 0u;      // (dZ is 0 past the last pixel)
+            } else {
+#pragma unroll
+                for (int m = 0; m < 4; ++m) {
+                    const int i = base + (pg + m) * 8 + (lane >> 2);
+                    v[m] = i < npix ? __ldg(reinterpret_cast<const uint32_t*>(dZ + (int64_t)i * 16 + (r - kb - 1) * 8 + c2))
+                                    : 0u;
+                }
+            }
+            const uint32_t blk = r <= kb ? a0 + r * 2048 : b0 + (r - kb - 1) * 2048;
+            stmatrix_x4_trans(blk + (pg + (lane >> 3)) * 128 + (lane & 7) * 16, v);
         }
-        float se = 0.f;
-        for (int o = 0; o < kSkipCls; ++o) se += expf(z[o] - m);
-        const int y = labels[p];
-        for (int o = 0; o < 16; ++o) {
-            float d = 0.f;
-            if (o < kSkipCls) d = (expf(z[o] - m) / se - (o == y ? 1.f : 0.f)) * inv_npix;
-            dZ3[(size_t)p * 16 + o] = __float2bfloat16(d);
+        tc::fence_async_smem();
+        tc::fence_before_sync();
+        __syncthreads();
+        if (t == 0) {
+            tc::fence_after_sync();
+            for (int m = 0; m < mt; ++m)
+                for (int kk = 0; kk < 8; ++kk)
+                    tc::mma_bf16(s.tmem + 16 * m, tc::sdesc(a0 + m * 32768 + kk * 256, 128, 2048),
+                                 tc::sdesc(b0 + kk * 256, 128, 2048), tc::idesc_bf16(128, 16),
+                                 (kk > 0 || ch != (int)blockIdx.x) ? 1u : 0u);
+            tc::mma_commit(&s.bar);
         }
-        l = (double)(logf(se) + m - z[y < kSkipCls ? y : 0]);
+        ok = tc_wait(s, phase, err);            // the operands are read: the next chunk may replace them
+        phase ^= 1u;
+        ok = __syncthreads_and(ok ? 1 : 0) != 0;
     }
-    for (int off = 16; off; off >>= 1) l += __shfl_xor_sync(0xffffffffu, l, off);
-    if ((threadIdx.x & 31) == 0) atomicAdd(loss, l);
+    float* const pw = part + (size_t)blockIdx.x * (16 * kpad + 16);
+    if (warp < 4) {
+        for (int m = 0; m < mt; ++m) {
+            float v[16];
+            tc::tmem_ld16(s.tmem + ((uint32_t)(32 * warp) << 16) + 16 * m, v);
+            const int k = m * 128 + t;
+            if (k < kpad) {
+#pragma unroll
+                for (int o = 0; o < 16; ++o) pw[(size_t)o * kpad + k] = v[o];
+            } else if (k == kpad) {
+#pragma unroll
+                for (int o = 0; o < 16; ++o) pw[16 * kpad + o] = v[o];
+            }
+        }
+    }
+    tc_end(s, 32);
 }
 
-// dZ = dA * (Z > 0), to bf16
-__global__ void k_relu_bwd(const float* __restrict__ dA, const float* __restrict__ Z, int64_t n,
-                           bf16* __restrict__ dZ) {
-    for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x)
-        dZ[i] = __float2bfloat16(Z[i] > 0.f ? dA[i] : 0.f);
-}
-
-// dW [cout][kpad] (k = tap*cin + c) + db -> the flat FP32 gradient layout
-__global__ void k_unpack_grads(const float* __restrict__ dWl, const float* __restrict__ dbl, int layer,
-                               float* __restrict__ grads) {
-    const Layer ly = c_layers[layer];
-    for (int idx = threadIdx.x; idx < ly.cout * ly.cin * 9; idx += blockDim.x) {
-        const int o = idx / (ly.cin * 9), r = idx % (ly.cin * 9), c = r / 9, tap = r % 9;
-        grads[ly.offw + idx] = dWl[(size_t)o * ly.kpad + tap * ly.cin + c];
+// The flat FP32 gradients of the three layers: the nb blocks' parts of every
+// entry added in a fixed order (warp w of 32 adds parts w, w + 32, ..., the
+// warps' sums follow in order), 32 entries per CTA so that the parts are read
+// in full lines.  Entries of layer l: o * kpad + k, then 16 kpad + o.
+struct GradParts {
+    const float* part[3];
+    int nb[3];
+};
+__global__ void __launch_bounds__(1024) k_sum_grads(GradParts a, float* __restrict__ grads) {
+    const Layer ly = c_layers[blockIdx.y];
+    const int per = 16 * ly.kpad + 16, lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int e = blockIdx.x * 32 + lane;
+    __shared__ float sum[32][32];
+    float acc = 0.f;
+    if (e < per) {
+        const int l = blockIdx.y, nb = l == 0 ? a.nb[0] : (l == 1 ? a.nb[1] : a.nb[2]);
+        const float* src = (l == 0 ? a.part[0] : (l == 1 ? a.part[1] : a.part[2])) + e;
+#pragma unroll 4
+        for (int b = warp; b < nb; b += 32) acc += __ldg(src + (size_t)b * per);
     }
-    for (int o = threadIdx.x; o < ly.cout; o += blockDim.x) grads[ly.offb + o] = dbl[o];
+    sum[warp][lane] = acc;
+    __syncthreads();
+    if (warp != 0 || e >= per) return;
+    acc = sum[0][lane];
+#pragma unroll
+    for (int w = 1; w < 32; ++w) acc += sum[w][lane];
+    if (e < 16 * ly.kpad) {
+        const int o = e / ly.kpad, k = e % ly.kpad, tap = k / ly.cin, c = k % ly.cin;
+        if (o < ly.cout && tap < 9) grads[ly.offw + (o * ly.cin + c) * 9 + tap] = acc;
+    } else if (e - 16 * ly.kpad < ly.cout) {
+        grads[ly.offb + e - 16 * ly.kpad] = acc;
+    }
 }
 
 __global__ void k_adam(float* __restrict__ w, const float* __restrict__ g, float* __restrict__ m,
@@ -398,20 +441,17 @@ bool dalloc(P** p, size_t bytes) {
     return true;
 }
 
-size_t smem_fwd(int kpad) { return 288u * kpad; }
-size_t smem_bwd_data(int kpad) { return 4096u + 32u * kpad; }
-size_t smem_bwd_weight(int kpad) { return ((kpad + 127) / 128) * 32768u + 4096u; }
+size_t smem_conv(int kpad) { return 288u * kpad; }
+size_t smem_bwd_weight(int kpad) { return ((kpad + 16 + 127) / 128) * 32768u + 4096u; }
 
 }  // namespace
 
 struct SkipNet {
     float *params = nullptr, *grads = nullptr, *m = nullptr, *v = nullptr;
-    bf16 *wf = nullptr, *wt = nullptr;      // 3 layers x (16 x 144) and (144 x 16)
-    float *dW = nullptr, *db = nullptr;     // per-layer weight/bias gradient scratch [16][144], [16]
-    // training scratch of the fixed-order reductions: the input gradient's
-    // columns [pix][144] and the weight gradient's per-block parts
-    float *dcol = nullptr, *part = nullptr;
-    int64_t dcol_cap = 0, part_cap = 0;
+    bf16 *wf = nullptr, *wt = nullptr;      // 3 layers x (16 x 144): forward, input gradient
+    // the weight gradients' per-block parts, one array per layer
+    float* part = nullptr;
+    int part_blocks = 0;                    // most blocks of one layer
     int* err = nullptr;
     double* loss = nullptr;
     int64_t adam_t = 0;
@@ -425,15 +465,14 @@ static void pack(SkipNet* n, cudaStream_t st) {
 SkipNet* skipnet_create(uint32_t seed) {
     static bool attrs = false;
     if (!attrs) {
-        cudaFuncSetAttribute(k_conv_bwd_weight, cudaFuncAttributeMaxDynamicSharedMemorySize,
+        cudaFuncSetAttribute(k_conv_bwd_weight<16>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                              (int)smem_bwd_weight(144));
         attrs = true;
     }
     SkipNet* n = new SkipNet;
     bool ok = dalloc(&n->params, sizeof(float) * kSkipParams) && dalloc(&n->grads, sizeof(float) * kSkipParams) &&
               dalloc(&n->m, sizeof(float) * kSkipParams) && dalloc(&n->v, sizeof(float) * kSkipParams) &&
-              dalloc(&n->wf, sizeof(bf16) * 3 * 16 * 144) && dalloc(&n->wt, sizeof(bf16) * 3 * 144 * 16) &&
-              dalloc(&n->dW, sizeof(float) * 16 * 144) && dalloc(&n->db, sizeof(float) * 16) &&
+              dalloc(&n->wf, sizeof(bf16) * 3 * 16 * 144) && dalloc(&n->wt, sizeof(bf16) * 3 * 16 * 144) &&
               dalloc(&n->err, sizeof(int)) && dalloc(&n->loss, sizeof(double));
     if (!ok) {
         skipnet_destroy(n);
@@ -465,7 +504,7 @@ SkipNet* skipnet_create(uint32_t seed) {
 void skipnet_destroy(SkipNet* n) {
     if (!n) return;
     for (void* p : {(void*)n->params, (void*)n->grads, (void*)n->m, (void*)n->v, (void*)n->wf, (void*)n->wt,
-                    (void*)n->dW, (void*)n->db, (void*)n->err, (void*)n->loss, (void*)n->dcol, (void*)n->part})
+                    (void*)n->err, (void*)n->loss, (void*)n->part})
         if (p) cudaFree(p);
     skipwork_free(&n->work);
     delete n;
@@ -489,9 +528,8 @@ bool skipwork_reserve(SkipWork* w, int64_t npix) {
     if (w->cap >= npix) return true;
     skipwork_free(w);
     const size_t nf = sizeof(float) * 16 * npix, nb = sizeof(bf16) * 16 * npix;
-    bool ok = dalloc(&w->A1, nb) && dalloc(&w->A2, nb) && dalloc(&w->Z1, nf) && dalloc(&w->Z2, nf) &&
-              dalloc(&w->Z3, nf) && dalloc(&w->dZ1, nb) && dalloc(&w->dZ2, nb) && dalloc(&w->dZ3, nb) &&
-              dalloc(&w->dA1, nf) && dalloc(&w->dA2, nf);
+    bool ok = dalloc(&w->A1, nb) && dalloc(&w->A2, nb) && dalloc(&w->Z3, nf) && dalloc(&w->dZ1, nb) &&
+              dalloc(&w->dZ2, nb) && dalloc(&w->dZ3, nb);
     if (!ok) {
         skipwork_free(w);
         return false;
@@ -501,25 +539,44 @@ bool skipwork_reserve(SkipWork* w, int64_t npix) {
 }
 
 void skipwork_free(SkipWork* w) {
-    for (void* p : {(void*)w->A1, (void*)w->A2, (void*)w->Z1, (void*)w->Z2, (void*)w->Z3, (void*)w->dZ1,
-                    (void*)w->dZ2, (void*)w->dZ3, (void*)w->dA1, (void*)w->dA2})
+    for (void* p : {(void*)w->A1, (void*)w->A2, (void*)w->Z3, (void*)w->dZ1, (void*)w->dZ2, (void*)w->dZ3})
         if (p) cudaFree(p);
     *w = SkipWork();
+}
+
+// the two hidden layers: activations A1, A2
+static ConvArgs hidden_layers(const SkipNet* n, const bf16* x, int nimg, int H, int W, SkipWork* w, cudaStream_t st) {
+    const int nb = (nimg * H * W + 127) / 128;
+    ConvArgs a = {};
+    a.X = x;
+    a.g = Img{nimg, H, W, 4};
+    a.w = n->wf;
+    a.bias = n->params + kLayers[0].offb;
+    a.cout = 16;
+    a.A = w->A1;
+    a.err = n->err;
+    k_conv<4, kActivate><<<nb, 128, smem_conv(48), st>>>(a);
+    a.X = w->A1;
+    a.g.cin = 16;
+    a.w = n->wf + 16 * 144;
+    a.bias = n->params + kLayers[1].offb;
+    a.A = w->A2;
+    k_conv<16, kActivate><<<nb, 128, smem_conv(144), st>>>(a);
+    a.X = w->A2;
+    a.w = n->wf + 2 * 16 * 144;
+    a.bias = n->params + kLayers[2].offb;
+    a.cout = kLayers[2].cout;
+    return a;                                // the last layer's, its output left to the caller
 }
 
 cudaError_t skipnet_forward(const SkipNet* n, const bf16* x, int nimg, int H, int W, SkipWork* w,
                             cudaStream_t st) {
     const int npix = nimg * H * W;
     if (w->cap < npix) return cudaErrorInvalidValue;
-    const int nb = (npix + 127) / 128;
-    Img g{nimg, H, W, 4};
-    k_conv_fwd<<<nb, 128, smem_fwd(48), st>>>(x, g, n->wf, 48, n->params + kLayers[0].offb, 16, w->Z1, w->A1, 1,
-                                              n->err);
-    g.cin = 16;
-    k_conv_fwd<<<nb, 128, smem_fwd(144), st>>>(w->A1, g, n->wf + 16 * 144, 144, n->params + kLayers[1].offb, 16,
-                                               w->Z2, w->A2, 1, n->err);
-    k_conv_fwd<<<nb, 128, smem_fwd(144), st>>>(w->A2, g, n->wf + 2 * 16 * 144, 144, n->params + kLayers[2].offb,
-                                               5, w->Z3, nullptr, 0, n->err);
+    ConvArgs a = hidden_layers(n, x, nimg, H, W, w, st);
+    a.A = nullptr;
+    a.Z = w->Z3;
+    k_conv<16, kLogits><<<(npix + 127) / 128, 128, smem_conv(144), st>>>(a);
     return cudaGetLastError();
 }
 
@@ -529,46 +586,52 @@ static cudaError_t skipnet_backprop(SkipNet* n, const bf16* x, const uint8_t* la
     SkipWork* w = &n->work;
     const int npix = nimg * H * W;
     if (!skipwork_reserve(w, npix)) return cudaErrorMemoryAllocation;
-    const int64_t nb_all = (npix + 127) / 128;
-    if (n->dcol_cap < npix) {
-        if (n->dcol) cudaFree(n->dcol);
-        n->dcol = nullptr;
-        n->dcol_cap = 0;
-        if (!dalloc(&n->dcol, sizeof(float) * 144 * (size_t)npix)) return cudaErrorMemoryAllocation;
-        n->dcol_cap = npix;
-    }
-    if (n->part_cap < nb_all) {
+    const int nb = (npix + 127) / 128;
+    // three CTAs of the widest weight gradient (70 KB of operands) per SM
+    int dev = 0, nsm = 0;
+    cudaGetDevice(&dev);
+    cudaDeviceGetAttribute(&nsm, cudaDevAttrMultiProcessorCount, dev);
+    const int nw = std::min(nb, 3 * nsm);
+    constexpr size_t per = 16 * 144 + 16;
+    if (n->part_blocks < nw) {
         if (n->part) cudaFree(n->part);
         n->part = nullptr;
-        n->part_cap = 0;
-        if (!dalloc(&n->part, sizeof(float) * (16 * 144 + 16) * (size_t)nb_all)) return cudaErrorMemoryAllocation;
-        n->part_cap = nb_all;
+        n->part_blocks = 0;
+        if (!dalloc(&n->part, sizeof(float) * 3 * per * nw)) return cudaErrorMemoryAllocation;
+        n->part_blocks = nw;
     }
-    cudaError_t e = skipnet_forward(n, x, nimg, H, W, w, st);
-    if (e != cudaSuccess) return e;
-    const int nb = (npix + 127) / 128;
     cudaMemsetAsync(n->loss, 0, sizeof(double), st);
-    k_xent<<<(npix + 255) / 256, 256, 0, st>>>(w->Z3, labels, npix, 1.f / npix, w->dZ3, n->loss);
+    ConvArgs a = hidden_layers(n, x, nimg, H, W, w, st);
+    a.A = w->dZ3;
+    a.labels = labels;
+    a.inv_npix = 1.f / npix;
+    a.loss = n->loss;
+    k_conv<16, kLoss><<<nb, 128, smem_conv(144), st>>>(a);
     const bf16* acts[3] = {x, w->A1, w->A2};
     bf16* dZ[3] = {w->dZ1, w->dZ2, w->dZ3};
-    float* dA[3] = {nullptr, w->dA1, w->dA2};
-    const float* Zs[3] = {w->Z1, w->Z2, nullptr};
+    GradParts gp;
     for (int l = 2; l >= 0; --l) {
         const Layer ly = kLayers[l];
-        Img g{nimg, H, W, ly.cin};
-        k_conv_bwd_weight<<<nb, 128, smem_bwd_weight(ly.kpad), st>>>(acts[l], g, dZ[l], ly.kpad, ly.cout, n->part,
-                                                                     n->err);
-        k_sum_parts<<<(16 * ly.kpad + 16 + 7) / 8, 256, 0, st>>>(n->part, nb, ly.kpad, n->dW, n->db);
-        k_unpack_grads<<<1, 256, 0, st>>>(n->dW, n->db, l, n->grads);
+        const Img g{nimg, H, W, ly.cin};
+        float* part = n->part + (size_t)l * per * n->part_blocks;
+        gp.part[l] = part;
+        gp.nb[l] = nw;
         if (l > 0) {
-            // gradient w.r.t. this layer's input = the previous layer's activation
-            k_conv_bwd_data<<<nb, 128, smem_bwd_data(ly.kpad), st>>>(dZ[l], g, n->wt + l * 144 * 16, ly.kpad,
-                                                                     n->dcol, n->err);
-            k_col2im<<<(int)std::min<int64_t>(((int64_t)npix * g.cin + 255) / 256, 4096), 256, 0, st>>>(
-                n->dcol, g, ly.kpad, dA[l]);
-            k_relu_bwd<<<(npix * 16 + 255) / 256, 256, 0, st>>>(dA[l], Zs[l - 1], (int64_t)npix * 16, dZ[l - 1]);
+            k_conv_bwd_weight<16><<<nw, 256, smem_bwd_weight(144), st>>>(acts[l], g, dZ[l], ly.cout, part, n->err);
+            // gradient w.r.t. this layer's input, through the layer below's relu
+            ConvArgs b = {};
+            b.X = dZ[l];
+            b.g = Img{nimg, H, W, 16};
+            b.w = n->wt + l * 16 * 144;
+            b.A = dZ[l - 1];
+            b.act = acts[l];
+            b.err = n->err;
+            k_conv<16, kInputGrad><<<nb, 128, smem_conv(144), st>>>(b);
+        } else {
+            k_conv_bwd_weight<4><<<nw, 256, smem_bwd_weight(48), st>>>(acts[l], g, dZ[l], ly.cout, part, n->err);
         }
     }
+    k_sum_grads<<<dim3((unsigned)((per + 31) / 32), 3), 1024, 0, st>>>(gp, n->grads);
     return cudaGetLastError();
 }
 

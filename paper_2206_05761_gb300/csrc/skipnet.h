@@ -21,9 +21,8 @@ struct SkipNet;                   // weights, gradients, optimiser state (device
 struct SkipWork {
     int64_t cap = 0;
     __nv_bfloat16 *A1 = nullptr, *A2 = nullptr;           // post-ReLU, [pix][16]
-    float *Z1 = nullptr, *Z2 = nullptr, *Z3 = nullptr;     // pre-activations, [pix][16]
-    __nv_bfloat16 *dZ1 = nullptr, *dZ2 = nullptr, *dZ3 = nullptr;
-    float *dA1 = nullptr, *dA2 = nullptr;
+    float* Z3 = nullptr;                                   // logits, [pix][16]
+    __nv_bfloat16 *dZ1 = nullptr, *dZ2 = nullptr, *dZ3 = nullptr;   // gradients of the pre-activations
 };
 
 SkipNet* skipnet_create(uint32_t seed);
