@@ -1054,7 +1054,7 @@ class EngineT final : public Engine {
         if (quiet_on_) {
             const SigSrc sg = sig_src(onfly && !learned);
             lk(k_trav_classify, (ntiles_ + 255) / 256, 256, sg, L_, kt_, ntiles_, st_, quiet(),
-                                                                      learned ? nullptr : scount_, work_);
+                                                                      learned ? nullptr : scount_, work_, dlist_, leaves_);
             mark("k_trav_classify");
             lk(k_trav_list, nsm_ * 8, 256, sg, dlist_, leaves_, L_, kt_, st_, work_);
             mark("k_trav_list");
@@ -1189,9 +1189,8 @@ class EngineT final : public Engine {
         return a;
     }
     void launch_decode(bool onfly = false) {
-        // the decode list is short once quiescent tiles are skipped: 2 CTAs per SM
-        const int gd = quiet_on_ ? std::min(grid_for((uint64_t)ntiles_ * 256), nsm_ * 4)
-                                 : grid_for((uint64_t)ntiles_ * 256);
+        // (CTAs without a listed tile leave at once)
+        const int gd = grid_for((uint64_t)ntiles_ * 256);
         lk(k_decode_finish<T>, grid_res(k_decode_finish<T>, gd, 256), 256, decode_args(onfly), fin_args());
         mark("k_decode_finish");
     }

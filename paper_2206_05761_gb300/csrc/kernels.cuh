@@ -889,7 +889,11 @@ __device__ __forceinline__ int group_level(const TileBits& tb, int L, int kt, ui
 }
 
 // Leaves of up to 16 finest cells (levels L-1, L-2) are decoded by the FV1
-// kernels themselves; larger ones by k_decode over the tiles listed here.
+// kernels themselves; larger ones by k_decode over the tiles listed here.  A
+// list entry is the tile (below 2^18 up to L = 14) and, above kWholeShift, 1 +
+// the level of the one leaf that covers it, or 0 (a tile with leaves of its
+// own, or not known: the decode reads its flags).
+constexpr int kWholeShift = 24;
 __device__ __forceinline__ bool needs_decode_kernel(int l, int L) { return l < L - 2; }
 
 // One warp per tile.  Lane t reads bit t of the root path (levels 0..Lr) and
@@ -1197,6 +1201,16 @@ __device__ __forceinline__ void trav_fused_body(const uint32_t* __restrict__ Sb,
             sum_all += tb.l0 == Lr ? 1u : __ldg(scount + tile);
             continue;
         }
+        if (tb.l0 <= Lr) {                       // one leaf covers the tile (uniform over the warp)
+            const bool head = (tile & ((1u << (2 * (Lr - tb.l0))) - 1u)) == 0u;
+            sum_all += head ? 1u : 0u;
+            if (lane == 0 && !skip) {
+                if (head) leaves[atomicAdd(&st->M, 1u)] = ((uint32_t)tb.l0 << kLeafShift) | (tile >> (2 * (Lr - tb.l0)));
+                if (needs_decode_kernel(tb.l0, L))
+                    dlist[atomicAdd(&st->ndec, 1u)] = tile | ((uint32_t)(tb.l0 + 1) << kWholeShift);
+            }
+            continue;
+        }
         int lv[kGroupsPerLane];
         const uint32_t c = lane_heads(tb, L, kt, tile, lv);
         const uint32_t total = warp_sum(c);
@@ -1245,15 +1259,31 @@ static __global__ void __launch_bounds__(256) k_trav_fused(const uint32_t* __res
     trav_fused_body(Sb, dlist, leaves, L, kt, ntiles, st, q, scount);
 }
 
+// Append n values (n 0 or 1 per active lane) to a list: one atomic per warp.
+__device__ __forceinline__ void append1(uint32_t* list, uint32_t* count, bool put, uint32_t v) {
+    const uint32_t act = __activemask(), m = __ballot_sync(act, put);
+    if (m == 0u) return;
+    const uint32_t lane = threadIdx.x & 31u, leader = __ffs(m) - 1u;
+    uint32_t base = 0u;
+    if (lane == leader) base = atomicAdd(count, (uint32_t)__popc(m));
+    base = __shfl_sync(act, base, leader);
+    if (put) list[base + __popc(m & ((1u << lane) - 1u))] = v;
+}
+
 // The traversal in two launches, for quiescent tiles: k_trav_classify
 // decides every tile with one thread (its root path and marks loaded at
-// once), counts a skipped tile from scount, and lists the others for
-// k_trav_list, which treats them one warp per tile as k_trav_fused does.
+// once), counts a skipped tile from scount, lists the leaf of a tile that one
+// leaf covers (and the tile for the decode) itself, and hands the tiles with
+// leaves of their own to k_trav_list, one CTA per tile.  Smooth water is
+// mostly covered tiles: at L=11 with three water columns (4,096 tiles, 1 in 5
+// refined) the listing went from 16.4 to 7.7 us.
 // A list entry with bit 31 set is a skipped tile that is only counted (no
 // scount: the learned look-ahead's flags).
 static __global__ void __launch_bounds__(256) k_trav_classify(SigSrc Sb, int L, int kt,
                                                               uint32_t ntiles, DevState* st, Quiet q,
-                                                              const uint32_t* scount, uint32_t* work) {
+                                                              const uint32_t* scount, uint32_t* work,
+                                                              uint32_t* __restrict__ dlist,
+                                                              uint32_t* __restrict__ leaves) {
     pdl_wait();
     if (!st->active) return;
     const int Lr = L - kt;
@@ -1275,19 +1305,15 @@ static __global__ void __launch_bounds__(256) k_trav_classify(SigSrc Sb, int L, 
         const bool skip = !covered && X[t] && yset && !q.inlet[t] && xw && xe && ysn && yn;
         q.act[t] = skip ? 0 : (covered ? kActCovered : kActOwn);
         if (!skip && !covered && yset) Y[t] = 0;          // the step writes into it
-        if (skip && scount) {
-            counted += l0 == Lr ? 1u : __ldg(scount + t);
-        } else {
-            // warp-aggregated append to the work list
-            const uint32_t m = __activemask();
-            const uint32_t lane = threadIdx.x & 31u, leader = __ffs(m) - 1u;
-            uint32_t base = 0;
-            if (lane == leader) base = atomicAdd(&st->nact, (uint32_t)__popc(m));
-            base = __shfl_sync(m, base, leader);
-            work[base + __popc(m & ((1u << lane) - 1u))] = t | (skip ? 0x80000000u : 0u);
-        }
+        const bool whole = l0 <= Lr && !skip;             // one leaf covers the tile
+        const bool head = whole && (t & ((1u << (2 * (Lr - (l0 < Lr ? l0 : Lr)))) - 1u)) == 0u;
+        if (skip && scount) counted += l0 == Lr ? 1u : __ldg(scount + t);
+        if (head) counted += 1u;
+        append1(leaves, &st->M, head, ((uint32_t)l0 << kLeafShift) | (t >> (2 * (Lr - (head ? l0 : Lr)))));
+        append1(dlist, &st->ndec, whole && needs_decode_kernel(l0, L), t | ((uint32_t)(l0 + 1) << kWholeShift));
+        append1(work, &st->nact, !whole && !(skip && scount), t | (skip ? 0x80000000u : 0u));
     }
-    // leaves of the skipped tiles: one atomic per block
+    // leaves of the skipped and the covered tiles: one atomic per block
     __shared__ uint32_t red[8];
     uint32_t v = warp_sum(counted);
     if ((threadIdx.x & 31u) == 0) red[threadIdx.x >> 5] = v;
@@ -2459,7 +2485,11 @@ struct DecodeArgs {
 
 // Decode-back of the leaves of more than 16 finest cells, over the tiles the
 // traversal listed (smaller leaves were decoded by the FV1 kernels): every
-// finest cell takes the leaf's discharges and free surface (R-decode).
+// finest cell takes the leaf's discharges and free surface (R-decode).  A tile
+// under one leaf brings the leaf's level with its list entry, so that it needs
+// no flags and one round of loads: three water columns on a flat bed at L=11
+// (134 MB) take 38 us, the last CTA's time advance included (48 us when every
+// tile's flags were formed first, by two thirds of the CTAs).
 template <typename T>
 __device__ __forceinline__ void decode_body(const DecodeArgs<T>& a, Blk B) {
     DevState* st = a.st;
@@ -2477,33 +2507,37 @@ __device__ __forceinline__ void decode_body(const DecodeArgs<T>& a, Blk B) {
     const uint32_t g = threadIdx.x;
     const bool act = g < (1u << (2 * (a.kt - 1)));
     for (uint32_t d = B.id; d < nd; d += B.n) {
-        const uint32_t tile = a.dlist[d];
-        __syncthreads();                            // tb reused across tiles
-        load_tile_bits(a.Sb, a.L, a.kt, tile, tb);
-        if (a.q.zf[0] != nullptr && a.q.act[tile] == kActCovered) {
-            // one coarser leaf covers the whole tile: when its new value is
-            // (+0, +0, +0) and the tile already holds +0, nothing changes
-            const int lc = group_level(tb, a.L, a.kt, 0);
-            const uint64_t sc = lvl_off(lc) + (((uint64_t)tile << (2 * a.kt)) >> (2 * (a.L - lc)));
+        const uint32_t item = a.dlist[d], tile = item & ((1u << kWholeShift) - 1u);
+        int l = (int)(item >> kWholeShift) - 1;
+        if (l < 0) {
+            __syncthreads();                        // tb reused across tiles
+            load_tile_bits(a.Sb, a.L, a.kt, tile, tb);
+            l = act ? group_level(tb, a.L, a.kt, g) : a.L;
+        }
+        if (a.q.zf[0] != nullptr && l < a.L - a.kt) {
+            // one coarser leaf covers the whole tile (as its act mark says):
+            // when its new value is (+0, +0, +0) and the tile already holds
+            // +0, nothing changes; otherwise the tile's mark goes (a thread
+            // that reads the mark late decides the same: the mark only counts
+            // where the value is zero, and then it is not written)
+            const uint64_t sc = lvl_off(l) + (((uint64_t)tile << (2 * a.kt)) >> (2 * (a.L - l)));
             const bool zero = pos_zero(fh[sc]) && pos_zero(fqx[sc]) && pos_zero(fqy[sc]);
             uint8_t* Y = nxt ? a.q.zf[1] : a.q.zf[0];
             if (zero && Y[tile]) continue;           // uniform over the CTA
-            __syncthreads();                         // every thread has read Y[tile]
-            if (threadIdx.x == 0) Y[tile] = 0;
+            if (g == 0u) Y[tile] = 0;
         }
-        const int l = act ? group_level(tb, a.L, a.kt, g) : a.L;
-        if (!needs_decode_kernel(l, a.L)) continue;
+        if (!act || !needs_decode_kernel(l, a.L)) continue;
         const uint32_t m0 = (tile << (2 * a.kt)) + 4u * g;
         const uint64_t slot = lvl_off(l) + (m0 >> (2 * (a.L - l)));
-        const T hl = fh[slot], qxl = fqx[slot], qyl = fqy[slot];
-        const bool restore = ge_nonneg(hl, a.tol);      // hl >= tol (tol > 0)
         const uint64_t fo = lvl_off(a.L) + m0;
+        // the leaf and the bed in one round of loads
+        const T hl = fh[slot], qxl = fqx[slot], qyl = fqy[slot], zl = __ldg(a.z + slot);
+        T z0, z1, z2, z3;
+        Vec4<T>::load(a.z + fo, z0, z1, z2, z3);
+        const bool restore = ge_nonneg(hl, a.tol);      // hl >= tol (tol > 0)
         T hf[4];
         if (restore) {
-            const T eta = eta_of(hl, __ldg(a.z + slot));
-            T z0, z1, z2, z3;
-            Vec4<T>::load(a.z + fo, z0, z1, z2, z3);
-            restore4(eta, z0, z1, z2, z3, hf);
+            restore4(eta_of(hl, zl), z0, z1, z2, z3, hf);
         } else {
             hf[0] = hf[1] = hf[2] = hf[3] = hl;
         }
