@@ -72,11 +72,11 @@ static __global__ void __launch_bounds__(256) kb_clear(const DomainPlan<T>* P, c
 // reloaded after each store the body makes (the store could alias it).
 
 template <typename T>
-static __global__ void __launch_bounds__(256) kb_encode(const DomainPlan<T>* P, const uint32_t* base, int D,
+static __global__ void __launch_bounds__(128, 6) kb_encode(const DomainPlan<T>* P, const uint32_t* base, int D,
                                                         int pass) {
     const int d = find_domain(base, D, blockIdx.x);
     const EncodeArgs<T, 3> a = P[d].enc;
-    encode_body<T, 3>(a, P[d].ls[pass], P[d].kk[pass], blockIdx.x - base[d]);
+    encode_blk<T, 3, 4>(a, P[d].ls[pass], P[d].kk[pass], blockIdx.x - base[d]);
 }
 
 template <typename T>
@@ -290,8 +290,7 @@ class BatchT final : public Batch {
             auto set = [&](int kind, uint32_t n) { nb[(size_t)kind * D + d] = n; };
             set(BK_CLEAR, std::min<uint32_t>(64u, (p.clear_n + 255u) / 256u));
             for (int q = 0; q < kMaxPasses; ++q)
-                set(BK_ENC0 + q, q < p.npass ? (1u << (2 * (p.ls[q] - ((q == 0 && p.enc.span) ? p.enc.span
-                                                                                          : p.kk[q])))) : 0u);
+                set(BK_ENC0 + q, q < p.npass ? (1u << (2 * (p.ls[q] - p.kk[q]))) : 0u);
             set(BK_FLAG, std::min<uint32_t>(64u, (bits_words(p.L) + 255u) / 256u));
             set(BK_TCOUNT, p.nct);
             set(BK_TSCAN, 1u);
@@ -336,7 +335,7 @@ class BatchT final : public Batch {
         if (total_[BK_CLEAR]) kb_clear<T><<<total_[BK_CLEAR], 256, 0, stream_>>>(d_plans_, base(BK_CLEAR), D);
         for (int q = 0; q < kMaxPasses; ++q)
             if (total_[BK_ENC0 + q])
-                kb_encode<T><<<total_[BK_ENC0 + q], 256, 0, stream_>>>(d_plans_, base(BK_ENC0 + q), D, q);
+                kb_encode<T><<<total_[BK_ENC0 + q], 128, 0, stream_>>>(d_plans_, base(BK_ENC0 + q), D, q);
         kb_flag<T><<<total_[BK_FLAG], 256, 0, stream_>>>(d_plans_, base(BK_FLAG), D);
         kb_trav_count<T><<<total_[BK_TCOUNT], 256, 0, stream_>>>(d_plans_, base(BK_TCOUNT), D);
         kb_trav_scan<T><<<total_[BK_TSCAN], 1024, 0, stream_>>>(d_plans_, base(BK_TSCAN), D);

@@ -813,16 +813,8 @@ class EngineT final : public Engine {
         p.enc.ls = L_;
         p.enc.k = enc_k;
         p.npass = 0;
-        p.enc.span = 0;
         for (int ls = L_; ls > 0 && p.npass < (int)(sizeof(p.ls) / sizeof(p.ls[0]));) {
             int k = ls < enc_k ? ls : enc_k;
-            // with 5 levels per pass, the first pass of a domain of L >= 8
-            // stops after three levels of each 1024-cell block, as the
-            // single-domain full sweep does (a shorter chain per CTA)
-            if (ls == L_ && enc_k == 5 && ls >= 8) {
-                k = 3;
-                p.enc.span = 5;
-            }
             p.ls[p.npass] = ls;
             p.kk[p.npass] = k;
             p.npass++;
@@ -950,32 +942,25 @@ class EngineT final : public Engine {
     void encode_passes(EncodeArgs<T, NF> a, uint32_t* ticket = nullptr, int from = -1) {
         int ls = from < 0 ? L_ : from;
         bool list_reset = a.list == nullptr;
+        const uint32_t few = (uint32_t)(nsm_ * enc_ctas(8));   // tiles that eight-warp CTAs hold at once
         while (ls > 0) {
             int k = ls < 5 ? ls : 5;
-            a.span = 0;
-            // a first pass over every one of many tiles stops after three
-            // levels of each 1024-cell block: a shorter chain per CTA, and the
-            // block's two top levels move to the next pass, which reads 1/64
-            // of the data
-            if (ls == L_ && a.zf[0] == nullptr && a.list == nullptr && NF == 3 && ls >= 8 &&
-                (1u << (2 * (ls - 5))) > (uint32_t)nsm_ * 8u) {
-                k = 3;
-                a.span = 5;
-            }
             a.ls = ls;
             a.k = k;
-            const uint32_t nb = 1u << (2 * (ls - (a.span ? a.span : k)));
+            const uint32_t nb = 1u << (2 * (ls - k));
             const int ls2 = ls - k, k2 = ls2 < 5 ? ls2 : 5;
             if (ls == L_ && a.list != nullptr) {
-                lk(k_encode_tiles<T, NF>, nsm_ * 8, 256, a);
+                lk(k_encode_tiles<T, NF, 4>, nsm_ * enc_ctas(4), 128, a);
                 mark("k_encode_tiles");
             } else if (ticket && ls2 > 0 && ls2 == k2) {      // next pass is the last (one CTA)
-                lk(k_encode_tail<T, NF>, nb, 256, a, ls2, k2, ticket);
+                if (nb > few) lk(k_encode_tail<T, NF, 4>, nb, 128, a, ls2, k2, ticket);
+                else lk(k_encode_tail<T, NF, 8>, nb, 256, a, ls2, k2, ticket);
                 mark("k_encode_tail");
                 list_reset = true;                         // its last CTA resets the list
                 break;                                     // levels ls2-1 .. 0 done too
             } else {
-                lk(k_encode<T, NF>, nb, 256, a);
+                if (nb > few) lk(k_encode<T, NF, 4>, nb, 128, a);
+                else lk(k_encode<T, NF, 8>, nb, 256, a);
                 mark("k_encode");
             }
             ls -= k;

@@ -95,14 +95,10 @@ __device__ __forceinline__ float absval(float x) { return __int_as_float(__float
 // whose FP64 pipe is the bottleneck.  Each returns the bits the IEEE
 // operation returns (NaN inputs aside, which the state checks report).
 // ---------------------------------------------------------------------------
-// x * 2^k for k in {-2, -1, 1}: an exponent step when input and result are
-// normal numbers, x itself for a zero; otherwise the IEEE product, in a
-// function of its own (an FP64 instruction the compiler predicates would
-// hold the pipe even where no lane needs it).
-template <int K>
-static __device__ __noinline__ double pow2_rare(double x) {
-    return x * (K == -2 ? 0.25 : (K == -1 ? 0.5 : 2.0));
-}
+// x * 2^K for K in {-2, -1, 1}: an exponent step when input and result are
+// normal numbers; otherwise the IEEE product formed by integer operations (an
+// FP64 instruction the compiler predicates would hold the pipe even where no
+// lane needs it).
 template <int K>
 __device__ __forceinline__ double pow2_scale(double x) {
     uint32_t lo, hi;
@@ -111,8 +107,7 @@ __device__ __forceinline__ double pow2_scale(double x) {
     // exponents e and e + K in [1, 2046]
     constexpr uint32_t e0 = (uint32_t)(K < 0 ? 1 - K : 1), e1 = (uint32_t)(K > 0 ? 2046 - K : 2046);
     if (m - (e0 << 20) < ((e1 - e0 + 1u) << 20)) return d_join((uint64_t)(hi + ((uint32_t)K << 20)) << 32 | lo);
-    if ((m | lo) == 0u) return x;
-    return pow2_rare<K>(x);
+    return d_join(pow2_bits<K>((uint64_t)hi << 32 | lo));
 }
 template <int K>
 __device__ __forceinline__ float pow2_scale(float x) {
@@ -295,7 +290,6 @@ struct EncodeArgs {
     uint32_t* Cb;         // upward closure of the threshold flags
     const DevState* st;   // NULL: buffer 0, always active
     int L, ls, k;         // source level ls; produces levels ls-1 .. ls-k
-    int span = 0;         // a CTA covers 4^span cells of level ls (0: 4^k)
     // Quiescent tiles (first pass only, its tiles are the traversal's):
     // zf[b][t] = 1 when every value of buffer b in tile t, levels ls-k..ls,
     // is +0.  NULL: no skipping.
@@ -342,20 +336,27 @@ __device__ __forceinline__ void parent_coef(const Thr<T>& h, T c0, T c1, T c2, T
 template <typename T, int NF>
 __device__ __forceinline__ void parents_all(const Thr<T>* th, const T (&c)[NF][4], T (&s)[NF], bool& tf) {
     if constexpr (sizeof(T) == 8) {
-        bool eq[NF];
+        bool eq[NF], all = true;
         T sa[NF], sb[NF];
 #pragma unroll
         for (int q = 0; q < NF; ++q) {
             eq[q] = same4<T>(c[q][0], c[q][1], c[q][2], c[q][3]);
+            all = all && eq[q];
             sa[q] = T(0);
             sb[q] = T(0);
-            if (!eq[q]) {
+            s[q] = c[q][0];
+        }
+        // still water and dry ground: a branch around all the sums (an FP64
+        // instruction predicated off would hold the pipe as well)
+        if (!all) {
+#pragma unroll
+            for (int q = 0; q < NF; ++q) {
                 sa[q] = c[q][0] + c[q][2];
                 sb[q] = c[q][1] + c[q][3];
             }
-        }
 #pragma unroll
-        for (int q = 0; q < NF; ++q) s[q] = eq[q] ? c[q][0] : quarter(sa[q] + sb[q]);
+            for (int q = 0; q < NF; ++q) s[q] = eq[q] ? c[q][0] : quarter(sa[q] + sb[q]);
+        }
 #pragma unroll
         for (int q = 0; q < NF; ++q) {
             if (tf) break;
@@ -437,8 +438,8 @@ __device__ __forceinline__ void restore4(T eta, T z0, T z1, T z2, T z3, T (&hf)[
     hf[3] = gt_zero(d3) ? d3 : T(0);
 }
 
-// One CTA encodes one tile: the 4^k cells of level ls under one level-(ls-k)
-// cell, k <= 5 levels in one pass.  The first level reads four children
+// One CTA encodes the 4^k cells of level ls under one level-(ls-k) cell, k <=
+// 4 levels in one pass (five: encode_tile).  The first level reads four children
 // per thread with 128-bit loads; the next levels work from shared memory.
 // CG: read the source level and the closure bits through L2 only (the tail
 // pass reads what other CTAs of the same launch wrote).
@@ -452,15 +453,12 @@ __device__ __forceinline__ void encode_body(const EncodeArgs<T, NF>& a, int ls, 
     const bool quiet = a.zf[0] != nullptr && ls == a.L;
     uint8_t* const zfp = par ? a.zf[1] : a.zf[0];   // (no dynamic index into parameters)
     if (quiet && zfp[bid]) return;
-    __shared__ T sv0[NF][256];        // level ls-1 (and ls-3, ls-5)
-    __shared__ T sv1[NF][64];         // level ls-2 (and ls-4)
+    __shared__ T sv0[NF][64];         // level ls-1 (and ls-3)
+    __shared__ T sv1[NF][16];         // level ls-2 (and ls-4)
     __shared__ uint32_t sc[2][8];
-    __shared__ Thr<T> sthr[5][NF];    // thresholds of the pass's levels (one load each)
+    __shared__ Thr<T> sthr[4][NF];    // thresholds of the pass's levels (one load each)
     const uint32_t tile = bid, tid = threadIdx.x, lane = tid & 31u, warp = tid >> 5;
-    // parents of level ls-1 under the CTA (its block of 4^span cells of
-    // level ls; a pass may stop short of the block's top level)
-    const int span = (ls == a.ls && a.span > kk) ? a.span : kk;
-    uint32_t cnt = 1u << (2 * (span - 1));
+    uint32_t cnt = 1u << (2 * (kk - 1));   // parents of level ls-1 under the CTA
     int n = ls - 1;
     {   // level ls-1
         const bool act = tid < cnt;
@@ -512,8 +510,10 @@ __device__ __forceinline__ void encode_body(const EncodeArgs<T, NF>& a, int ls, 
         const bool cf = act && (tf || cchild);
         put_bits(a.Tb, n, tile * cnt, cnt, act && tf);
         const uint32_t cball = put_bits(a.Cb, n, tile * cnt, cnt, cf);
+        if (act) {
 #pragma unroll
-        for (int q = 0; q < NF; ++q) sv0[q][tid] = s[q];
+            for (int q = 0; q < NF; ++q) sv0[q][tid] = s[q];
+        }
         if (lane == 0) sc[0][warp] = cball;
         if (quiet) {   // all finest values +0 => every coarser value written is +0
             const int any = __syncthreads_or(nz ? 1 : 0);
@@ -570,47 +570,194 @@ __device__ __forceinline__ void encode_body(const EncodeArgs<T, NF>& a, int ls, 
     }
 }
 
-template <typename T, int NF>
-static __global__ void __launch_bounds__(256) k_encode(EncodeArgs<T, NF> a) {
+// One CTA of W warps (4 or 8) encodes one tile, the 32 x 32 cells of level ls
+// under one level-(ls-5) cell: five levels.  Each warp takes its 256 / W parents
+// of the first level (a parent per lane) and the cells above them through three
+// levels (W = 8) or four (W = 4) on its own, with a lane per parent and quantity
+// above the first; then one barrier, and the first warp forms the rest.  A
+// parent is formed by the operations of encode_body, so the values and flags
+// are the same.
+//
+// Bound by latency (a chain of 21 FP64 additions with W = 8, 33 with W = 4, 77
+// cycles each, with the threshold decisions in between) until enough warps are
+// resident to fill the FP64 pipe.
+template <typename T, int NF, int W, bool CG = false>
+__device__ __forceinline__ void encode_tile(const EncodeArgs<T, NF>& a, int ls, uint32_t tile) {
+    if (a.st && !a.st->active) return;
+    const int par = a.st ? (int)a.st->cur : 0;
+    // a tile known to hold only +0 encodes to +0 (as in encode_body)
+    const bool quiet = a.zf[0] != nullptr && ls == a.L;
+    uint8_t* const zfp = par ? a.zf[1] : a.zf[0];
+    if (quiet && zfp[tile]) return;
+    constexpr uint32_t P1 = 256 / W, P2 = P1 / 4, P3 = P2 / 4;   // a warp's parents per level
+    __shared__ T sv1[W][NF][P1], sv2[W][NF][P2], sv3[NF][16], sv4[NF][4];
+    __shared__ Thr<T> sthr[W][5][NF];
+    __shared__ uint32_t scl[W];
+    const uint32_t lane = threadIdx.x & 31u, w = threadIdx.x >> 5;
+    const uint32_t b = tile * W + w;                  // the warp's share of every level
+    if (lane < 5u * NF) {
+        const int j = (int)lane / NF, q = (int)lane % NF, idx = (ls - 1 - j) * NF + q;
+        Thr<T> h;
+        h.thr = a.thr[idx];
+        h.thr4 = a.thr4[idx];
+        h.lo = a.thr4lo ? a.thr4lo[idx] : -1.0f;
+        h.hi = a.thr4hi ? a.thr4hi[idx] : -1.0f;
+        sthr[w][j][q] = h;
+    }
+    __syncwarp();
+    bool nz = false;
+    uint32_t cw[2] = {0u, 0u};                        // closure bits of the level below
+#pragma unroll 1
+    for (uint32_t r = 0; r * 32u < P1; ++r) {         // level ls-1
+        const uint32_t p = b * P1 + r * 32u + lane;
+        T c[NF][4], s[NF];
+        uint32_t cchild = 0u;
+#pragma unroll
+        for (int q = 0; q < NF; ++q) {
+            const T* fq = par ? a.f[1][q] : a.f[0][q];
+            if (CG) Vec4<T>::load_cg(fq + lvl_off(ls) + 4ull * p, c[q][0], c[q][1], c[q][2], c[q][3]);
+            else Vec4<T>::load(fq + lvl_off(ls) + 4ull * p, c[q][0], c[q][1], c[q][2], c[q][3]);
+        }
+        if (ls < a.L) {
+            const uint32_t* wd = a.Cb + word_off(ls) + (p >> 3);
+            cchild = ((CG ? __ldcg(wd) : __ldg(wd)) >> ((4u * p) & 31u)) & 0xFu;
+        }
+#pragma unroll
+        for (int q = 0; q < NF; ++q)
+            nz = nz || !(pos_zero(c[q][0]) && pos_zero(c[q][1]) && pos_zero(c[q][2]) && pos_zero(c[q][3]));
+        bool tf = false;
+        parents_all<T, NF>(sthr[w][0], c, s, tf);
+#pragma unroll
+        for (int q = 0; q < NF; ++q) {
+            (par ? a.f[1][q] : a.f[0][q])[lvl_off(ls - 1) + p] = s[q];
+            sv1[w][q][r * 32u + lane] = s[q];
+        }
+        const uint32_t tb = __ballot_sync(0xffffffffu, tf), cb = __ballot_sync(0xffffffffu, tf || cchild != 0u);
+        if (lane == 0u) {
+            a.Tb[word_off(ls - 1) + (b * P1) / 32u + r] = tb;
+            a.Cb[word_off(ls - 1) + (b * P1) / 32u + r] = cb;
+        }
+        if (r == 0u) cw[0] = cb;
+        else cw[1] = cb;
+    }
+    __syncwarp();
+    // bits t (threshold) and cl (closure) of cells of level n from code `first`
+    // on: OR-ed into words cleared before the pass
+    auto put = [&](int n, uint32_t first, uint32_t t, uint32_t cl) {
+        if (lane != 0u) return;
+        if (t) atomicOr(a.Tb + word_off(n) + (first >> 5), t << (first & 31u));
+        if (cl) atomicOr(a.Cb + word_off(n) + (first >> 5), cl << (first & 31u));
+    };
+    // one level of n parents (a power of two): lane = (quantity, parent),
+    // children at v[q * stride + 4 i], results to out[q * ostride + i] and to
+    // the hierarchy from cell `first` on; returns the threshold bits
+    auto level = [&](int j, uint32_t n, const T* v, uint32_t stride, T* out, uint32_t ostride, uint32_t first) -> uint32_t {
+        uint32_t t = 0u;
+#pragma unroll 1
+        for (uint32_t r = 0; r < n * NF; r += 32u) {
+            const uint32_t id = r + lane, q = id / n, i = id & (n - 1u);
+            bool f = false;
+            if (q < (uint32_t)NF) {
+                const T* x = v + q * stride + 4u * i;
+                T sp = T(0);
+                parent_coef(sthr[w][j - 1][q], x[0], x[1], x[2], x[3], sp, f);
+                quantity_ptr(a, par, q)[lvl_off(ls - j) + first + i] = sp;
+                out[q * ostride + i] = sp;
+            }
+            uint32_t m = __ballot_sync(0xffffffffu, f);
+            for (uint32_t k = 0; k < 32u; k += n) t |= m >> k;
+        }
+        __syncwarp();
+        return t & ((1u << n) - 1u);
+    };
+    // the closure of n parents: their own flags or a closed child's
+    auto close = [&](uint32_t n, uint32_t t, bool child) { return t | (__ballot_sync(0xffffffffu, child) & ((1u << n) - 1u)); };
+    const uint32_t T2 = level(2, P2, sv1[w][0], P1, sv2[w][0], P2, b * P2);
+    const uint32_t C2 = close(P2, T2, (((lane < 8u ? cw[0] : cw[1]) >> (4u * (lane & 7u))) & 0xFu) != 0u);
+    put(ls - 2, b * P2, T2, C2);
+    const uint32_t T3 = level(3, P3, sv2[w][0], P2, &sv3[0][w * P3], 16u, b * P3);
+    const uint32_t C3 = close(P3, T3, lane < P3 && ((C2 >> (4u * lane)) & 0xFu) != 0u);
+    put(ls - 3, b * P3, T3, C3);
+    uint32_t C4 = 0u;
+    if constexpr (W == 4) {
+        const uint32_t T4 = level(4, 1u, &sv3[0][w * 4u], 16u, &sv4[0][w], 4u, b);
+        C4 = (T4 | C3) ? 1u : 0u;
+        put(ls - 4, b, T4, C4);
+    }
+    if (lane == 0u) scl[w] = W == 4 ? C4 : C3;
+    const int any = __syncthreads_or(nz ? 1 : 0);
+    // all source values +0 => every coarser value written is +0
+    if (quiet && threadIdx.x == 0) zfp[tile] = any ? 0 : 1;
+    if (w != 0u) return;
+    if constexpr (W == 4) {
+        C4 = __ballot_sync(0xffffffffu, lane < 4u && scl[lane & 3u] != 0u);
+    } else {
+        const uint32_t all = __ballot_sync(0xffffffffu, lane < 16u && ((scl[(lane >> 1) & 7u] >> (lane & 1u)) & 1u) != 0u);
+        const uint32_t T4 = level(4, 4u, sv3[0], 16u, sv4[0], 4u, tile * 4u);
+        C4 = close(4u, T4, lane < 4u && ((all >> (4u * lane)) & 0xFu) != 0u);
+        put(ls - 4, tile * 4u, T4, C4);
+    }
+    __shared__ T top[NF];
+    const uint32_t T5 = level(5, 1u, sv4[0], 4u, top, 1u, tile);
+    put(ls - 5, tile, T5, (T5 | C4) ? 1u : 0u);
+}
+
+// Passes of fewer than five levels have at most 64 parents a block: either W
+// has the threads.
+template <typename T, int NF, int W, bool CG = false>
+__device__ __forceinline__ void encode_blk(const EncodeArgs<T, NF>& a, int ls, int kk, uint32_t bid) {
+    if (kk == 5) encode_tile<T, NF, W, CG>(a, ls, bid);
+    else encode_body<T, NF, CG>(a, ls, kk, bid);
+}
+
+// With many tiles four warps a tile (72 registers a thread: seven CTAs per SM,
+// so that 1024 tiles are resident at once), with few eight (the shorter
+// chain).
+constexpr int enc_ctas(int W) { return W == 4 ? 7 : 2; }
+template <typename T, int NF, int W>
+static __global__ void __launch_bounds__(W * 32, enc_ctas(W)) k_encode(EncodeArgs<T, NF> a) {
     pdl_wait();
-    encode_body<T, NF>(a, a.ls, a.k, blockIdx.x);
+    encode_blk<T, NF, W>(a, a.ls, a.k, blockIdx.x);
 }
 
 // A pass followed, in its last CTA to finish, by the final one-CTA pass
 // (levels ls2-1 .. 0), saving a launch; ticket counts the finished CTAs and
 // is reset by the last one.
-template <typename T, int NF>
-static __global__ void __launch_bounds__(256) k_encode_tail(EncodeArgs<T, NF> a, int ls2, int k2,
-                                                            uint32_t* ticket) {
+template <typename T, int NF, int W>
+static __global__ void __launch_bounds__(W * 32, enc_ctas(W)) k_encode_tail(EncodeArgs<T, NF> a, int ls2, int k2,
+                                                                       uint32_t* ticket) {
     pdl_wait();
-    encode_body<T, NF>(a, a.ls, a.k, blockIdx.x);
-    __threadfence();                     // this CTA's coefficients and bits are visible
-    __syncthreads();
     __shared__ bool last;
-    if (threadIdx.x == 0) last = atomicAdd(ticket, 1u) == gridDim.x - 1u;
-    __syncthreads();
-    if (!last) return;
-    __threadfence();
-    if (threadIdx.x == 0) {
-        *ticket = 0u;
-        // the tile list of the pass before (k_encode_tiles, done) starts
-        // empty next step
-        if (a.list) const_cast<DevState*>(a.st)->ntodo = 0u;
+#pragma unroll 1
+    for (int pass = 0; pass < 2; ++pass) {           // (one copy of the code)
+        encode_blk<T, NF, W, true>(a, pass == 0 ? a.ls : ls2, pass == 0 ? a.k : k2, pass == 0 ? blockIdx.x : 0u);
+        if (pass == 1) return;
+        __threadfence();                     // this CTA's coefficients and bits are visible
+        __syncthreads();
+        if (threadIdx.x == 0) last = atomicAdd(ticket, 1u) == gridDim.x - 1u;
+        __syncthreads();
+        if (!last) return;
+        __threadfence();
+        if (threadIdx.x == 0) {
+            *ticket = 0u;
+            // the tile list of the pass before (k_encode_tiles, done) starts
+            // empty next step
+            if (a.list) const_cast<DevState*>(a.st)->ntodo = 0u;
+        }
     }
-    encode_body<T, NF, true>(a, ls2, k2, 0u);
 }
 
-// The same pass with a fixed grid when quiescent tiles are skipped: the
+// The first pass with a fixed grid when quiescent tiles are skipped: the
 // tiles that are not marked quiescent were listed by k_clear_words, and CTA
 // b encodes list entries b, b + grid, ...: a step's active tiles, which
 // cluster where the water is, spread one per CTA.
-template <typename T, int NF>
-static __global__ void __launch_bounds__(256) k_encode_tiles(EncodeArgs<T, NF> a) {
+template <typename T, int NF, int W>
+static __global__ void __launch_bounds__(W * 32, enc_ctas(W)) k_encode_tiles(EncodeArgs<T, NF> a) {
     pdl_wait();
     if (!a.st->active) return;
     const uint32_t n = *(volatile const uint32_t*)&a.st->ntodo;
     for (uint32_t e = blockIdx.x; e < n; e += gridDim.x) {
-        encode_body<T, NF>(a, a.ls, a.k, __ldg(a.list + e));
+        encode_tile<T, NF, W>(a, a.ls, __ldg(a.list + e));
         __syncthreads();                 // shared memory is reused by the next tile
     }
 }

@@ -172,6 +172,28 @@ __host__ __device__ __forceinline__ uint64_t mul_bits(uint32_t al, uint32_t ah, 
     return (uint64_t)rh << 32 | rl;
 }
 
+// ---- scaling by a power of two -----------------------------------------------
+// x 2^K, |K| <= 2, where x or the result is not normal: zeros and subnormals
+// (rounded where bits are lost), overflow, infinities (NaN: x)
+template <int K>
+__host__ __device__ __forceinline__ uint64_t pow2_bits(uint64_t b) {
+    const uint64_t s = b & 0x8000000000000000ull, a = b ^ s;
+    const int e = (int)(a >> 52);
+    if (e == 0x7FF) return b;
+    if (K > 0) {
+        if (e + K > 2046) return s | 0x7FF0000000000000ull;
+        if (e != 0) return b + ((uint64_t)K << 52);
+        uint64_t m = a;
+        for (int k = 0; k < K; ++k) m = m >> 52 ? m + (1ull << 52) : m << 1;
+        return s | m;
+    }
+    if (e > -K) return b - ((uint64_t)(-K) << 52);
+    const uint64_t m = e == 0 ? a : (a & 0x000FFFFFFFFFFFFFull) | 0x0010000000000000ull;
+    const int sh = e == 0 ? -K : 1 - K - e;
+    const uint64_t r = m >> sh, rem = m & ((1ull << sh) - 1ull), half = 1ull << (sh - 1);
+    return s | (r + (rem > half || (rem == half && (r & 1ull)) ? 1ull : 0ull));
+}
+
 #ifdef __CUDACC__
 // Device forms on doubles.  Operands outside an operation's range (next to
 // no lane meets one) take the FP64 instruction in a function of its own: a

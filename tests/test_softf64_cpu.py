@@ -81,6 +81,11 @@ int main(int, char** argv) {
             const uint32_t y = fbits((float)(1.0 / (double)fval(rcp_seed_arg(lo, hi)))) + d;
             check("rcp", x, rcp_bits(lo, hi, y), 1.0 / val(x));
         }
+        if (a << 1 <= 0x7FF0000000000000ull << 1) {            // (not a NaN)
+            check("2 x", a, pow2_bits<1>(a), 2.0 * val(a));
+            check("x / 2", a, pow2_bits<-1>(a), 0.5 * val(a));
+            check("x / 4", a, pow2_bits<-2>(a), 0.25 * val(a));
+        }
         uint64_t p = a, q = operand();
         if (i % 4 == 2) {                      // 27-bit factors: products of 53 and 54 bits, ties among them
             p = (p & 0xFFF0000000000000ull) | (rnd() & 0x3FFFFFF) << 26;
