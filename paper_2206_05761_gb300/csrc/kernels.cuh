@@ -2421,37 +2421,48 @@ __device__ __forceinline__ void queued_face(const StepArgs<T>& a, const CellSrc<
         // face's other side belongs to no leaf)
         matched_face(a, src, s, d.n, compact16(d.code), compact16(d.code >> 1), F, own2);
     } else {
+        // the two sides' records by queue slot: normal and tangential
+        // velocity, free surface and bed (the sides' order is a choice of
+        // slots, not of values)
         const unsigned long long m = __ldg(a.mark + iX), mc = __ldg(a.mark + d.iC);
-        const typename Pair2<T>::V uv = *pair_at(a.face, cap, kLeafUV, w), ez = *pair_at(a.face, cap, kLeafEZ, w);
-        typename Pair2<T>::V xuv, xez;
-        bool safe = ok && !((uint32_t)mc & kUnsafe);
-        if ((uint32_t)(m >> 32) == tag) {                 // queued too (at an edge: the leaf itself)
-            const uint32_t wx = (uint32_t)m & ~kUnsafe;
-            xuv = *pair_at(a.face, cap, kLeafUV, wx);
-            xez = *pair_at(a.face, cap, kLeafEZ, wx);
-            safe = safe && !((uint32_t)m & kUnsafe);
-        } else {
-            Cell<T> X = fetch(src, iX);
+        const bool queued = (uint32_t)(m >> 32) == tag;   // (at an edge: the leaf itself)
+        const uint32_t wx = queued ? (uint32_t)m & ~kUnsafe : w;
+        const uint32_t wL = right ? wx : w, wR = right ? w : wx;
+        const T* const rec = a.face + kLeafUV * cap;
+        const uint32_t on = yface ? 1u : 0u;
+        T nL = rec[2 * (size_t)wL + on], tL = rec[2 * (size_t)wL + (on ^ 1u)];
+        T nR = rec[2 * (size_t)wR + on], tR = rec[2 * (size_t)wR + (on ^ 1u)];
+        typename Pair2<T>::V ezL = *pair_at(a.face, cap, kLeafEZ, wL), ezR = *pair_at(a.face, cap, kLeafEZ, wR);
+        bool safe = ok && !(((uint32_t)mc | (queued ? (uint32_t)m : 0u)) & kUnsafe);
+        if (!queued) {
+            const Cell<T> X = fetch(src, iX);
             T u, v;
             velocity(X, a.P.tol, u, v);
             safe = safe && cell_window(X.h, X.z, u, v);
-            xuv = make_pair2(u, v);
-            xez = make_pair2(eta_of(X.h, X.z), X.z);
-        }
-        T un = yface ? uv.y : uv.x, ut = yface ? uv.x : uv.y;
-        T xn = yface ? xuv.y : xuv.x, xt = yface ? xuv.x : xuv.y;
-        if (edge) {
+            const T xn = yface ? v : u, xt = yface ? u : v;
+            if (right) {
+                nL = xn;
+                tL = xt;
+                ezL = make_pair2(eta_of(X.h, X.z), X.z);
+            } else {
+                nR = xn;
+                tR = xt;
+                ezR = make_pair2(eta_of(X.h, X.z), X.z);
+            }
+        } else if (edge) {
             // the ghost's velocity is the leaf's, the normal part reversed at
             // a wall (a dry leaf's is +0 either way)
             const int wall = s == 0 ? a.bc_ref[0] : (s == 1 ? a.bc_ref[1] : (s == 2 ? a.bc_ref[2] : a.bc_ref[3]));
-            if (wall && ge_nonneg(__ldg(src.h + d.iC), a.P.tol)) xn = -xn;
+            if (wall && ge_nonneg(__ldg(src.h + d.iC), a.P.tol)) {
+                if (right) nL = -nL;
+                else nR = -nR;
+            }
         }
         T hl, hr;
-        hll_face(a.P.g, a.P.hg, a.P.tol, right ? xez.x : ez.x, right ? xez.y : ez.y, right ? xn : un, right ? xt : ut,
-                 right ? ez.x : xez.x, right ? ez.y : xez.y, right ? un : xn, right ? ut : xt, safe, F, hl, hr);
-        const T own = right ? hr : hl, other = right ? hl : hr;
-        own2 = prod(own, own);
-        if (!right) other2 = prod(other, other);
+        hll_face(a.P.g, a.P.hg, a.P.tol, ezL.x, ezL.y, nL, tL, ezR.x, ezR.y, nR, tR, safe, F, hl, hr);
+        const T l2 = prod(hl, hl), r2 = prod(hr, hr);
+        own2 = right ? r2 : l2;
+        other2 = r2;
     }
     const int k = s == 0 ? kFaceW : (s == 1 ? kFaceE : (s == 2 ? kFaceS : kFaceN));
     *pair_at(a.face, cap, k, w) = make_pair2(F[0], F[1]);
@@ -2459,26 +2470,27 @@ __device__ __forceinline__ void queued_face(const StepArgs<T>& a, const CellSrc<
     if (!right) a.face[(k + 4) * cap + w] = other2;
 }
 
-// A block takes as many leaves as half its threads: the first half forms their
-// east faces, the second half their north faces.  The west and south faces
-// that no neighbour shares are gathered in shared memory meanwhile and formed
-// in a second round by as few warps as they fill: resolution changes and
-// shorelines would otherwise have every warp that holds one such leaf run
-// two more faces.  One face per thread and one copy of the face's code (some
-// 1200 instructions) for all four sides also halves the latency of a short
-// queue and keeps the loop in the instruction cache.
+// A warp takes 32 leaves (16 where the queue is too short to give every warp
+// 32): a face per lane, the east faces, then the north ones.  Meanwhile it
+// gathers the west and south faces that no neighbour shares, and forms them
+// last, 32 at a time: resolution changes and shorelines would otherwise have
+// every warp that holds one such leaf run two more faces.  One copy of the
+// face's code (some 1200 instructions) serves all four sides and stays in the
+// instruction cache; warps wait for nobody.
 //
 // Bound by the FP64 pipe and the integer pipe together: 1 M leaves (uniform
-// FV1, L=10) take 148 us, in which the FP64 pipe's 24 sums a face fill 71 % of
-// the cycles and 790 integer instructions 61 %; 321 us with every operation on
-// the FP64 pipe and two faces per thread.
+// FV1, L=10) take 133 us, in which the FP64 pipe's 24 sums a face fill 78 %
+// of the cycles and 780 integer instructions 66 %; 321 us with every operation
+// on the FP64 pipe and two faces per thread.
 template <typename T, bool FM = false>
 __device__ __forceinline__ void fv1_faces_body(const StepArgs<T>& a, Blk B) {
     DevState* st = a.st;
     if (!st->active) return;
     const uint32_t nw = st->nwet, nq = nw < a.fcap ? nw : a.fcap;
-    const uint32_t hb = blockDim.x >> 1, tid = threadIdx.x;
-    if (B.id * hb >= nq) return;                  // whole block idle
+    const uint32_t lane = threadIdx.x & 31u, warp = threadIdx.x >> 5, wpb = blockDim.x >> 5;
+    const uint32_t warps = B.n * wpb;
+    const uint32_t per = nq < 32u * warps ? 16u : 32u;
+    const uint32_t below = (1u << lane) - 1u;
     const int par = (int)st->cur;
     CellSrc<T> src;
     src.h = par ? a.f[1][0] : a.f[0][0];
@@ -2487,41 +2499,40 @@ __device__ __forceinline__ void fv1_faces_body(const StepArgs<T>& a, Blk B) {
     src.z = a.z;
     const uint32_t tag = st->epoch + 1u;
     const bool ok = const_window(a.P.g, a.P.tol);
-    __shared__ uint32_t nlist;
-    __shared__ uint16_t list[256];
-    const bool first = tid < hb;
-    const uint32_t l0 = first ? tid : tid - hb;
-    for (uint32_t base = B.id * hb; base < nq; base += B.n * hb) {
-        if (tid == 0) nlist = 0u;
-        __syncthreads();
-        uint32_t l = l0;
-        int s = first ? 1 : 3;
-        bool on = base + l < nq;
-        AxisProbe d = {};
-        if (on) {
-            // the face opposite to this thread's: shared by a queued neighbour?
-            d = axis_probe(a.wet[base + l], !first);
-            if (d.endM || (uint32_t)(__ldg(a.mark + d.iM) >> 32) != tag)
-                list[atomicAdd(&nlist, 1u)] = (uint16_t)(first ? l : l | 0x8000u);
-        }
+    __shared__ uint8_t lists[8][64];              // (blocks of up to 8 warps)
+    uint8_t* const list = lists[warp];
+    for (uint32_t base = (B.id * wpb + warp) * per; base < nq; base += warps * per) {
+        uint32_t n = 0u;                          // faces gathered
 #pragma unroll 1
-        for (int round = 0; round < 2; ++round) {
-            if (on) queued_face<T, FM>(a, src, tag, ok, base + l, s, d);
-            if (round == 1) break;
-            __syncthreads();
-            on = tid < nlist;
-            if (on) {
-                const uint32_t e = list[tid];
-                l = e & 0x7FFFu;
-                s = (e & 0x8000u) ? 2 : 0;
-                d = axis_probe(a.wet[base + l], s == 2);
+        for (uint32_t t0 = 0u; t0 < 2u * per + n; t0 += 32u) {
+            const uint32_t t = t0 + lane;
+            uint32_t l = t & (per - 1u);
+            int s = t < per ? 1 : 3;
+            bool on = true;
+            if (t0 >= 2u * per) {                 // (uniform: 2 per is a multiple of 32)
+                const uint32_t k = t - 2u * per;
+                on = k < n;
+                const uint32_t e = on ? list[k] : 0u;
+                l = e & 31u;
+                s = (e & 32u) ? 2 : 0;
             }
+            on = on && base + l < nq;
+            AxisProbe d = {};
+            if (on) d = axis_probe(a.wet[base + l], s >= 2);
+            if (t0 < 2u * per) {
+                // the face opposite to this lane's: shared by a queued neighbour?
+                const bool miss = on && (d.endM || (uint32_t)(__ldg(a.mark + d.iM) >> 32) != tag);
+                const uint32_t m = __ballot_sync(0xffffffffu, miss);
+                if (miss) list[n + __popc(m & below)] = (uint8_t)(s == 1 ? l : l | 32u);
+                n += __popc(m);
+            }
+            if (on) queued_face<T, FM>(a, src, tag, ok, base + l, s, d);
+            __syncwarp();                         // the list before its readers and the next writers
         }
-        __syncthreads();                          // the list is read before the next chunk's
     }
 }
 template <typename T, bool FM = false>
-static __global__ void __launch_bounds__(128) k_fv1_faces(StepArgs<T> a) {
+static __global__ void __launch_bounds__(128, 8) k_fv1_faces(StepArgs<T> a) {
     pdl_wait();
     fv1_faces_body<T, FM>(a, this_blk());
 }

@@ -152,7 +152,7 @@ __host__ __device__ __forceinline__ uint64_t mul_bits(uint32_t al, uint32_t ah, 
     const uint32_t e = (ah & mask) + (bh & mask) - (1012u << 20) - (z << 20);
     uint32_t rl, rh;
 #ifdef __CUDA_ARCH__
-    asm("{.reg .u32 t; and.b32 t, %2, 1; add.u32 t, t, 0x7fffffff; add.cc.u32 t, t, %4; addc.cc.u32 %0, %2, 0; "
+    asm("{.reg .u32 t; shl.b32 t, %2, 31; add.cc.u32 t, t, t; addc.cc.u32 t, %4, 0x7fffffff; addc.cc.u32 %0, %2, 0; "
         "addc.u32 %1, %3, %5;}"
         : "=r"(rl), "=r"(rh) : "r"(kl), "r"(kh), "r"(f), "r"(e));
 #else
