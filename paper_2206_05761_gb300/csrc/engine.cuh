@@ -852,6 +852,7 @@ class EngineT final : public Engine {
         const uint64_t g = (N_ + 63) / 64, cap = (uint64_t)nsm_ * 16;
         return (int)(g < cap ? (g < 1 ? 1 : g) : cap);
     }
+    // four warps a block, sixteen leaves or more a warp
     int faces_grid() const {
         const uint64_t g = (N_ + 63) / 64, cap = (uint64_t)nsm_ * 16;
         return (int)(g < cap ? g : cap);

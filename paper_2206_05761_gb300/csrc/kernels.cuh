@@ -17,23 +17,23 @@
 namespace hwfv1 {
 
 template <typename T> struct Vec4;
+// Four doubles as one 256-bit access: a lane's 32 bytes are a full sector, and a
+// pass takes half the load and store instructions of 128-bit ones.  Every
+// level starts on a multiple of 64 elements and the groups on multiples of
+// four, so p is 32-byte aligned.  Decode of water columns at L=11 (100 MB
+// written): 38 to 29 us.
 template <> struct Vec4<double> {
     static __device__ __forceinline__ void load(const double* p, double& a, double& b, double& c,
                                                 double& d) {
-        const double2 u = __ldg(reinterpret_cast<const double2*>(p));
-        const double2 v = __ldg(reinterpret_cast<const double2*>(p) + 1);
-        a = u.x; b = u.y; c = v.x; d = v.y;
+        asm("ld.global.nc.v4.f64 {%0, %1, %2, %3}, [%4];" : "=d"(a), "=d"(b), "=d"(c), "=d"(d) : "l"(p));
     }
     static __device__ __forceinline__ void store(double* p, double a, double b, double c, double d) {
-        reinterpret_cast<double2*>(p)[0] = make_double2(a, b);
-        reinterpret_cast<double2*>(p)[1] = make_double2(c, d);
+        asm volatile("st.global.v4.f64 [%0], {%1, %2, %3, %4};" ::"l"(p), "d"(a), "d"(b), "d"(c), "d"(d) : "memory");
     }
     // through L2 only: for data other CTAs of the same kernel wrote
     static __device__ __forceinline__ void load_cg(const double* p, double& a, double& b, double& c,
                                                    double& d) {
-        const double2 u = __ldcg(reinterpret_cast<const double2*>(p));
-        const double2 v = __ldcg(reinterpret_cast<const double2*>(p) + 1);
-        a = u.x; b = u.y; c = v.x; d = v.y;
+        asm volatile("ld.global.cg.v4.f64 {%0, %1, %2, %3}, [%4];" : "=d"(a), "=d"(b), "=d"(c), "=d"(d) : "l"(p) : "memory");
     }
 };
 template <> struct Vec4<float> {
@@ -333,30 +333,33 @@ __device__ __forceinline__ void parent_coef(const Thr<T>& h, T c0, T c1, T c2, T
 // shortcut: once a quantity has flagged the parent the others need their
 // parent only.  Every value is formed by the same operations as in
 // haar4_pre.
+//
+// zero: whether a detail of 0 passes some quantity's threshold.  Returns
+// whether every quantity's four children are equal: still water and dry ground
+// then branch around the sums and the decisions (an FP64 instruction predicated
+// off would hold the pipe as well).
 template <typename T, int NF>
-__device__ __forceinline__ void parents_all(const Thr<T>* th, const T (&c)[NF][4], T (&s)[NF], bool& tf) {
+__device__ __forceinline__ bool parents_all(const Thr<T>* th, const T (&c)[NF][4], T (&s)[NF], bool& tf, bool zero) {
+    bool eq[NF], all = true;
+#pragma unroll
+    for (int q = 0; q < NF; ++q) {
+        eq[q] = same4<T>(c[q][0], c[q][1], c[q][2], c[q][3]);
+        all = all && eq[q];
+        s[q] = c[q][0];
+    }
+    if (all) {
+        tf = tf || zero;
+        return true;
+    }
     if constexpr (sizeof(T) == 8) {
-        bool eq[NF], all = true;
         T sa[NF], sb[NF];
 #pragma unroll
         for (int q = 0; q < NF; ++q) {
-            eq[q] = same4<T>(c[q][0], c[q][1], c[q][2], c[q][3]);
-            all = all && eq[q];
-            sa[q] = T(0);
-            sb[q] = T(0);
-            s[q] = c[q][0];
+            sa[q] = c[q][0] + c[q][2];
+            sb[q] = c[q][1] + c[q][3];
         }
-        // still water and dry ground: a branch around all the sums (an FP64
-        // instruction predicated off would hold the pipe as well)
-        if (!all) {
 #pragma unroll
-            for (int q = 0; q < NF; ++q) {
-                sa[q] = c[q][0] + c[q][2];
-                sb[q] = c[q][1] + c[q][3];
-            }
-#pragma unroll
-            for (int q = 0; q < NF; ++q) s[q] = eq[q] ? c[q][0] : quarter(sa[q] + sb[q]);
-        }
+        for (int q = 0; q < NF; ++q) s[q] = eq[q] ? c[q][0] : quarter(sa[q] + sb[q]);
 #pragma unroll
         for (int q = 0; q < NF; ++q) {
             if (tf) break;
@@ -392,6 +395,7 @@ __device__ __forceinline__ void parents_all(const Thr<T>* th, const T (&c)[NF][4
 #pragma unroll
         for (int q = 0; q < NF; ++q) parent_coef(th[q], c[q][0], c[q][1], c[q][2], c[q][3], s[q], tf);
     }
+    return false;
 }
 
 // Hierarchy of quantity q in the current state buffer (selects, so that the
@@ -408,6 +412,9 @@ __device__ __forceinline__ T* quantity_ptr(const EncodeArgs<T, NF>& a, int par, 
 // the value is +0 (all bits clear)
 __device__ __forceinline__ bool pos_zero(double x) { return dbits(x) == 0ll; }
 __device__ __forceinline__ bool pos_zero(float x) { return __float_as_int(x) == 0; }
+
+__device__ __forceinline__ bool same_bits(double a, double b) { return dbits(a) == dbits(b); }
+__device__ __forceinline__ bool same_bits(float a, float b) { return __float_as_int(a) == __float_as_int(b); }
 
 // R-decode's free surface and finest depths with the FP64 work a flat bed
 // does not need: x + (+0) = x for x != -0 and x - (+0) = x for every x are
@@ -500,7 +507,10 @@ __device__ __forceinline__ void encode_body(const EncodeArgs<T, NF>& a, int ls, 
 #pragma unroll
             for (int q = 0; q < NF; ++q)
                 nz = nz || !(pos_zero(c[q][0]) && pos_zero(c[q][1]) && pos_zero(c[q][2]) && pos_zero(c[q][3]));
-            parents_all<T, NF>(sthr[0], c, s, tf);
+            bool zero = false;
+#pragma unroll
+            for (int q = 0; q < NF; ++q) zero = zero || passes_thr(T(0), sthr[0][q].thr, sthr[0][q].thr4);
+            parents_all<T, NF>(sthr[0], c, s, tf, zero);
 #pragma unroll
             for (int q = 0; q < NF; ++q) {
                 T* fq = par ? a.f[1][q] : a.f[0][q];
@@ -595,6 +605,7 @@ __device__ __forceinline__ void encode_tile(const EncodeArgs<T, NF>& a, int ls, 
     __shared__ uint32_t scl[W];
     const uint32_t lane = threadIdx.x & 31u, w = threadIdx.x >> 5;
     const uint32_t b = tile * W + w;                  // the warp's share of every level
+    bool zp = false;
     if (lane < 5u * NF) {
         const int j = (int)lane / NF, q = (int)lane % NF, idx = (ls - 1 - j) * NF + q;
         Thr<T> h;
@@ -603,9 +614,14 @@ __device__ __forceinline__ void encode_tile(const EncodeArgs<T, NF>& a, int ls, 
         h.lo = a.thr4lo ? a.thr4lo[idx] : -1.0f;
         h.hi = a.thr4hi ? a.thr4hi[idx] : -1.0f;
         sthr[w][j][q] = h;
+        zp = passes_thr(T(0), h.thr, h.thr4);
     }
-    __syncwarp();
-    bool nz = false;
+    // bit j NF + q: a detail of 0 passes the threshold of level ls-1-j, quantity q
+    const uint32_t zbits = __ballot_sync(0xffffffffu, zp);
+    bool nz = false, same = true;                     // same: the warp's cells have held one value so far
+    T one[NF];
+#pragma unroll
+    for (int q = 0; q < NF; ++q) one[q] = T(0);
     uint32_t cw[2] = {0u, 0u};                        // closure bits of the level below
 #pragma unroll 1
     for (uint32_t r = 0; r * 32u < P1; ++r) {         // level ls-1
@@ -622,11 +638,22 @@ __device__ __forceinline__ void encode_tile(const EncodeArgs<T, NF>& a, int ls, 
             const uint32_t* wd = a.Cb + word_off(ls) + (p >> 3);
             cchild = ((CG ? __ldcg(wd) : __ldg(wd)) >> ((4u * p) & 31u)) & 0xFu;
         }
-#pragma unroll
-        for (int q = 0; q < NF; ++q)
-            nz = nz || !(pos_zero(c[q][0]) && pos_zero(c[q][1]) && pos_zero(c[q][2]) && pos_zero(c[q][3]));
         bool tf = false;
-        parents_all<T, NF>(sthr[w][0], c, s, tf);
+        const bool eq = parents_all<T, NF>(sthr[w][0], c, s, tf, (zbits & ((1u << NF) - 1u)) != 0u);
+        // four children that differ are not all +0
+        nz = nz || !eq;
+#pragma unroll
+        for (int q = 0; q < NF; ++q) nz = nz || !pos_zero(s[q]);
+        same = same && __all_sync(0xffffffffu, eq);
+        if (same) {
+            bool is = true;
+#pragma unroll
+            for (int q = 0; q < NF; ++q) {
+                if (r == 0u) one[q] = __shfl_sync(0xffffffffu, s[q], 0);
+                is = is && same_bits(s[q], one[q]);
+            }
+            same = __all_sync(0xffffffffu, is);
+        }
 #pragma unroll
         for (int q = 0; q < NF; ++q) {
             (par ? a.f[1][q] : a.f[0][q])[lvl_off(ls - 1) + p] = s[q];
@@ -660,7 +687,14 @@ __device__ __forceinline__ void encode_tile(const EncodeArgs<T, NF>& a, int ls, 
             if (q < (uint32_t)NF) {
                 const T* x = v + q * stride + 4u * i;
                 T sp = T(0);
-                parent_coef(sthr[w][j - 1][q], x[0], x[1], x[2], x[3], sp, f);
+                if (same) {                   // equal children all the way (warp-uniform)
+#pragma unroll
+                    for (int k = 0; k < NF; ++k)
+                        if (q == (uint32_t)k) sp = one[k];
+                    f = ((zbits >> ((j - 1) * NF + q)) & 1u) != 0u;
+                } else {
+                    parent_coef(sthr[w][j - 1][q], x[0], x[1], x[2], x[3], sp, f);
+                }
                 quantity_ptr(a, par, q)[lvl_off(ls - j) + first + i] = sp;
                 out[q * ostride + i] = sp;
             }
@@ -689,6 +723,7 @@ __device__ __forceinline__ void encode_tile(const EncodeArgs<T, NF>& a, int ls, 
     // all source values +0 => every coarser value written is +0
     if (quiet && threadIdx.x == 0) zfp[tile] = any ? 0 : 1;
     if (w != 0u) return;
+    same = false;                            // the other warps' cells may hold other values
     if constexpr (W == 4) {
         C4 = __ballot_sync(0xffffffffu, lane < 4u && scl[lane & 3u] != 0u);
     } else {
@@ -2646,8 +2681,9 @@ struct DecodeArgs {
 // finest cell takes the leaf's discharges and free surface (R-decode).  A tile
 // under one leaf brings the leaf's level with its list entry, so that it needs
 // no flags and one round of loads: three water columns on a flat bed at L=11
-// (134 MB) take 38 us, the last CTA's time advance included (48 us when every
-// tile's flags were formed first, by two thirds of the CTAs).
+// (134 MB) take 29 us, the last CTA's time advance included (48 us when every
+// tile's flags were formed first, by two thirds of the CTAs, and a lane's 32
+// bytes went out as two halves).
 template <typename T>
 __device__ __forceinline__ void decode_body(const DecodeArgs<T>& a, Blk B) {
     DevState* st = a.st;

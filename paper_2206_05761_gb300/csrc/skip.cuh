@@ -163,6 +163,9 @@ static __global__ void __launch_bounds__(256, 3) k_skip_encode(SkipArgs<T> a) {
         for (int n = E - 1; n >= Ls; --n) {
             const uint32_t cnt = 1u << (2 * (n - Ls));
             const bool first = n == E - 1;
+            const Thr<T>* const th = sth[n - Ls];
+            const bool zero = passes_thr(T(0), th[0].thr, th[0].thr4) || passes_thr(T(0), th[1].thr, th[1].thr4) ||
+                              passes_thr(T(0), th[2].thr, th[2].thr4);
 #pragma unroll 1
             for (uint32_t t0 = 0u; t0 < (first ? cnt : 32u); t0 += 32u) {   // warp-uniform rounds
                 const uint32_t t = t0 + lane;
@@ -186,7 +189,7 @@ static __global__ void __launch_bounds__(256, 3) k_skip_encode(SkipArgs<T> a) {
                         cch = (scl[wib][4 * t] | scl[wib][4 * t + 1] | scl[wib][4 * t + 2] | scl[wib][4 * t + 3]) != 0;
                     }
                     bool tf = false;
-                    parents_all<T, 3>(sth[n - Ls], c, sq, tf);
+                    parents_all<T, 3>(th, c, sq, tf, zero);
                     fh[lvl_off(n) + pc] = sq[0];
                     fqx[lvl_off(n) + pc] = sq[1];
                     fqy[lvl_off(n) + pc] = sq[2];
