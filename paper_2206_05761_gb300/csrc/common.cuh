@@ -127,21 +127,18 @@ __device__ __forceinline__ double from_obits(unsigned long long b) {
 }
 constexpr unsigned long long kInfBits = 0x7FF0000000000000ull;
 
+// Warp-wide min and max of a uint64 (every lane must call): of the high words,
+// then of the low words of the lanes that hold it, by the 32-bit reduction
+// instruction.
 __device__ __forceinline__ unsigned long long warp_min_u64(unsigned long long v) {
-#pragma unroll
-    for (int o = 16; o; o >>= 1) {
-        unsigned long long w = __shfl_xor_sync(0xffffffffu, v, o);
-        v = w < v ? w : v;
-    }
-    return v;
+    const uint32_t hi = (uint32_t)(v >> 32), mh = __reduce_min_sync(0xffffffffu, hi);
+    const uint32_t ml = __reduce_min_sync(0xffffffffu, hi == mh ? (uint32_t)v : 0xffffffffu);
+    return (unsigned long long)mh << 32 | ml;
 }
 __device__ __forceinline__ unsigned long long warp_max_u64(unsigned long long v) {
-#pragma unroll
-    for (int o = 16; o; o >>= 1) {
-        unsigned long long w = __shfl_xor_sync(0xffffffffu, v, o);
-        v = w > v ? w : v;
-    }
-    return v;
+    const uint32_t hi = (uint32_t)(v >> 32), mh = __reduce_max_sync(0xffffffffu, hi);
+    const uint32_t ml = __reduce_max_sync(0xffffffffu, hi == mh ? (uint32_t)v : 0u);
+    return (unsigned long long)mh << 32 | ml;
 }
 
 // Block-wide min (IS_MAX = false) or max of a uint64 followed by one
@@ -195,6 +192,45 @@ __device__ __forceinline__ void block_max3_u64(unsigned long long a, unsigned lo
             if (c) atomicMax(dst + 2, c);
         }
     }
+}
+
+// Block-wide max of five uint64 values, then one atomicMax each of those above
+// 0 into dst_a[0..2] and dst_b[0..1].  Every thread of the block must call it,
+// once.
+__device__ __forceinline__ void block_max5_u64(const unsigned long long (&v)[5], unsigned long long* dst_a,
+                                               unsigned long long* dst_b) {
+    __shared__ unsigned long long red5[8][5];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+#pragma unroll
+    for (int k = 0; k < 5; ++k) {
+        const unsigned long long m = warp_max_u64(v[k]);
+        if (lane == 0) red5[warp][k] = m;
+    }
+    __syncthreads();
+    if (threadIdx.x < 5u) {
+        const int nw = (blockDim.x + 31) >> 5;
+        unsigned long long m = 0ull;
+        for (int w = 0; w < nw; ++w) {
+            const unsigned long long x = red5[w][threadIdx.x];
+            m = x > m ? x : m;
+        }
+        if (m) atomicMax(threadIdx.x < 3u ? dst_a + threadIdx.x : dst_b + threadIdx.x - 3, m);
+    }
+}
+
+// A word read where the statement stands: the compiler neither sinks the load
+// below a branch nor merges it, so that several are on their way at once.  (An
+// ordinary load through L1: as volatile accesses, which go to L2, every warp's
+// read of the same line made a step 10 to 30 % longer.)
+__device__ __forceinline__ uint32_t now(const uint32_t* p) {
+    uint32_t v;
+    asm volatile("ld.global.u32 %0, [%1];" : "=r"(v) : "l"(p));
+    return v;
+}
+__device__ __forceinline__ uint8_t now(const uint8_t* p) {
+    uint32_t v;
+    asm volatile("ld.global.u8 %0, [%1];" : "=r"(v) : "l"(p));
+    return (uint8_t)v;
 }
 
 // Exclusive block scan of one uint32 per thread (blockDim <= 1024).

@@ -1459,13 +1459,18 @@ class EngineT final : public Engine {
         a.inflow_Q = iq_d_;
         a.inflow_n = it_.empty() ? 0 : (int)it_.size();
         a.L = L_;
-        a.eps = spec_.eps;
         a.cfl = spec_.cfl;
         a.dt_max = spec_.dt_max;
         a.lx = spec_.lx;
         a.ly = spec_.ly;
+        a.dxL = std::ldexp(spec_.lx, -L_);
+        a.dyL = std::ldexp(spec_.ly, -L_);
         a.g = spec_.g;
         a.manning_n = spec_.manning_n;
+        for (int n = 0; n < kMaxL; ++n) {
+            a.eps_n[n] = n < L_ ? std::ldexp(spec_.eps, n - L_) : 0.0;
+            a.epsf_n[n] = n < L_ ? std::ldexp((float)spec_.eps, n - L_) : 0.0f;
+        }
         return a;
     }
     // s_max (and dt when set_dt) from the finest fields of the current buffer

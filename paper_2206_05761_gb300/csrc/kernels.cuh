@@ -325,6 +325,33 @@ __device__ __forceinline__ void parent_coef(const Thr<T>& h, T c0, T c1, T c2, T
     tf = tf || passes_thr(dm, h.thr, h.thr4);
 }
 
+// The parts of parent_coef on their own: the parent (four equal children give
+// quarter(2 c + 2 c) = c), and its threshold decision.
+template <typename T>
+__device__ __forceinline__ T parent_value(T c0, T c1, T c2, T c3) { return quarter((c0 + c2) + (c1 + c3)); }
+__device__ __forceinline__ bool parent_flag(const Thr<double>& h, double c0, double c1, double c2, double c3) {
+    if (same4<double>(c0, c1, c2, c3)) return passes_thr(0.0, h.thr, h.thr4);
+    if (h.lo >= 0.0f) {
+        const float f0 = trunc_float(c0), f1 = trunc_float(c1), f2 = trunc_float(c2), f3 = trunc_float(c3);
+        const float af = f0 + f2, bf = f1 + f3, df = f0 - f2, ef = f1 - f3;
+        const float m = fmaxf(fmaxf(fabsf(df + ef), fabsf(af - bf)), fabsf(df - ef));
+        const float S = __fadd_ru(__fadd_ru(fabsf(f0), fabsf(f1)), __fadd_ru(fabsf(f2), fabsf(f3)));
+        const float E = __fadd_ru(__fmul_ru(S, 0x1p-20f), 0x1p-120f);
+        if (float_finite(m) && float_finite(E)) {
+            if (__fsub_rd(m, E) >= h.hi) return true;
+            if (__fadd_ru(m, E) < h.lo) return false;
+        }
+    }
+    const double a = c0 + c2, b = c1 + c3, d = c0 - c2, e = c1 - c3;
+    const double m4 = sel_max(sel_max(absval(d + e), absval(a - b)), absval(d - e));
+    return passes_thr(m4, h.thr, h.thr4);
+}
+__device__ __forceinline__ bool parent_flag(const Thr<float>& h, float c0, float c1, float c2, float c3) {
+    float s, dm;
+    haar4<float>(c0, c1, c2, c3, s, dm);
+    return passes_thr(dm, h.thr, h.thr4);
+}
+
 // The parents of all NF quantities of one cell and its threshold flag.  In
 // float64 the sums of every quantity come first (independent of one
 // another, so the FP64 pipe takes them back to back instead of one
@@ -593,12 +620,17 @@ __device__ __forceinline__ void encode_body(const EncodeArgs<T, NF>& a, int ls, 
 // resident to fill the FP64 pipe.
 template <typename T, int NF, int W, bool CG = false>
 __device__ __forceinline__ void encode_tile(const EncodeArgs<T, NF>& a, int ls, uint32_t tile) {
-    if (a.st && !a.st->active) return;
-    const int par = a.st ? (int)a.st->cur : 0;
-    // a tile known to hold only +0 encodes to +0 (as in encode_body)
     const bool quiet = a.zf[0] != nullptr && ls == a.L;
+    int par = 0;
+    if (a.st) {
+        // the state and the tile's marks in both buffers in one round of loads
+        const uint32_t active = now(&a.st->active), cur = now(&a.st->cur);
+        const uint8_t z0 = quiet ? now(a.zf[0] + tile) : (uint8_t)0, z1 = quiet ? now(a.zf[1] + tile) : (uint8_t)0;
+        par = (int)cur;
+        // a tile known to hold only +0 encodes to +0 (as in encode_body)
+        if (!active || (par ? z1 : z0)) return;
+    }
     uint8_t* const zfp = par ? a.zf[1] : a.zf[0];
-    if (quiet && zfp[tile]) return;
     constexpr uint32_t P1 = 256 / W, P2 = P1 / 4, P3 = P2 / 4;   // a warp's parents per level
     __shared__ T sv1[W][NF][P1], sv2[W][NF][P2], sv3[NF][16], sv4[NF][4];
     __shared__ Thr<T> sthr[W][5][NF];
@@ -675,15 +707,14 @@ __device__ __forceinline__ void encode_tile(const EncodeArgs<T, NF>& a, int ls, 
         if (t) atomicOr(a.Tb + word_off(n) + (first >> 5), t << (first & 31u));
         if (cl) atomicOr(a.Cb + word_off(n) + (first >> 5), cl << (first & 31u));
     };
-    // one level of n parents (a power of two): lane = (quantity, parent),
-    // children at v[q * stride + 4 i], results to out[q * ostride + i] and to
-    // the hierarchy from cell `first` on; returns the threshold bits
-    auto level = [&](int j, uint32_t n, const T* v, uint32_t stride, T* out, uint32_t ostride, uint32_t first) -> uint32_t {
-        uint32_t t = 0u;
+    // the values of one level of n parents (a power of two): lane = (quantity,
+    // parent), children at v[q * stride + 4 i], results to out[q * ostride + i]
+    // and to the hierarchy from cell `first` on.  The threshold decisions of
+    // the levels follow together, off the chain of the values.
+    auto values = [&](int j, uint32_t n, const T* v, uint32_t stride, T* out, uint32_t ostride, uint32_t first) {
 #pragma unroll 1
         for (uint32_t r = 0; r < n * NF; r += 32u) {
             const uint32_t id = r + lane, q = id / n, i = id & (n - 1u);
-            bool f = false;
             if (q < (uint32_t)NF) {
                 const T* x = v + q * stride + 4u * i;
                 T sp = T(0);
@@ -691,49 +722,94 @@ __device__ __forceinline__ void encode_tile(const EncodeArgs<T, NF>& a, int ls, 
 #pragma unroll
                     for (int k = 0; k < NF; ++k)
                         if (q == (uint32_t)k) sp = one[k];
-                    f = ((zbits >> ((j - 1) * NF + q)) & 1u) != 0u;
                 } else {
-                    parent_coef(sthr[w][j - 1][q], x[0], x[1], x[2], x[3], sp, f);
+                    sp = parent_value(x[0], x[1], x[2], x[3]);
                 }
                 quantity_ptr(a, par, q)[lvl_off(ls - j) + first + i] = sp;
                 out[q * ostride + i] = sp;
             }
-            uint32_t m = __ballot_sync(0xffffffffu, f);
-            for (uint32_t k = 0; k < 32u; k += n) t |= m >> k;
         }
         __syncwarp();
-        return t & ((1u << n) - 1u);
+    };
+    // whether the parent of x[0..3] passes its threshold in quantity q
+    auto flag = [&](int j, uint32_t q, const T* x) -> bool {
+        return same ? ((zbits >> ((j - 1) * NF + q)) & 1u) != 0u
+                    : parent_flag(sthr[w][j - 1][q], x[0], x[1], x[2], x[3]);
     };
     // the closure of n parents: their own flags or a closed child's
     auto close = [&](uint32_t n, uint32_t t, bool child) { return t | (__ballot_sync(0xffffffffu, child) & ((1u << n) - 1u)); };
-    const uint32_t T2 = level(2, P2, sv1[w][0], P1, sv2[w][0], P2, b * P2);
-    const uint32_t C2 = close(P2, T2, (((lane < 8u ? cw[0] : cw[1]) >> (4u * (lane & 7u))) & 0xFu) != 0u);
-    put(ls - 2, b * P2, T2, C2);
-    const uint32_t T3 = level(3, P3, sv2[w][0], P2, &sv3[0][w * P3], 16u, b * P3);
-    const uint32_t C3 = close(P3, T3, lane < P3 && ((C2 >> (4u * lane)) & 0xFu) != 0u);
-    put(ls - 3, b * P3, T3, C3);
-    uint32_t C4 = 0u;
-    if constexpr (W == 4) {
-        const uint32_t T4 = level(4, 1u, &sv3[0][w * 4u], 16u, &sv4[0][w], 4u, b);
-        C4 = (T4 | C3) ? 1u : 0u;
-        put(ls - 4, b, T4, C4);
+    values(2, P2, sv1[w][0], P1, sv2[w][0], P2, b * P2);
+    values(3, P3, sv2[w][0], P2, &sv3[0][w * P3], 16u, b * P3);
+    if constexpr (W == 4) values(4, 1u, &sv3[0][w * 4u], 16u, &sv4[0][w], 4u, b);
+    // the decisions: (level, quantity, parent) items over the lanes
+    constexpr uint32_t o3 = NF * P2, o4 = o3 + NF * P3, items = o4 + (W == 4 ? NF : 0);
+    unsigned long long fl = 0ull;
+#pragma unroll 1
+    for (uint32_t r = 0; r < items; r += 32u) {
+        const uint32_t id = r + lane;
+        bool f = false;
+        if (id < items) {
+            int j = 2;
+            uint32_t q = id / P2;
+            const T* x = sv1[w][0] + q * P1 + 4u * (id % P2);
+            if (id >= o4) {
+                j = 4;
+                q = id - o4;
+                x = sv3[0] + q * 16u + w * 4u;
+            } else if (id >= o3) {
+                j = 3;
+                q = (id - o3) / P3;
+                x = sv2[w][0] + q * P2 + 4u * ((id - o3) % P3);
+            }
+            f = flag(j, q, x);
+        }
+        fl |= (unsigned long long)__ballot_sync(0xffffffffu, f) << r;
     }
+    uint32_t T2 = 0u, T3 = 0u, T4 = 0u;
+#pragma unroll
+    for (uint32_t q = 0; q < (uint32_t)NF; ++q) {
+        T2 |= (uint32_t)(fl >> (q * P2));
+        T3 |= (uint32_t)(fl >> (o3 + q * P3));
+        if (W == 4) T4 |= (uint32_t)(fl >> (o4 + q)) & 1u;
+    }
+    T2 &= (1u << P2) - 1u;
+    T3 &= (1u << P3) - 1u;
+    const uint32_t C2 = close(P2, T2, (((lane < 8u ? cw[0] : cw[1]) >> (4u * (lane & 7u))) & 0xFu) != 0u);
+    const uint32_t C3 = close(P3, T3, lane < P3 && ((C2 >> (4u * lane)) & 0xFu) != 0u);
+    uint32_t C4 = (T4 | C3) ? 1u : 0u;
+    put(ls - 2, b * P2, T2, C2);
+    put(ls - 3, b * P3, T3, C3);
+    if (W == 4) put(ls - 4, b, T4, C4);
     if (lane == 0u) scl[w] = W == 4 ? C4 : C3;
     const int any = __syncthreads_or(nz ? 1 : 0);
     // all source values +0 => every coarser value written is +0
     if (quiet && threadIdx.x == 0) zfp[tile] = any ? 0 : 1;
     if (w != 0u) return;
     same = false;                            // the other warps' cells may hold other values
+    __shared__ T top[NF];
+    if constexpr (W == 8) values(4, 4u, sv3[0], 16u, sv4[0], 4u, tile * 4u);
+    values(5, 1u, sv4[0], 4u, top, 1u, tile);
+    constexpr uint32_t o5 = W == 8 ? 4u * NF : 0u;
+    bool f = false;
+    if (lane < o5 + NF) {
+        const bool five = lane >= o5;
+        const uint32_t q = five ? lane - o5 : lane >> 2;
+        f = flag(five ? 5 : 4, q, five ? sv4[0] + q * 4u : sv3[0] + q * 16u + 4u * (lane & 3u));
+    }
+    const uint32_t m = __ballot_sync(0xffffffffu, f);
+    const uint32_t T5 = (m >> o5) & ((1u << NF) - 1u) ? 1u : 0u;
     if constexpr (W == 4) {
         C4 = __ballot_sync(0xffffffffu, lane < 4u && scl[lane & 3u] != 0u);
     } else {
+        T4 = 0u;
+#pragma unroll
+        for (int q = 0; q < NF; ++q) T4 |= m >> (4 * q);
+        T4 &= 0xFu;
+        // (o5 bits hold the level-(ls-4) flags; the top's follow them)
         const uint32_t all = __ballot_sync(0xffffffffu, lane < 16u && ((scl[(lane >> 1) & 7u] >> (lane & 1u)) & 1u) != 0u);
-        const uint32_t T4 = level(4, 4u, sv3[0], 16u, sv4[0], 4u, tile * 4u);
         C4 = close(4u, T4, lane < 4u && ((all >> (4u * lane)) & 0xFu) != 0u);
         put(ls - 4, tile * 4u, T4, C4);
     }
-    __shared__ T top[NF];
-    const uint32_t T5 = level(5, 1u, sv4[0], 4u, top, 1u, tile);
     put(ls - 5, tile, T5, (T5 | C4) ? 1u : 0u);
 }
 
@@ -1736,13 +1812,14 @@ template <typename T>
 __device__ __forceinline__ void cell_update_faces(const Phys<T>& P, T rx, T ry, T fk, const Cell<T>& C,
                                                   const T FW[3], const T FE[3], const T GS[3], const T GN[3],
                                                   T hW_R, T hE_L, T hS_R, T hN_L, bool inlet, T dh, T out[3],
-                                                  T* rh_out = nullptr);
+                                                  T sp[2]);
 
-// New (h, qx, qy) of a cell of size dx x dy: rx = dt/dx, ry = dt/dy.
+// New (h, qx, qy) of a cell of size dx x dy: rx = dt/dx, ry = dt/dy; sp (float64)
+// its CFL speeds |u|+sqrt(gh), |v|+sqrt(gh), 0 where it is dry.
 template <typename T>
 __device__ __forceinline__ void cell_update(const Phys<T>& P, T rx, T ry, T fk, const Cell<T>& C,
                                             const Cell<T>& W, const Cell<T>& E, const Cell<T>& S,
-                                            const Cell<T>& N, bool inlet, T dh, T out[3]) {
+                                            const Cell<T>& N, bool inlet, T dh, T out[3], T sp[2]) {
     const T g = P.g, hg = P.hg, tol = P.tol;
     T FW[3], FE[3], GS[3], GN[3];
     T hW_R, hE_L, hS_R, hN_L, dummy;
@@ -1770,7 +1847,7 @@ __device__ __forceinline__ void cell_update(const Phys<T>& P, T rx, T ry, T fk, 
         hll_face(g, hg, tol, eC, C.z, vC, uC, eta_of(N.h, N.z), N.z, vN, uN, ok && cell_window(N.h, N.z, uN, vN), GN,
                  hN_L, dummy);
     }
-    cell_update_faces(P, rx, ry, fk, C, FW, FE, GS, GN, hW_R, hE_L, hS_R, hN_L, inlet, dh, out);
+    cell_update_faces(P, rx, ry, fk, C, FW, FE, GS, GN, hW_R, hE_L, hS_R, hN_L, inlet, dh, out, sp);
 }
 
 // The friction term's per-step factor ((dt * g) * n) * n (formed once per
@@ -1779,70 +1856,166 @@ template <typename T> __device__ __forceinline__ T fric_k_of(const DevState* st)
 template <> __device__ __forceinline__ double fric_k_of<double>(const DevState* st) { return st->fric_k; }
 template <> __device__ __forceinline__ float fric_k_of<float>(const DevState* st) { return st->fric_kf; }
 
-// h^(-1/3) of a double h whose float truncation is a normal number: the
-// float inverse cube root as the seed, then one Newton step for
-// f(r) = r^-3 - h, r <- r + r (1 - h r^3) / 3, which squares the seed's
-// relative error (below 2^-21) up to a factor 2: about 2^-41 in all, where
-// the double cube root and a division cost some 20 FP64 additions' worth of
-// the FP64 pipe.  Not correctly rounded; the friction term is the one use.
-__device__ __forceinline__ double rcbrt_newton(float hf, double h) {
+// The arithmetic of the update.  PlainOps: the operations as written (float64
+// on the FP64 pipe).  IntOps (float64): products, roots and reciprocals in
+// integer instructions without a branch; an operation whose operands are out of
+// its range sets `bad`, and the caller forms the whole update again with
+// PlainOps.  With a branch around every operation's rare case instead, the
+// operations of a cell cannot overlap: 32 steps of the 4096 x 4096 flood took
+// 1.7 % longer, of 16 basins of 512 x 512 1.1 %, of 2048 x 2048 columns 0.7 %.
+template <typename T>
+struct PlainOps {
+    bool bad = false;
+    __device__ __forceinline__ T mul(T a, T b) { return a * b; }
+    __device__ __forceinline__ T root(T x) { return sqrt(x); }
+    __device__ __forceinline__ T recip(T x) { return T(1) / x; }
+};
+struct IntOps {
+    bool bad = false;
+    __device__ __forceinline__ double mul(double a, double b) {
+        uint32_t al, ah, bl, bh;
+        d_split(a, al, ah);
+        d_split(b, bl, bh);
+        const bool na = ((ah + 0x00100000u) & 0x7FE00000u) != 0u, nb = ((bh + 0x00100000u) & 0x7FE00000u) != 0u;
+        const bool za = ((ah & 0x7FFFFFFFu) | al) == 0u, zb = ((bh & 0x7FFFFFFFu) | bl) == 0u;
+        const bool in = (ah & 0x7FF00000u) + (bh & 0x7FF00000u) - (1024u << 20) < (2044u << 20);
+        bad = bad || !((na || za) && (nb || zb) && (in || za || zb));
+        return d_join(mul_bits<true>(al, ah, bl, bh));
+    }
+    __device__ __forceinline__ double root(double x) {
+        uint32_t lo, hi;
+        d_split(x, lo, hi);
+        const bool zero = (lo | hi) == 0u;
+        bad = bad || !(sqrt_in_range(hi) || zero);
+        float y;
+        asm("rsqrt.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(__uint_as_float(sqrt_seed_arg(lo, hi))));
+        const double r = d_join(sqrt_bits(lo, hi, __float_as_uint(y)));
+        return zero ? x : r;
+    }
+    __device__ __forceinline__ double recip(double x) {
+        uint32_t lo, hi;
+        d_split(x, lo, hi);
+        bad = bad || !rcp_in_range(hi);
+        float y;
+        asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(__uint_as_float(rcp_seed_arg(lo, hi))));
+        return d_join(rcp_bits(lo, hi, __float_as_uint(y)));
+    }
+};
+
+// x / (h cbrt(h)) = x h^(-4/3) of Manning's friction term for a wet cell
+// (h >= tol > 0, rh = 1/h).  float64: x (1/h) h^(-1/3), with h^(-1/3) from the
+// float inverse cube root of h's float truncation as the seed, then one Newton
+// step for f(r) = r^-3 - h, r <- r + r (1 - h r^3) / 3, which squares the seed's
+// relative error (below 2^-21) up to a factor 2: about 2^-41 in all (the
+// friction factor 1 + this term then within 2^-40 (D - 1)/D), where the double
+// cube root and a division cost some 20 FP64 additions' worth of the FP64 pipe.
+// Not correctly rounded.  Outside the float range, and in float32, the quotient
+// as written.
+template <class Ops>
+__device__ __forceinline__ double friction_newton(Ops& o, double x, double h, double rh, float hf) {
     const float rf = rcbrtf(hf);
     // the float widened to a double by integer operations (exact)
     const uint32_t b = (uint32_t)__float_as_int(rf);
     const long long e = (long long)((b >> 23) & 0xFFu) - 127 + 1023;
     const double r = dval((e << 52) | ((long long)(b & 0x7FFFFFu) << 29));
-    const double r3 = prod(prod(r, r), r);
+    const double r3 = o.mul(o.mul(r, r), r);
     const double d = __fma_rn(-h, r3, 1.0);
-    return __fma_rn(prod(r, d), 1.0 / 3.0, r);
+    return o.mul(o.mul(x, rh), __fma_rn(o.mul(r, d), 1.0 / 3.0, r));
 }
-
-// x / (h cbrt(h)) = x h^(-4/3) of Manning's friction term for a wet cell
-// (h >= tol > 0, rh = 1/h).  float64: x (1/h) h^(-1/3) with the Newton
-// inverse cube root, within some 2^-40 relative of the quotient as written
-// (the friction factor 1 + this term then within 2^-40 (D - 1)/D); outside
-// the float range the quotient as written.  float32: the quotient as written.
-__device__ __forceinline__ double friction_term(double x, double h, double rh) {
+__device__ __forceinline__ double friction_term(PlainOps<double>& o, double x, double h, double rh) {
     const float hf = trunc_float(h);
     const uint32_t eb = ((uint32_t)__float_as_int(hf) >> 23) & 0xFFu;
-    if (eb != 0u && eb != 0xFFu) return prod(prod(x, rh), rcbrt_newton(hf, h));
+    if (eb != 0u && eb != 0xFFu) return friction_newton(o, x, h, rh, hf);
     return x / (h * cbrt(h));
 }
-__device__ __forceinline__ float friction_term(float x, float h, float /*rh*/) { return x / (h * cbrtf(h)); }
+__device__ __forceinline__ double friction_term(IntOps& o, double x, double h, double rh) {
+    const float hf = trunc_float(h);
+    const uint32_t eb = ((uint32_t)__float_as_int(hf) >> 23) & 0xFFu;
+    o.bad = o.bad || eb == 0u || eb == 0xFFu;
+    return friction_newton(o, x, h, rh, hf);
+}
+__device__ __forceinline__ float friction_term(PlainOps<float>&, float x, float h, float /*rh*/) { return x / (h * cbrtf(h)); }
 
-// The update from the four face fluxes and the squares of the cell's own
-// reconstructed depths at them (hW2, hE2, hS2, hN2: the bed source term's
-// face values).  rh_out (if given) receives 1/h of the new depth when the
-// friction step formed it, else 0.
-template <typename T>
-__device__ __forceinline__ void cell_update_faces_sq(const Phys<T>& P, T rx, T ry, T fk, const Cell<T>& C,
-                                                     const T FW[3], const T FE[3], const T GS[3], const T GN[3],
-                                                     T hW2, T hE2, T hS2, T hN2, bool inlet, T dh, T out[3],
-                                                     T* rh_out = nullptr) {
-    if (rh_out) *rh_out = T(0);
+template <typename T, class Ops>
+__device__ __forceinline__ void cell_update_ops(Ops& o, const Phys<T>& P, T rx, T ry, T fk, const Cell<T>& C,
+                                                const T FW[3], const T FE[3], const T GS[3], const T GN[3], T hW2,
+                                                T hE2, T hS2, T hN2, bool inlet, T dh, T out[3], T sp[2]) {
     const T hg = P.hg, tol = P.tol;
-    const T bx = prod(hg, hW2 - hE2);
-    const T by = prod(hg, hS2 - hN2);
-    T h = C.h - prod(rx, FE[0] - FW[0]) - prod(ry, GN[0] - GS[0]);
-    T qx = C.qx - prod(rx, (FE[1] - FW[1]) + bx) - prod(ry, GN[2] - GS[2]);
-    T qy = C.qy - prod(rx, FE[2] - FW[2]) - prod(ry, (GN[1] - GS[1]) + by);
+    const T bx = o.mul(hg, hW2 - hE2);
+    const T by = o.mul(hg, hS2 - hN2);
+    T h = C.h - o.mul(rx, FE[0] - FW[0]) - o.mul(ry, GN[0] - GS[0]);
+    T qx = C.qx - o.mul(rx, (FE[1] - FW[1]) + bx) - o.mul(ry, GN[2] - GS[2]);
+    T qy = C.qy - o.mul(rx, FE[2] - FW[2]) - o.mul(ry, (GN[1] - GS[1]) + by);
     if (inlet) h = h + dh;
     h = gt_zero(h) ? h : T(0);
+    sp[0] = sp[1] = T(0);
     if (!ge_nonneg(h, tol)) {                           // h < tol (tol > 0)
         qx = T(0);
         qy = T(0);
-    } else if (gt_zero(P.nM)) {
-        const T rh = recip(h);
-        if (rh_out) *rh_out = rh;
-        const T u = prod(qx, rh), v = prod(qy, rh);
-        const T speed = root(prod(u, u) + prod(v, v));
-        const T D = T(1) + friction_term(prod(fk, speed), h, rh);
-        const T rD = recip(D);
-        qx = prod(qx, rD);
-        qy = prod(qy, rD);
+    } else if (sizeof(T) == 8 || gt_zero(P.nM)) {
+        const T rh = o.recip(h);
+        if (gt_zero(P.nM)) {
+            const T u = o.mul(qx, rh), v = o.mul(qy, rh);
+            const T speed = o.root(o.mul(u, u) + o.mul(v, v));
+            const T D = T(1) + friction_term(o, o.mul(fk, speed), h, rh);
+            const T rD = o.recip(D);
+            qx = o.mul(qx, rD);
+            qy = o.mul(qy, rD);
+        }
+        if (sizeof(T) == 8) {
+            // the CFL speeds (the divisions are formed once per step from
+            // their maxima, finish_body); the operations of cfl_bound
+            const T aa = o.root(o.mul(P.g, h));
+            sp[0] = absval(o.mul(qx, rh)) + aa;
+            sp[1] = absval(o.mul(qy, rh)) + aa;
+        }
     }
     out[0] = h;
     out[1] = qx;
     out[2] = qy;
+}
+// (in: the operands of cell_update_ops in its order)
+static __device__ __noinline__ void cell_update_rare(const Phys<double>& P, const double* in, bool inlet, double* res) {
+    PlainOps<double> o;
+    Cell<double> C;
+    C.h = in[3];
+    C.qx = in[4];
+    C.qy = in[5];
+    C.z = 0.0;
+    cell_update_ops<double>(o, P, in[0], in[1], in[2], C, in + 6, in + 9, in + 12, in + 15, in[18], in[19], in[20],
+                            in[21], inlet, in[22], res, res + 3);
+}
+
+// The update from the four face fluxes and the squares of the cell's own
+// reconstructed depths at them (hW2, hE2, hS2, hN2: the bed source term's
+// face values).
+__device__ __forceinline__ void cell_update_faces_sq(const Phys<double>& P, double rx, double ry, double fk,
+                                                     const Cell<double>& C, const double FW[3], const double FE[3],
+                                                     const double GS[3], const double GN[3], double hW2, double hE2,
+                                                     double hS2, double hN2, bool inlet, double dh, double out[3],
+                                                     double sp[2]) {
+    IntOps o;
+    cell_update_ops<double>(o, P, rx, ry, fk, C, FW, FE, GS, GN, hW2, hE2, hS2, hN2, inlet, dh, out, sp);
+    if (o.bad) {
+        const double in[23] = {rx,    ry,    fk,    C.h,   C.qx,  C.qy,  FW[0], FW[1], FW[2], FE[0], FE[1], FE[2],
+                               GS[0], GS[1], GS[2], GN[0], GN[1], GN[2], hW2,   hE2,   hS2,   hN2,   dh};
+        double res[5];
+        const Phys<double> Q = P;
+        cell_update_rare(Q, in, inlet, res);
+        out[0] = res[0];
+        out[1] = res[1];
+        out[2] = res[2];
+        sp[0] = res[3];
+        sp[1] = res[4];
+    }
+}
+__device__ __forceinline__ void cell_update_faces_sq(const Phys<float>& P, float rx, float ry, float fk,
+                                                     const Cell<float>& C, const float FW[3], const float FE[3],
+                                                     const float GS[3], const float GN[3], float hW2, float hE2,
+                                                     float hS2, float hN2, bool inlet, float dh, float out[3],
+                                                     float sp[2]) {
+    PlainOps<float> o;
+    cell_update_ops<float>(o, P, rx, ry, fk, C, FW, FE, GS, GN, hW2, hE2, hS2, hN2, inlet, dh, out, sp);
 }
 
 // The update of cell_update from its four face fluxes and its own
@@ -1851,10 +2024,9 @@ template <typename T>
 __device__ __forceinline__ void cell_update_faces(const Phys<T>& P, T rx, T ry, T fk, const Cell<T>& C,
                                                   const T FW[3], const T FE[3], const T GS[3], const T GN[3],
                                                   T hW_R, T hE_L, T hS_R, T hN_L, bool inlet, T dh, T out[3],
-                                                  T* rh_out) {
-    cell_update_faces_sq(P, rx, ry, fk, C, FW, FE, GS, GN, prod(hW_R, hW_R), prod(hE_L, hE_L),
-                         prod(hS_R, hS_R), prod(hN_L, hN_L),
-                         inlet, dh, out, rh_out);
+                                                  T sp[2]) {
+    cell_update_faces_sq(P, rx, ry, fk, C, FW, FE, GS, GN, prod(hW_R, hW_R), prod(hE_L, hE_L), prod(hS_R, hS_R),
+                         prod(hN_L, hN_L), inlet, dh, out, sp);
 }
 
 // CFL bound of an updated cell: min(dx/(|u|+a), dy/(|v|+a)), +inf if dry
@@ -1877,8 +2049,11 @@ enum : int {
     kFaceN = 9,          // north face, as the east one
     kFaceW = 14,         // west face where it is not shared: F0, F1 | F2, its own depth squared
     kFaceS = 18,         // south face, as the west one
-    kFaceArrays = 22
+    kLeafWS = 22,        // queue slots of the west and south neighbours, kShared set, or the leaf's own
+                         // (two uint32)
+    kFaceArrays = 24
 };
+constexpr uint32_t kShared = 0x80000000u;
 // A leaf's stamp: (epoch + 1) << 32 | queue slot, with kUnsafe set where the
 // leaf is out of the window of hll_flux_mixed.
 constexpr uint32_t kUnsafe = 0x80000000u;
@@ -1889,6 +2064,10 @@ template <> struct Pair2<float> { typedef float2 V; };
 template <typename T>
 __device__ __forceinline__ typename Pair2<T>::V* pair_at(T* face, size_t cap, int k, uint32_t w) {
     return reinterpret_cast<typename Pair2<T>::V*>(face + k * cap) + w;
+}
+template <typename T>
+__device__ __forceinline__ uint32_t* slots_at(T* face, size_t cap, uint32_t w) {
+    return reinterpret_cast<uint32_t*>(face + kLeafWS * cap) + 2 * (size_t)w;
 }
 template <typename T>
 __device__ __forceinline__ typename Pair2<T>::V make_pair2(T a, T b) {
@@ -2079,16 +2258,16 @@ __device__ __forceinline__ void dry_finish(const StepArgs<T>& a, DevState* st, T
 template <typename T>
 __device__ __forceinline__ void fv1_dry_body(const StepArgs<T>& a, Blk B) {
     DevState* st = a.st;
-    if (!st->active) return;
-    const int par = (int)st->cur, nxt = par ^ 1;
-    const uint32_t M = st->M;
+    const uint32_t active = now(&st->active), M = now(&st->M), cur = now(&st->cur), epoch = now(&st->epoch);
+    if (!active) return;
+    const int par = (int)cur, nxt = par ^ 1;
     const T* __restrict__ hsrc = par ? a.f[1][0] : a.f[0][0];
     CellSrc<T> src;
     src.h = hsrc;
     src.qx = par ? a.f[1][1] : a.f[0][1];
     src.qy = par ? a.f[1][2] : a.f[0][2];
     src.z = a.z;
-    const unsigned long long stamp = (unsigned long long)(st->epoch + 1u) << 32;
+    const unsigned long long stamp = (unsigned long long)(epoch + 1u) << 32;
     T* const oh = nxt ? a.f[1][0] : a.f[0][0];
     T* const oqx = nxt ? a.f[1][1] : a.f[0][1];
     T* const oqy = nxt ? a.f[1][2] : a.f[0][2];
@@ -2122,21 +2301,13 @@ static __global__ void __launch_bounds__(256) k_fv1_dry(StepArgs<T> a) {
 template <typename T>
 __device__ __forceinline__ void wet_leaf_store(const StepArgs<T>& a, DevState* st, const T* z, T* oh, T* oqx,
                                                T* oqy, int n, uint32_t code, uint64_t iC, const Cell<T>& C,
-                                               const T out[3], unsigned long long& rmin, unsigned long long& mh,
-                                               unsigned long long& mqx, unsigned long long& mqy,
-                                               unsigned long long* spd = nullptr, T rh_known = T(0)) {
-    if (sizeof(T) == 8 && spd != nullptr) {
-        // float64: the CFL speeds of the leaf (the divisions are formed once
-        // per step from their maxima, finish_body); the same operations as
-        // cfl_bound up to the division, reusing the friction step's 1/h
-        if (ge_nonneg(out[0], a.P.tol)) {
-            const T rh = is_zero(rh_known) ? recip(out[0]) : rh_known;
-            const T u = absval(prod(out[1], rh)), v = absval(prod(out[2], rh));
-            const T aa = root(prod(a.P.g, out[0]));
-            const unsigned long long bx = abs_obits(u + aa), by = abs_obits(v + aa);
-            spd[0] = bx > spd[0] ? bx : spd[0];
-            spd[1] = by > spd[1] ? by : spd[1];
-        }
+                                               const T out[3], const T sp[2], unsigned long long& rmin,
+                                               unsigned long long& mh, unsigned long long& mqx,
+                                               unsigned long long& mqy, unsigned long long* spd) {
+    if (sizeof(T) == 8) {
+        const unsigned long long bx = abs_obits(sp[0]), by = abs_obits(sp[1]);
+        spd[0] = bx > spd[0] ? bx : spd[0];
+        spd[1] = by > spd[1] ? by : spd[1];
     } else {
         const T r = cfl_bound(a.P, out[0], out[1], out[2]);
         const unsigned long long rb = obits((double)r);
@@ -2234,13 +2405,12 @@ __device__ __forceinline__ void fv1_wet_body(const StepArgs<T>& a, Blk B) {
             const T dxn = a.lx * inv2n, dyn = a.ly * inv2n;
             dh = (Qdt * frac) / (dxn * dyn);
         }
-        T out[3];
-        cell_update(a.P, rx, ry, fk, C, W, E, S, N, inlet, dh, out);
-        wet_leaf_store(a, st, src.z, oh, oqx, oqy, n, code, iC, C, out, rmin, mh, mqx, mqy, spd);
+        T out[3], sp[2];
+        cell_update(a.P, rx, ry, fk, C, W, E, S, N, inlet, dh, out, sp);
+        wet_leaf_store(a, st, src.z, oh, oqx, oqy, n, code, iC, C, out, sp, rmin, mh, mqx, mqy, spd);
     }
-    block_atomic_u64<false>(rmin, &st->rmin_bits);
-    block_max3_u64(mh, mqx, mqy, st->max_bits);
-    block_max3_u64(spd[0], spd[1], 0ull, st->speed_bits);
+    if (sizeof(T) != 8) block_atomic_u64<false>(rmin, &st->rmin_bits);   // (float64: the speeds)
+    block_max5_u64({mh, mqx, mqy, spd[0], spd[1]}, st->max_bits, st->speed_bits);
 }
 template <typename T>
 static __global__ void __launch_bounds__(256) k_fv1_wet(StepArgs<T> a) {
@@ -2397,13 +2567,12 @@ __device__ __forceinline__ void fv1_match_body(const StepArgs<T>& a, Blk B) {
             const T dxn = a.lx * inv2n, dyn = a.ly * inv2n;
             dh = (Qdt * frac) / (dxn * dyn);
         }
-        T out[3], rh;
-        cell_update_faces_sq(a.P, rx, ry, fk, C, FW, FE, GS, GN, w2, e2, s2, n2, inlet, dh, out, &rh);
-        wet_leaf_store(a, st, src.z, oh, oqx, oqy, n, code, iC, C, out, rmin, mh, mqx, mqy, spd, rh);
+        T out[3], sp[2];
+        cell_update_faces_sq(a.P, rx, ry, fk, C, FW, FE, GS, GN, w2, e2, s2, n2, inlet, dh, out, sp);
+        wet_leaf_store(a, st, src.z, oh, oqx, oqy, n, code, iC, C, out, sp, rmin, mh, mqx, mqy, spd);
     }
-    block_atomic_u64<false>(rmin, &st->rmin_bits);
-    block_max3_u64(mh, mqx, mqy, st->max_bits);
-    block_max3_u64(spd[0], spd[1], 0ull, st->speed_bits);
+    if (sizeof(T) != 8) block_atomic_u64<false>(rmin, &st->rmin_bits);   // (float64: the speeds)
+    block_max5_u64({mh, mqx, mqy, spd[0], spd[1]}, st->max_bits, st->speed_bits);
 }
 template <typename T>
 static __global__ void __launch_bounds__(256) k_fv1_match(StepArgs<T> a) {
@@ -2520,19 +2689,19 @@ __device__ __forceinline__ void queued_face(const StepArgs<T>& a, const CellSrc<
 template <typename T, bool FM = false>
 __device__ __forceinline__ void fv1_faces_body(const StepArgs<T>& a, Blk B) {
     DevState* st = a.st;
-    if (!st->active) return;
-    const uint32_t nw = st->nwet, nq = nw < a.fcap ? nw : a.fcap;
+    const uint32_t active = now(&st->active), nw = now(&st->nwet), cur = now(&st->cur), tag = now(&st->epoch) + 1u;
+    if (!active) return;
+    const uint32_t nq = nw < a.fcap ? nw : a.fcap;
     const uint32_t lane = threadIdx.x & 31u, warp = threadIdx.x >> 5, wpb = blockDim.x >> 5;
     const uint32_t warps = B.n * wpb;
     const uint32_t per = nq < 32u * warps ? 16u : 32u;
     const uint32_t below = (1u << lane) - 1u;
-    const int par = (int)st->cur;
+    const int par = (int)cur;
     CellSrc<T> src;
     src.h = par ? a.f[1][0] : a.f[0][0];
     src.qx = par ? a.f[1][1] : a.f[0][1];
     src.qy = par ? a.f[1][2] : a.f[0][2];
     src.z = a.z;
-    const uint32_t tag = st->epoch + 1u;
     const bool ok = const_window(a.P.g, a.P.tol);
     __shared__ uint8_t lists[8][64];              // (blocks of up to 8 warps)
     uint8_t* const list = lists[warp];
@@ -2556,7 +2725,11 @@ __device__ __forceinline__ void fv1_faces_body(const StepArgs<T>& a, Blk B) {
             if (on) d = axis_probe(a.wet[base + l], s >= 2);
             if (t0 < 2u * per) {
                 // the face opposite to this lane's: shared by a queued neighbour?
-                const bool miss = on && (d.endM || (uint32_t)(__ldg(a.mark + d.iM) >> 32) != tag);
+                const unsigned long long mm = on && !d.endM ? __ldg(a.mark + d.iM) : 0ull;
+                const bool miss = on && (uint32_t)(mm >> 32) != tag;
+                if (on)
+                    slots_at(a.face, a.fcap, base + l)[s == 1 ? 0 : 1] =
+                        miss ? base + l : ((uint32_t)mm & ~kUnsafe) | kShared;
                 const uint32_t m = __ballot_sync(0xffffffffu, miss);
                 if (miss) list[n + __popc(m & below)] = (uint8_t)(s == 1 ? l : l | 32u);
                 n += __popc(m);
@@ -2575,10 +2748,10 @@ static __global__ void __launch_bounds__(128, 8) k_fv1_faces(StepArgs<T> a) {
 template <typename T>
 __device__ __forceinline__ void fv1_update_body(const StepArgs<T>& a, Blk B) {
     DevState* st = a.st;
-    if (!st->active) return;
-    const uint32_t nw = st->nwet, nq = nw < a.fcap ? nw : a.fcap;
-    if (B.id * blockDim.x >= nq) return;          // whole block idle
-    const int par = (int)st->cur, nxt = par ^ 1;
+    const uint32_t active = now(&st->active), nw = now(&st->nwet), cur = now(&st->cur);
+    const uint32_t nq = nw < a.fcap ? nw : a.fcap;
+    if (!active || B.id * blockDim.x >= nq) return;          // whole block idle
+    const int par = (int)cur, nxt = par ^ 1;
     const T fk = fric_k_of<T>(st);
     const T rx0 = rx0_of<T>(st), ry0 = ry0_of<T>(st);
     const T Qdt = (T)st->Qdt;
@@ -2590,16 +2763,17 @@ __device__ __forceinline__ void fv1_update_body(const StepArgs<T>& a, Blk B) {
     T* const oh = nxt ? a.f[1][0] : a.f[0][0];
     T* const oqx = nxt ? a.f[1][1] : a.f[0][1];
     T* const oqy = nxt ? a.f[1][2] : a.f[0][2];
-    const uint32_t tag = st->epoch + 1u;
     const size_t cap = a.fcap;
     unsigned long long rmin = kInfBits, mh = 0, mqx = 0, mqy = 0, spd[2] = {0ull, 0ull};
     for (uint32_t w = B.id * blockDim.x + threadIdx.x; w < nq; w += B.n * blockDim.x) {
-        const DryProbe d = dry_probe(a.wet[w]);
-        const int n = d.n;
+        const uint32_t pk = a.wet[w];
+        const uint2 ws = *reinterpret_cast<const uint2*>(slots_at(a.face, cap, w));
+        const int n = (int)(pk >> kLeafShift);
+        const uint32_t code = pk & kCodeMask;
+        const uint64_t iC = lvl_off(n) + code;
         // the west and south faces: the queued neighbour's, or the leaf's own
-        const unsigned long long mW = __ldg(a.mark + d.iW), mS = __ldg(a.mark + d.iS);
-        const bool sW = d.iW != d.iC && (uint32_t)(mW >> 32) == tag, sS = d.iS != d.iC && (uint32_t)(mS >> 32) == tag;
-        const uint32_t wW = sW ? (uint32_t)mW & ~kUnsafe : w, wS = sS ? (uint32_t)mS & ~kUnsafe : w;
+        const bool sW = (ws.x & kShared) != 0u, sS = (ws.y & kShared) != 0u;
+        const uint32_t wW = ws.x & ~kShared, wS = ws.y & ~kShared;
         const typename Pair2<T>::V e0 = *pair_at(a.face, cap, kFaceE, w), e1 = *pair_at(a.face, cap, kFaceE + 2, w);
         const typename Pair2<T>::V n0 = *pair_at(a.face, cap, kFaceN, w), n1 = *pair_at(a.face, cap, kFaceN + 2, w);
         const int kW = sW ? kFaceE : kFaceW, kS = sS ? kFaceN : kFaceS;
@@ -2610,16 +2784,16 @@ __device__ __forceinline__ void fv1_update_body(const StepArgs<T>& a, Blk B) {
         if (sW) hW2 = a.face[(kFaceE + 4) * cap + wW];
         if (sS) hS2 = a.face[(kFaceN + 4) * cap + wS];
         Cell<T> C;
-        C.h = __ldg(src.h + d.iC);
-        C.qx = __ldg(src.qx + d.iC);
-        C.qy = __ldg(src.qy + d.iC);
+        C.h = __ldg(src.h + iC);
+        C.qx = __ldg(src.qx + iC);
+        C.qy = __ldg(src.qy + iC);
         const T FE[3] = {e0.x, e0.y, e1.x}, hE2 = e1.y;
         const T GN[3] = {n0.x, n0.y, n1.x}, hN2 = n1.y;
         const T FW[3] = {w0.x, w0.y, w1.x};
         const T GS[3] = {s0.x, s0.y, s1.x};
         const T rx = mul_pow2(rx0, n), ry = mul_pow2(ry0, n);   // rx0 * 2^n, exact
         int64_t lo = 0, hi = 0;
-        const bool inlet = a.inflow_side >= 0 && inlet_range(a, n, compact16(d.code), compact16(d.code >> 1),
+        const bool inlet = a.inflow_side >= 0 && inlet_range(a, n, compact16(code), compact16(code >> 1),
                                                              (1u << n) - 1u, lo, hi);
         T dh = T(0);
         if (inlet) {
@@ -2629,13 +2803,12 @@ __device__ __forceinline__ void fv1_update_body(const StepArgs<T>& a, Blk B) {
             const T dxn = a.lx * inv2n, dyn = a.ly * inv2n;
             dh = (Qdt * frac) / (dxn * dyn);
         }
-        T out[3], rh;
-        cell_update_faces_sq(a.P, rx, ry, fk, C, FW, FE, GS, GN, hW2, hE2, hS2, hN2, inlet, dh, out, &rh);
-        wet_leaf_store(a, st, src.z, oh, oqx, oqy, n, d.code, d.iC, C, out, rmin, mh, mqx, mqy, spd, rh);
+        T out[3], sp[2];
+        cell_update_faces_sq(a.P, rx, ry, fk, C, FW, FE, GS, GN, hW2, hE2, hS2, hN2, inlet, dh, out, sp);
+        wet_leaf_store(a, st, src.z, oh, oqx, oqy, n, code, iC, C, out, sp, rmin, mh, mqx, mqy, spd);
     }
-    block_atomic_u64<false>(rmin, &st->rmin_bits);
-    block_max3_u64(mh, mqx, mqy, st->max_bits);
-    block_max3_u64(spd[0], spd[1], 0ull, st->speed_bits);
+    if (sizeof(T) != 8) block_atomic_u64<false>(rmin, &st->rmin_bits);   // (float64: the speeds)
+    block_max5_u64({mh, mqx, mqy, spd[0], spd[1]}, st->max_bits, st->speed_bits);
 }
 // 64 us for 1 M leaves (uniform FV1, L=10; 116 us with its products on the
 // FP64 pipe and the unshared faces formed here): the FP64 pipe's 19 sums a leaf
@@ -2687,12 +2860,11 @@ struct DecodeArgs {
 template <typename T>
 __device__ __forceinline__ void decode_body(const DecodeArgs<T>& a, Blk B) {
     DevState* st = a.st;
-    // the state is read through L2 only: k_decode_finish's last CTA reads
-    // what the other CTAs' atomics wrote and must not find stale L1 lines
-    if (!__ldcg(&st->active)) return;
-    const uint32_t nd = __ldcg(&st->ndec);
-    if (B.id >= nd) return;                   // whole block idle
-    const int nxt = (int)__ldcg(&st->cur) ^ 1;
+    // (words this kernel changes only in its last CTA's finish, which reads the
+    // state through L2: every warp going there for them would queue on one line)
+    const uint32_t active = now(&st->active), nd = now(&st->ndec), cur = now(&st->cur);
+    if (!active || B.id >= nd) return;        // whole block idle
+    const int nxt = (int)cur ^ 1;
     __shared__ TileBits tb;
     T* const fh = nxt ? a.f[1][0] : a.f[0][0];
     T* const fqx = nxt ? a.f[1][1] : a.f[0][1];
@@ -2762,8 +2934,10 @@ struct FinishArgs {
     const double* inflow_Q;
     int inflow_n;
     int L;
-    double eps, cfl, dt_max, lx, ly;
+    double cfl, dt_max, lx, ly, dxL, dyL;  // dxL, dyL: finest spacings
     double g, manning_n;
+    double eps_n[kMaxL];                   // eps 2^(n-L), and in float arithmetic
+    float epsf_n[kMaxL];
 };
 
 __device__ inline double inflow_Q(const FinishArgs& a, double t) {
@@ -2781,34 +2955,45 @@ __device__ inline double inflow_Q(const FinishArgs& a, double t) {
 // Called by every thread of a one-block launch after s_max is final; the
 // (level, quantity) thresholds are spread over the threads.
 // 4 thr for passes_thr when the comparison against it is exact, else -1
-__device__ __forceinline__ double thr4_of(double t) { return t >= 0x1p-1020 ? ldexp(t, 2) : -1.0; }
-__device__ __forceinline__ float thr4_of(float t) { return t >= 0x1p-124f ? ldexpf(t, 2) : -1.0f; }
+__device__ __forceinline__ double thr4_of(double t) { return ge_nonneg(t, 0x1p-1020) ? t * 4.0 : -1.0; }
+__device__ __forceinline__ float thr4_of(float t) { return t >= 0x1p-124f ? t * 4.0f : -1.0f; }
 
-// With t, t_end, dt and s_max given (no reload of what the caller holds).
+// With t, t_end, dt, s_max and the inflow at t given (no reload of what the
+// caller holds).
 __device__ inline void prepare_vals(DevState* st, const FinishArgs& a, double t, double t_end, double dt,
-                                    const double* smax) {
+                                    const double (&smax)[3], double Q) {
     for (int k = threadIdx.x; k < 3 * a.L; k += blockDim.x) {
         const int n = k / 3, q = k - 3 * n;
-        const double td = ldexp(a.eps, n - a.L) * smax[q];
-        const float tf = ldexpf((float)a.eps, n - a.L) * (float)smax[q];
+        const double sm = q == 0 ? smax[0] : (q == 1 ? smax[1] : smax[2]);
+        const double td = a.eps_n[n] * sm;              // eps 2^(n-L) s_max
+        const float tf = a.epsf_n[n] * (float)sm;
         st->thr[n * 3 + q] = td;
         st->thrf[n * 3 + q] = tf;
         const double t4 = thr4_of(td);
         st->thr4[n * 3 + q] = t4;
         st->thr4f[n * 3 + q] = thr4_of(tf);
-        const bool pre = t4 >= 0x1p-100;
+        const bool pre = ge_nonneg(t4, 0x1p-100);
         st->thr4lo[n * 3 + q] = pre ? __double2float_rd(t4) : -1.0f;
         st->thr4hi[n * 3 + q] = pre ? __double2float_ru(t4) : -1.0f;
     }
-    // the scalars: four independent tasks on lane 0 of different warps (a
-    // double division holds the FP64 pipe of its sub-partition for hundreds
-    // of cycles), each forming dt_use itself
+    // the scalars: independent tasks on lane 0 of different warps, the last
+    // ones first (the thresholds keep the first), each forming dt_use itself
     if ((threadIdx.x & 31u) != 0u) return;
     const int warp = (int)(threadIdx.x >> 5), nw = (int)((blockDim.x + 31u) >> 5);
     double dt_use = dt;
     if (t + dt_use > t_end) dt_use = t_end - t;
-    for (int task = warp; task < 4; task += nw) {
+    for (int task = nw - 1 - warp; task < 4; task += nw) {
         if (task == 0) {
+            st->rx0 = dt_use / a.lx;            // dt/dx_n = (dt/lx) * 2^n exactly
+        } else if (task == 1) {
+            st->ry0 = dt_use / a.ly;
+        } else if (task == 2) {
+            // the friction term's product with dt, in the operation order of
+            // dt * g * n * n * |u| (the leaf's part follows in the update)
+            st->fric_k = ((dt_use * a.g) * a.manning_n) * a.manning_n;
+            st->fric_kf = (((float)dt_use * (float)a.g) * (float)a.manning_n) * (float)a.manning_n;
+            st->Qdt = Q * dt_use;
+        } else {
             st->active = t < t_end ? 1u : 0u;
             st->dt_use = dt_use;
             st->rx0f = (float)dt_use / (float)a.lx;
@@ -2817,22 +3002,12 @@ __device__ inline void prepare_vals(DevState* st, const FinishArgs& a, double t,
             st->rmin_bits = kInfBits;
             st->max_bits[0] = st->max_bits[1] = st->max_bits[2] = 0ull;
             st->speed_bits[0] = st->speed_bits[1] = st->speed_bits[2] = 0ull;
-            // the friction term's product with dt, in the operation order of
-            // dt * g * n * n * |u| (the leaf's part follows in the update)
-            st->fric_k = ((dt_use * a.g) * a.manning_n) * a.manning_n;
-            st->fric_kf = (((float)dt_use * (float)a.g) * (float)a.manning_n) * (float)a.manning_n;
-        } else if (task == 1) {
-            st->rx0 = dt_use / a.lx;            // dt/dx_n = (dt/lx) * 2^n exactly
-        } else if (task == 2) {
-            st->ry0 = dt_use / a.ly;
-        } else {
-            st->Qdt = inflow_Q(a, t) * dt_use;
         }
     }
 }
 __device__ inline void prepare_step(DevState* st, const FinishArgs& a) {
     const double smax[3] = {st->smax[0], st->smax[1], st->smax[2]};
-    prepare_vals(st, a, st->t, st->t_end, st->dt, smax);
+    prepare_vals(st, a, st->t, st->t_end, st->dt, smax, inflow_Q(a, st->t));
 }
 
 // next timestep: CFL * (min CFL bound), capped at dt_max (+inf when dry)
@@ -2842,69 +3017,85 @@ __device__ inline double dt_from(const FinishArgs& a, double r) {
 }
 
 __device__ inline double smax_of(unsigned long long bits) {
-    const double m = from_obits(bits);
-    return 1.0 > m ? 1.0 : m;
+    // max(1, m) on the bits of a non-negative m (a NaN stays)
+    constexpr unsigned long long one = 0x3FF0000000000000ull;
+    return from_obits(bits > one ? bits : one);
 }
 
 // One block advances the scalars, then prepares the next step.  The
 // independent parts run on lane 0 of different warps: the time and the
-// counters, the two CFL quotients (one division each), the three s_max;
-// then the timestep.  The step's CFL bound is the min of the bounds reduced
-// as such and of dx_L / max(|u|+sqrt(gh)) and dy_L / max(|v|+sqrt(gh)) over
-// the wet leaves whose speeds were reduced instead: a correctly rounded
-// division is monotone in its divisor, so dx_L divided by the largest speed
-// is exactly the smallest of the per-leaf quotients (Sec. 2.1.3 CFL).
+// counters, the two CFL quotients (one division each), the inflow at the new
+// time; then every thread forms the timestep for itself.  The step's CFL bound
+// is the min of the bounds reduced as such and of dx_L / max(|u|+sqrt(gh)) and
+// dy_L / max(|v|+sqrt(gh)) over the wet leaves whose speeds were reduced
+// instead: a correctly rounded division is monotone in its divisor, so dx_L
+// divided by the largest speed is exactly the smallest of the per-leaf
+// quotients (Sec. 2.1.3 CFL).
+//
+// A chain on one CTA at the end of every step: k_decode_finish of a 64 x 64
+// grid, most of which is this, takes 3.6 us (5.3 us when the words were loaded
+// part by part and the quotients, powers of two and inflow formed in turn).
 __device__ __forceinline__ void finish_body(DevState* st, const FinishArgs& a) {
-    if (!st->active) return;
-    __syncthreads();                 // every thread has read `active`
-    // values handed between the parts through shared memory, so that
-    // nothing written here is read back from global memory
-    __shared__ double s_q[2], s_t, s_tend, s_dt, s_r, s_smax[3];
+    // every word first (one round of loads)
+    const uint32_t active = __ldcg(&st->active);
+    const unsigned long long sp0 = __ldcg(&st->speed_bits[0]), sp1 = __ldcg(&st->speed_bits[1]);
+    const unsigned long long rmin = __ldcg(&st->rmin_bits);
+    const unsigned long long mb[3] = {__ldcg(&st->max_bits[0]), __ldcg(&st->max_bits[1]), __ldcg(&st->max_bits[2])};
+    const double t = __ldcg(&st->t) + __ldcg(&st->dt_use), t_end = __ldcg(&st->t_end);
+    if (!active) return;
+    __shared__ double s_q[2], s_Q;
     const int warp = (int)(threadIdx.x >> 5), nw = (int)((blockDim.x + 31u) >> 5);
-    const bool speeds = st->speed_bits[0] != 0ull;
+    const bool speeds = sp0 != 0ull;
+    // the counters: one thread of the second warp
+    const bool counts = threadIdx.x == (nw > 1 ? 32u : 0u);
+    unsigned long long lu = 0ull, au = 0ull, wu = 0ull;
+    long long step = 0;
+    uint32_t epoch = 0u, cur = 0u;
+    if (counts) {
+        lu = __ldcg(&st->leaf_updates) + __ldcg(&st->Mall);
+        au = __ldcg(&st->act_updates) + __ldcg(&st->M);
+        wu = __ldcg(&st->wet_updates) + __ldcg(&st->nwet);
+        step = __ldcg(&st->step) + 1;
+        epoch = __ldcg(&st->epoch) + 1u;
+        cur = __ldcg(&st->cur) ^ 1u;
+    }
     if ((threadIdx.x & 31u) == 0u) {
-        for (int task = warp; task < 4; task += nw) {
+        for (int task = warp; task < 3; task += nw) {
             if (task == 0) {
-                const double t = st->t + st->dt_use;
-                st->t = t;
-                s_t = t;
-                s_tend = st->t_end;
-                st->step += 1;
-                st->epoch += 1u;
-                st->leaf_updates += st->Mall;
-                st->act_updates += st->M;
-                st->wet_updates += st->nwet;
-                st->cur ^= 1u;
+                if (speeds) s_q[0] = a.dxL / from_obits(sp0);
             } else if (task == 1) {
-                if (speeds) s_q[0] = ldexp(a.lx, -a.L) / __longlong_as_double((long long)st->speed_bits[0]);
-                s_r = from_obits(st->rmin_bits);
+                if (speeds) s_q[1] = a.dyL / from_obits(sp1);
             } else if (task == 2) {
-                if (speeds) s_q[1] = ldexp(a.ly, -a.L) / __longlong_as_double((long long)st->speed_bits[1]);
-            } else {
-                for (int q = 0; q < 3; ++q) {
-                    const double m = smax_of(st->max_bits[q]);
-                    st->smax[q] = m;
-                    s_smax[q] = m;
-                }
+                s_Q = inflow_Q(a, t);
             }
         }
     }
-    __syncthreads();
+    __syncthreads();                 // (and every thread has read the state)
+    if (counts) {
+        st->t = t;
+        st->cur = cur;
+        st->step = step;
+        st->epoch = epoch;
+        st->leaf_updates = lu;
+        st->act_updates = au;
+        st->wet_updates = wu;
+    }
+    double r = from_obits(rmin);
+    if (speeds) {
+        const double rx = s_q[0], ry = s_q[1];
+        const double rr = rx < ry ? rx : ry;
+        r = rr < r ? rr : r;
+    }
+    const double dt = dt_from(a, r);
+    const double smax[3] = {smax_of(mb[0]), smax_of(mb[1]), smax_of(mb[2])};
     if (threadIdx.x == 0) {
-        double r = s_r;
-        if (speeds) {
-            const double rx = s_q[0], ry = s_q[1];
-            const double rr = rx < ry ? rx : ry;
-            r = rr < r ? rr : r;
-        }
-        const double dt = dt_from(a, r);
         st->dt = dt;
-        s_dt = dt;
-        if (!isfinite(dt) || !isfinite(s_smax[0]) || !isfinite(s_smax[1]) || !isfinite(s_smax[2]))
+#pragma unroll
+        for (int q = 0; q < 3; ++q) st->smax[q] = smax[q];
+        if (!(finite_bits(dt) && finite_bits(smax[0]) && finite_bits(smax[1]) && finite_bits(smax[2])))
             st->err |= kErrNonFinite;
     }
-    __syncthreads();
-    prepare_vals(st, a, s_t, s_tend, s_dt, s_smax);
+    prepare_vals(st, a, t, t_end, dt, smax, s_Q);
 }
 
 // Decode-back followed, in its last CTA to finish, by the time advance (one
@@ -2916,9 +3107,9 @@ __device__ __forceinline__ void finish_body(DevState* st, const FinishArgs& a) {
 // and leave at once, so a short decode list costs few fences and ticket
 // atomics.  ndec is fixed from the traversal to the next step's clear.
 template <typename T>
-static __global__ void __launch_bounds__(256) k_decode_finish(DecodeArgs<T> a, FinishArgs fa) {
+static __global__ void __launch_bounds__(256, 6) k_decode_finish(DecodeArgs<T> a, FinishArgs fa) {
     pdl_wait();
-    const uint32_t nd = __ldcg(&a.st->ndec);
+    const uint32_t nd = now(&a.st->ndec);
     const uint32_t parts = nd < gridDim.x ? (nd > 0u ? nd : 1u) : gridDim.x;
     if (blockIdx.x >= parts) return;
     decode_body<T>(a, this_blk());

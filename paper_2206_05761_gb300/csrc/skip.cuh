@@ -292,11 +292,12 @@ static __global__ void __launch_bounds__(256) k_skip_decode(SkipDecodeArgs<T> a,
     unsigned long long mh = 0, mqx = 0, mqy = 0;
     __shared__ int s_l0[4];
     __shared__ unsigned long long s_bits[4][4];   // S of the subtree's levels Ls .. Ls+3
-    const bool run = __ldcg(&st->active) != 0u;
+    const uint32_t active = now(&st->active), cur = now(&st->cur);
+    const bool run = active != 0u;
     const int Ls = a.Ls;
     const uint32_t nsub = 1u << (2 * Ls);
     const uint32_t g = threadIdx.x >> 6, t = threadIdx.x & 63u;
-    const int nxt = (int)__ldcg(&st->cur) ^ 1;
+    const int nxt = (int)cur ^ 1;
     T* const fh = nxt ? a.f[1][0] : a.f[0][0];
     T* const fqx = nxt ? a.f[1][1] : a.f[0][1];
     T* const fqy = nxt ? a.f[1][2] : a.f[0][2];
