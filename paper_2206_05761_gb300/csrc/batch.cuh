@@ -112,40 +112,54 @@ static __global__ void __launch_bounds__(256) kb_trav_write(const DomainPlan<T>*
     trav_write_body(p.Sb, p.coffs, p.leaves, p.L, p.kt, p.ntiles, p.st, domain_blk(base, d), nullptr);
 }
 
+// A member's arguments in shared memory, where the single-domain kernels have
+// theirs in the constant bank: copied into registers they cost the update 40 of
+// them and the faces 16 (16 basins: kb_fv1_update 188 -> 154 us a step, all of 32
+// steps 6.57 -> 6.08 ms with this and the register limits below).
+template <typename A>
+__device__ __forceinline__ const A& shared_args(const A& g) {
+    static_assert(sizeof(A) % 4 == 0, "copied as words");
+    __shared__ __align__(16) uint32_t w[sizeof(A) / 4];
+    for (uint32_t i = threadIdx.x; i < sizeof(A) / 4; i += blockDim.x)
+        w[i] = reinterpret_cast<const uint32_t*>(&g)[i];
+    __syncthreads();
+    return *reinterpret_cast<const A*>(w);
+}
+
 template <typename T>
 static __global__ void __launch_bounds__(256) kb_fv1_dry(const DomainPlan<T>* P, const uint32_t* base, int D) {
     const int d = find_domain(base, D, blockIdx.x);
-    const StepArgs<T> a = P[d].step;
+    const StepArgs<T>& a = shared_args(P[d].step);
     fv1_dry_body<T>(a, domain_blk(base, d));
 }
 
 // the shared-face pair of the single-domain path (float64), and the one-pass
 // update of the leaves it leaves out (float32: all of them)
 template <typename T>
-static __global__ void __launch_bounds__(128) kb_fv1_faces(const DomainPlan<T>* P, const uint32_t* base, int D) {
+static __global__ void __launch_bounds__(128, 8) kb_fv1_faces(const DomainPlan<T>* P, const uint32_t* base, int D) {
     const int d = find_domain(base, D, blockIdx.x);
-    const StepArgs<T> a = P[d].step;
+    const StepArgs<T>& a = shared_args(P[d].step);
     fv1_faces_body<T>(a, domain_blk(base, d));
 }
 
 template <typename T>
-static __global__ void __launch_bounds__(64) kb_fv1_update(const DomainPlan<T>* P, const uint32_t* base, int D) {
+static __global__ void __launch_bounds__(64, 12) kb_fv1_update(const DomainPlan<T>* P, const uint32_t* base, int D) {
     const int d = find_domain(base, D, blockIdx.x);
-    const StepArgs<T> a = P[d].step;
+    const StepArgs<T>& a = shared_args(P[d].step);
     fv1_update_body<T>(a, domain_blk(base, d));
 }
 
 template <typename T>
 static __global__ void __launch_bounds__(64) kb_fv1_wet(const DomainPlan<T>* P, const uint32_t* base, int D) {
     const int d = find_domain(base, D, blockIdx.x);
-    const StepArgs<T> a = P[d].step;
+    const StepArgs<T>& a = shared_args(P[d].step);
     fv1_wet_body<T>(a, domain_blk(base, d));
 }
 
 template <typename T>
 static __global__ void __launch_bounds__(256) kb_decode(const DomainPlan<T>* P, const uint32_t* base, int D) {
     const int d = find_domain(base, D, blockIdx.x);
-    const DecodeArgs<T> a = P[d].dec;
+    const DecodeArgs<T>& a = shared_args(P[d].dec);
     decode_body<T>(a, domain_blk(base, d));
 }
 

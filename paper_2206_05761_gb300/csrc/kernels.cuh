@@ -2153,12 +2153,6 @@ template <typename T> __device__ __forceinline__ T ry0_of(const DevState* st);
 template <> __device__ __forceinline__ double ry0_of<double>(const DevState* st) { return st->ry0; }
 template <> __device__ __forceinline__ float ry0_of<float>(const DevState* st) { return st->ry0f; }
 
-// FV1, first kernel: every leaf whose own and four same-level neighbour
-// depths are exactly zero and that has no inflow gets (+0, +0, +0) -- what
-// the full update computes for it (all reconstructed depths and fluxes are
-// 0, its CFL bound is infinite) -- decided on the depth bits alone.  Every
-// other leaf is queued for k_fv1_wet.  Needs few registers, so many warps
-// hide the gather latency.
 // Neighbour depth addresses of a leaf from its packed id (Morton-domain
 // arithmetic; ghosts read the leaf itself).
 struct DryProbe {
@@ -2300,10 +2294,10 @@ static __global__ void __launch_bounds__(256) k_fv1_dry(StepArgs<T> a) {
 // cells) and reductions of one updated wet leaf.
 template <typename T>
 __device__ __forceinline__ void wet_leaf_store(const StepArgs<T>& a, DevState* st, const T* z, T* oh, T* oqx,
-                                               T* oqy, int n, uint32_t code, uint64_t iC, const Cell<T>& C,
-                                               const T out[3], const T sp[2], unsigned long long& rmin,
-                                               unsigned long long& mh, unsigned long long& mqx,
-                                               unsigned long long& mqy, unsigned long long* spd) {
+                                               T* oqy, int n, uint32_t code, uint64_t iC, const T out[3],
+                                               const T sp[2], unsigned long long& rmin, unsigned long long& mh,
+                                               unsigned long long& mqx, unsigned long long& mqy,
+                                               unsigned long long* spd) {
     if (sizeof(T) == 8) {
         const unsigned long long bx = abs_obits(sp[0]), by = abs_obits(sp[1]);
         spd[0] = bx > spd[0] ? bx : spd[0];
@@ -2407,7 +2401,7 @@ __device__ __forceinline__ void fv1_wet_body(const StepArgs<T>& a, Blk B) {
         }
         T out[3], sp[2];
         cell_update(a.P, rx, ry, fk, C, W, E, S, N, inlet, dh, out, sp);
-        wet_leaf_store(a, st, src.z, oh, oqx, oqy, n, code, iC, C, out, sp, rmin, mh, mqx, mqy, spd);
+        wet_leaf_store(a, st, src.z, oh, oqx, oqy, n, code, iC, out, sp, rmin, mh, mqx, mqy, spd);
     }
     if (sizeof(T) != 8) block_atomic_u64<false>(rmin, &st->rmin_bits);   // (float64: the speeds)
     block_max5_u64({mh, mqx, mqy, spd[0], spd[1]}, st->max_bits, st->speed_bits);
@@ -2569,7 +2563,7 @@ __device__ __forceinline__ void fv1_match_body(const StepArgs<T>& a, Blk B) {
         }
         T out[3], sp[2];
         cell_update_faces_sq(a.P, rx, ry, fk, C, FW, FE, GS, GN, w2, e2, s2, n2, inlet, dh, out, sp);
-        wet_leaf_store(a, st, src.z, oh, oqx, oqy, n, code, iC, C, out, sp, rmin, mh, mqx, mqy, spd);
+        wet_leaf_store(a, st, src.z, oh, oqx, oqy, n, code, iC, out, sp, rmin, mh, mqx, mqy, spd);
     }
     if (sizeof(T) != 8) block_atomic_u64<false>(rmin, &st->rmin_bits);   // (float64: the speeds)
     block_max5_u64({mh, mqx, mqy, spd[0], spd[1]}, st->max_bits, st->speed_bits);
@@ -2745,6 +2739,91 @@ static __global__ void __launch_bounds__(128, 8) k_fv1_faces(StepArgs<T> a) {
     fv1_faces_body<T, FM>(a, this_blk());
 }
 
+// What the update of the queue's leaf w takes.
+template <typename T>
+struct UpdateIn {
+    Cell<T> C;
+    T FW[3], FE[3], GS[3], GN[3];
+    T hW2, hE2, hS2, hN2;    // squares of the reconstructed depths of the cell at its faces
+    T rx, ry, dh;
+    uint64_t iC;
+    uint32_t code;
+    int n;
+    bool inlet;
+};
+template <typename T>
+__device__ __forceinline__ void load_update(const StepArgs<T>& a, int par, T rx0, T ry0, T Qdt, uint32_t w,
+                                            UpdateIn<T>& u) {
+    const size_t cap = a.fcap;
+    const uint32_t pk = a.wet[w];
+    const uint2 ws = *reinterpret_cast<const uint2*>(slots_at(a.face, cap, w));
+    u.n = (int)(pk >> kLeafShift);
+    u.code = pk & kCodeMask;
+    u.iC = lvl_off(u.n) + u.code;
+    // the west and south faces: the queued neighbour's, or the leaf's own
+    const bool sW = (ws.x & kShared) != 0u, sS = (ws.y & kShared) != 0u;
+    const uint32_t wW = ws.x & ~kShared, wS = ws.y & ~kShared;
+    const typename Pair2<T>::V e0 = *pair_at(a.face, cap, kFaceE, w), e1 = *pair_at(a.face, cap, kFaceE + 2, w);
+    const typename Pair2<T>::V n0 = *pair_at(a.face, cap, kFaceN, w), n1 = *pair_at(a.face, cap, kFaceN + 2, w);
+    const int kW = sW ? kFaceE : kFaceW, kS = sS ? kFaceN : kFaceS;
+    const typename Pair2<T>::V w0 = *pair_at(a.face, cap, kW, wW), w1 = *pair_at(a.face, cap, kW + 2, wW);
+    const typename Pair2<T>::V s0 = *pair_at(a.face, cap, kS, wS), s1 = *pair_at(a.face, cap, kS + 2, wS);
+    u.hW2 = w1.y;
+    u.hS2 = s1.y;
+    if (sW) u.hW2 = a.face[(kFaceE + 4) * cap + wW];
+    if (sS) u.hS2 = a.face[(kFaceN + 4) * cap + wS];
+    u.C.h = __ldg((par ? a.f[1][0] : a.f[0][0]) + u.iC);
+    u.C.qx = __ldg((par ? a.f[1][1] : a.f[0][1]) + u.iC);
+    u.C.qy = __ldg((par ? a.f[1][2] : a.f[0][2]) + u.iC);
+    u.FE[0] = e0.x, u.FE[1] = e0.y, u.FE[2] = e1.x, u.hE2 = e1.y;
+    u.GN[0] = n0.x, u.GN[1] = n0.y, u.GN[2] = n1.x, u.hN2 = n1.y;
+    u.FW[0] = w0.x, u.FW[1] = w0.y, u.FW[2] = w1.x;
+    u.GS[0] = s0.x, u.GS[1] = s0.y, u.GS[2] = s1.x;
+    u.rx = mul_pow2(rx0, u.n);                   // rx0 * 2^n, exact
+    u.ry = mul_pow2(ry0, u.n);
+    int64_t lo = 0, hi = 0;
+    u.inlet = a.inflow_side >= 0 && inlet_range(a, u.n, compact16(u.code), compact16(u.code >> 1), (1u << u.n) - 1u,
+                                                lo, hi);
+    u.dh = T(0);
+    if (u.inlet) {
+        const T scale = (T)(1u << u.n);
+        const T frac = (T)(hi - lo) / (T)(a.a1 - a.a0);
+        const T inv2n = T(1) / scale;
+        const T dxn = a.lx * inv2n, dyn = a.ly * inv2n;
+        u.dh = (Qdt * frac) / (dxn * dyn);
+    }
+}
+// The update of leaf w; false where an operation was out of its range.
+template <class Ops, typename T>
+__device__ __forceinline__ bool update_leaf(const StepArgs<T>& a, T fk, const UpdateIn<T>& u, T out[3], T sp[2]) {
+    Ops o;
+    cell_update_ops<T>(o, a.P, u.rx, u.ry, fk, u.C, u.FW, u.FE, u.GS, u.GN, u.hW2, u.hE2, u.hS2, u.hN2, u.inlet, u.dh,
+                       out, sp);
+    return !o.bad;
+}
+// The update of leaf w with the operations as written, from its operands in
+// memory again: kept over the other form they would cost it 30 registers.
+static __device__ __noinline__ void update_rare(const StepArgs<double>& a, int par, uint32_t w, double* res) {
+    UpdateIn<double> u;
+    load_update<double>(a, par, rx0_of<double>(a.st), ry0_of<double>(a.st), a.st->Qdt, w, u);
+    update_leaf<PlainOps<double>>(a, fric_k_of<double>(a.st), u, res, res + 3);
+}
+__device__ __forceinline__ void update_queued(const StepArgs<double>& a, int par, uint32_t w, double fk,
+                                              const UpdateIn<double>& u, double out[3], double sp[2]) {
+    if (update_leaf<IntOps>(a, fk, u, out, sp)) return;
+    double res[5];
+    update_rare(a, par, w, res);
+    out[0] = res[0];
+    out[1] = res[1];
+    out[2] = res[2];
+    sp[0] = res[3];
+    sp[1] = res[4];
+}
+__device__ __forceinline__ void update_queued(const StepArgs<float>& a, int, uint32_t, float fk,
+                                              const UpdateIn<float>& u, float out[3], float sp[2]) {
+    update_leaf<PlainOps<float>>(a, fk, u, out, sp);
+}
+
 template <typename T>
 __device__ __forceinline__ void fv1_update_body(const StepArgs<T>& a, Blk B) {
     DevState* st = a.st;
@@ -2755,66 +2834,26 @@ __device__ __forceinline__ void fv1_update_body(const StepArgs<T>& a, Blk B) {
     const T fk = fric_k_of<T>(st);
     const T rx0 = rx0_of<T>(st), ry0 = ry0_of<T>(st);
     const T Qdt = (T)st->Qdt;
-    CellSrc<T> src;
-    src.h = par ? a.f[1][0] : a.f[0][0];
-    src.qx = par ? a.f[1][1] : a.f[0][1];
-    src.qy = par ? a.f[1][2] : a.f[0][2];
-    src.z = a.z;
     T* const oh = nxt ? a.f[1][0] : a.f[0][0];
     T* const oqx = nxt ? a.f[1][1] : a.f[0][1];
     T* const oqy = nxt ? a.f[1][2] : a.f[0][2];
-    const size_t cap = a.fcap;
     unsigned long long rmin = kInfBits, mh = 0, mqx = 0, mqy = 0, spd[2] = {0ull, 0ull};
     for (uint32_t w = B.id * blockDim.x + threadIdx.x; w < nq; w += B.n * blockDim.x) {
-        const uint32_t pk = a.wet[w];
-        const uint2 ws = *reinterpret_cast<const uint2*>(slots_at(a.face, cap, w));
-        const int n = (int)(pk >> kLeafShift);
-        const uint32_t code = pk & kCodeMask;
-        const uint64_t iC = lvl_off(n) + code;
-        // the west and south faces: the queued neighbour's, or the leaf's own
-        const bool sW = (ws.x & kShared) != 0u, sS = (ws.y & kShared) != 0u;
-        const uint32_t wW = ws.x & ~kShared, wS = ws.y & ~kShared;
-        const typename Pair2<T>::V e0 = *pair_at(a.face, cap, kFaceE, w), e1 = *pair_at(a.face, cap, kFaceE + 2, w);
-        const typename Pair2<T>::V n0 = *pair_at(a.face, cap, kFaceN, w), n1 = *pair_at(a.face, cap, kFaceN + 2, w);
-        const int kW = sW ? kFaceE : kFaceW, kS = sS ? kFaceN : kFaceS;
-        const typename Pair2<T>::V w0 = *pair_at(a.face, cap, kW, wW), w1 = *pair_at(a.face, cap, kW + 2, wW);
-        const typename Pair2<T>::V s0 = *pair_at(a.face, cap, kS, wS), s1 = *pair_at(a.face, cap, kS + 2, wS);
-        // squares of the reconstructed depths of the cell at its faces
-        T hW2 = w1.y, hS2 = s1.y;
-        if (sW) hW2 = a.face[(kFaceE + 4) * cap + wW];
-        if (sS) hS2 = a.face[(kFaceN + 4) * cap + wS];
-        Cell<T> C;
-        C.h = __ldg(src.h + iC);
-        C.qx = __ldg(src.qx + iC);
-        C.qy = __ldg(src.qy + iC);
-        const T FE[3] = {e0.x, e0.y, e1.x}, hE2 = e1.y;
-        const T GN[3] = {n0.x, n0.y, n1.x}, hN2 = n1.y;
-        const T FW[3] = {w0.x, w0.y, w1.x};
-        const T GS[3] = {s0.x, s0.y, s1.x};
-        const T rx = mul_pow2(rx0, n), ry = mul_pow2(ry0, n);   // rx0 * 2^n, exact
-        int64_t lo = 0, hi = 0;
-        const bool inlet = a.inflow_side >= 0 && inlet_range(a, n, compact16(code), compact16(code >> 1),
-                                                             (1u << n) - 1u, lo, hi);
-        T dh = T(0);
-        if (inlet) {
-            const T scale = (T)(1u << n);
-            const T frac = (T)(hi - lo) / (T)(a.a1 - a.a0);
-            const T inv2n = T(1) / scale;
-            const T dxn = a.lx * inv2n, dyn = a.ly * inv2n;
-            dh = (Qdt * frac) / (dxn * dyn);
-        }
+        UpdateIn<T> u;
+        load_update(a, par, rx0, ry0, Qdt, w, u);
         T out[3], sp[2];
-        cell_update_faces_sq(a.P, rx, ry, fk, C, FW, FE, GS, GN, hW2, hE2, hS2, hN2, inlet, dh, out, sp);
-        wet_leaf_store(a, st, src.z, oh, oqx, oqy, n, code, iC, C, out, sp, rmin, mh, mqx, mqy, spd);
+        update_queued(a, par, w, fk, u, out, sp);
+        wet_leaf_store(a, st, a.z, oh, oqx, oqy, u.n, u.code, u.iC, out, sp, rmin, mh, mqx, mqy, spd);
     }
     if (sizeof(T) != 8) block_atomic_u64<false>(rmin, &st->rmin_bits);   // (float64: the speeds)
     block_max5_u64({mh, mqx, mqy, spd[0], spd[1]}, st->max_bits, st->speed_bits);
 }
-// 64 us for 1 M leaves (uniform FV1, L=10; 116 us with its products on the
+// 55 us for 1 M leaves (uniform FV1, L=10; 116 us with its products on the
 // FP64 pipe and the unshared faces formed here): the FP64 pipe's 19 sums a leaf
-// fill two thirds of it, the rest is the latency of the gathers.
+// fill three quarters of it, the rest is the latency of the gathers, so twelve
+// blocks an SM (80 registers; 60 us with the eight that 110 registers leave).
 template <typename T>
-static __global__ void __launch_bounds__(64) k_fv1_update(StepArgs<T> a) {
+static __global__ void __launch_bounds__(64, 12) k_fv1_update(const __grid_constant__ StepArgs<T> a) {
     pdl_wait();
     fv1_update_body<T>(a, this_blk());
 }
