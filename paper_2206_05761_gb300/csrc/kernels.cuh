@@ -2193,71 +2193,80 @@ __device__ __forceinline__ bool dry5(const T* __restrict__ h, const DryProbe& d)
     return is_zero(a) && is_zero(b) && is_zero(c) && is_zero(e) && is_zero(f);
 }
 
-// FV1, first kernel: every leaf whose own and four same-level neighbour
-// depths are exactly zero and that has no inflow gets (+0, +0, +0) -- what
-// the full update computes for it (all reconstructed depths and fluxes are
-// 0, its CFL bound is infinite) -- decided on the depth bits alone.  Every
-// other leaf is queued for k_fv1_wet.  Few registers and two leaves per
-// iteration, so many independent loads are in flight.
+// The zeros of a dry leaf (all reconstructed depths and fluxes are 0, its CFL
+// bound is infinite).
 template <typename T>
-__device__ __forceinline__ void dry_finish(const StepArgs<T>& a, DevState* st, T* oh, T* oqx, T* oqy,
-                                           const DryProbe& d, bool dry, uint32_t pk, const CellSrc<T>& src,
-                                           unsigned long long stamp) {
-    if (dry && a.inflow_side >= 0) {
-        int64_t lo, hi;
-        dry = !inlet_range(a, d.n, compact16(d.code), compact16(d.code >> 1), (1u << d.n) - 1u, lo, hi);
-    }
-    if (dry) {
-        if (d.n == a.L || needs_decode_kernel(d.n, a.L) || a.own_slot) {
-            oh[d.iC] = T(0);
-            oqx[d.iC] = T(0);
-            oqy[d.iC] = T(0);
-        } else {                              // 4 or 16 finest cells: decode here
-            const uint64_t fo = lvl_off(a.L) + ((uint64_t)d.code << (2 * (a.L - d.n)));
-            const uint32_t cnt = 1u << (2 * (a.L - d.n));
-            for (uint32_t e = 0; e < cnt; e += 4) {
-                Vec4<T>::store(oh + fo + e, T(0), T(0), T(0), T(0));
-                Vec4<T>::store(oqx + fo + e, T(0), T(0), T(0), T(0));
-                Vec4<T>::store(oqy + fo + e, T(0), T(0), T(0), T(0));
-            }
-        }
-    } else {
-        // warp-aggregated append to the queue of full updates
-        const uint32_t m = __activemask();
-        const uint32_t lane = threadIdx.x & 31u;
-        const uint32_t leader = __ffs(m) - 1u;
-        uint32_t base_pos = 0;
-        if (lane == leader) base_pos = atomicAdd(&st->nwet, (uint32_t)__popc(m));
-        base_pos = __shfl_sync(m, base_pos, leader);
-        const uint32_t w = base_pos + __popc(m & ((1u << lane) - 1u));
-        a.wet[w] = pk;                                            // the packed leaf
-        // float64 with shared faces: what the faces read of the leaf (its
-        // velocities, with the operations of velocity(), its free surface and
-        // bed) and its stamp, once per queued leaf
-        if (sizeof(T) == 8 && a.face != nullptr && w < a.fcap) {
-            Cell<T> C;
-            C.h = __ldg(src.h + d.iC);
-            C.qx = __ldg(src.qx + d.iC);
-            C.qy = __ldg(src.qy + d.iC);
-            C.z = __ldg(src.z + d.iC);
-            T u, v;
-            velocity(C, a.P.tol, u, v);
-            *pair_at(a.face, a.fcap, kLeafUV, w) = make_pair2(u, v);
-            *pair_at(a.face, a.fcap, kLeafEZ, w) = make_pair2(eta_of(C.h, C.z), C.z);
-            a.mark[d.iC] = stamp | w | (cell_window(C.h, C.z, u, v) ? 0u : kUnsafe);
+__device__ __forceinline__ void store_dry(const StepArgs<T>& a, T* oh, T* oqx, T* oqy, const DryProbe& d) {
+    if (d.n == a.L || needs_decode_kernel(d.n, a.L) || a.own_slot) {
+        oh[d.iC] = T(0);
+        oqx[d.iC] = T(0);
+        oqy[d.iC] = T(0);
+    } else {                              // 4 or 16 finest cells: decode here
+        const uint64_t fo = lvl_off(a.L) + ((uint64_t)d.code << (2 * (a.L - d.n)));
+        const uint32_t cnt = 1u << (2 * (a.L - d.n));
+        for (uint32_t e = 0; e < cnt; e += 4) {
+            Vec4<T>::store(oh + fo + e, T(0), T(0), T(0), T(0));
+            Vec4<T>::store(oqx + fo + e, T(0), T(0), T(0), T(0));
+            Vec4<T>::store(oqy + fo + e, T(0), T(0), T(0), T(0));
         }
     }
 }
+// float64 with shared faces: what the faces read of a queued leaf (its
+// velocities, with the operations of velocity(), its free surface and bed) and
+// its stamp, once per leaf.
+template <typename T>
+struct LeafPre {
+    T u, v, eta, z;
+    uint32_t unsafe;
+};
+template <typename T>
+__device__ __forceinline__ LeafPre<T> leaf_pre(const StepArgs<T>& a, const CellSrc<T>& src, uint64_t iC) {
+    LeafPre<T> r = {};
+    if (sizeof(T) == 8 && a.face != nullptr) {
+        Cell<T> C;
+        C.h = __ldg(src.h + iC);
+        C.qx = __ldg(src.qx + iC);
+        C.qy = __ldg(src.qy + iC);
+        C.z = __ldg(src.z + iC);
+        velocity(C, a.P.tol, r.u, r.v);
+        r.eta = eta_of(C.h, C.z);
+        r.z = C.z;
+        r.unsafe = cell_window(C.h, C.z, r.u, r.v) ? 0u : kUnsafe;
+    }
+    return r;
+}
+template <typename T>
+__device__ __forceinline__ void queue_leaf(const StepArgs<T>& a, uint32_t w, uint32_t pk, uint64_t iC,
+                                           const LeafPre<T>& r, unsigned long long stamp) {
+    a.wet[w] = pk;                                            // the packed leaf
+    if (sizeof(T) == 8 && a.face != nullptr && w < a.fcap) {
+        *pair_at(a.face, a.fcap, kLeafUV, w) = make_pair2(r.u, r.v);
+        *pair_at(a.face, a.fcap, kLeafEZ, w) = make_pair2(r.eta, r.z);
+        a.mark[iC] = stamp | w | r.unsafe;
+    }
+}
 
+// FV1, first kernel: every leaf whose own and four same-level neighbour
+// depths are exactly zero and that has no inflow gets (+0, +0, +0) -- what
+// the full update computes for it -- decided on the depth bits alone.  Every
+// other leaf is queued for the full update.  Two leaves a thread, so many
+// independent loads are in flight.
+//
+// A warp takes 64 leaves in a row (an 8 x 8 patch where they are of one size)
+// and appends its wet ones with one addition to the queue's length, whose
+// latency passes while it forms what the faces read of them.  With an addition
+// for each 32 leaves, all on one word, 1 M wet leaves took 34 us, now 24, and the
+// faces and the update of 1024 x 1024 bumps gain 3 % by the queue's order.  One
+// addition a block would want two barriers: slower where most leaves are dry
+// (2048 x 2048 float32 flood, 32 steps: 780 us, 763 with one per 32, now 745).
 template <typename T>
 __device__ __forceinline__ void fv1_dry_body(const StepArgs<T>& a, Blk B) {
     DevState* st = a.st;
     const uint32_t active = now(&st->active), M = now(&st->M), cur = now(&st->cur), epoch = now(&st->epoch);
     if (!active) return;
     const int par = (int)cur, nxt = par ^ 1;
-    const T* __restrict__ hsrc = par ? a.f[1][0] : a.f[0][0];
     CellSrc<T> src;
-    src.h = hsrc;
+    src.h = par ? a.f[1][0] : a.f[0][0];
     src.qx = par ? a.f[1][1] : a.f[0][1];
     src.qy = par ? a.f[1][2] : a.f[0][2];
     src.z = a.z;
@@ -2265,23 +2274,41 @@ __device__ __forceinline__ void fv1_dry_body(const StepArgs<T>& a, Blk B) {
     T* const oh = nxt ? a.f[1][0] : a.f[0][0];
     T* const oqx = nxt ? a.f[1][1] : a.f[0][1];
     T* const oqy = nxt ? a.f[1][2] : a.f[0][2];
-    const uint32_t stride = B.n * blockDim.x;
-    for (uint32_t k = B.id * blockDim.x + threadIdx.x; k < M; k += 2u * stride) {
-        const uint32_t k2 = k + stride;
-        const bool two = k2 < M;
-        const uint32_t p1 = __ldg(a.leaves + k), p2 = two ? __ldg(a.leaves + k2) : 0u;
+    const uint32_t lane = threadIdx.x & 31u, below = (1u << lane) - 1u;
+    const uint32_t warps = B.n * (blockDim.x / 32u);
+    // a list that leaves warps idle at that: 32 leaves a warp
+    const uint32_t per = M > warps * 32u ? 64u : 32u;
+    for (uint32_t b = (B.id * (blockDim.x / 32u) + threadIdx.x / 32u) * per; b < M; b += warps * per) {
+        const uint32_t k = b + lane, k2 = k + 32u;
+        const bool one = k < M, two = k2 < M && per == 64u;
+        const uint32_t p1 = one ? __ldg(a.leaves + k) : 0u, p2 = two ? __ldg(a.leaves + k2) : 0u;
         const DryProbe d1 = dry_probe(p1);
         const DryProbe d2 = dry_probe(p2);
-        bool y1 = dry5(hsrc, d1);
-        bool y2 = two && dry5(hsrc, d2);
+        bool y1 = dry5(src.h, d1);
+        bool y2 = two && dry5(src.h, d2);
         if (a.fm) {
             // with matched fluxes a face toward a refined neighbour averages
             // finer faces: such a leaf takes the full update
             y1 = y1 && !refined_nbr(a.Sb, d1, a.L);
             y2 = y2 && !refined_nbr(a.Sb, d2, a.L);
         }
-        dry_finish(a, st, oh, oqx, oqy, d1, y1, p1, src, stamp);
-        if (two) dry_finish(a, st, oh, oqx, oqy, d2, y2, p2, src, stamp);
+        if (a.inflow_side >= 0) {
+            int64_t lo, hi;
+            y1 = y1 && !inlet_range(a, d1.n, compact16(d1.code), compact16(d1.code >> 1), (1u << d1.n) - 1u, lo, hi);
+            y2 = y2 && !inlet_range(a, d2.n, compact16(d2.code), compact16(d2.code >> 1), (1u << d2.n) - 1u, lo, hi);
+        }
+        const bool q1 = one && !y1, q2 = two && !y2;
+        const uint32_t m1 = __ballot_sync(0xffffffffu, q1), m2 = __ballot_sync(0xffffffffu, q2);
+        uint32_t w = 0;
+        if (lane == 0 && (m1 | m2) != 0u) w = atomicAdd(&st->nwet, (uint32_t)(__popc(m1) + __popc(m2)));
+        LeafPre<T> r1 = {}, r2 = {};
+        if (q1) r1 = leaf_pre(a, src, d1.iC);
+        if (q2) r2 = leaf_pre(a, src, d2.iC);
+        if (one && y1) store_dry(a, oh, oqx, oqy, d1);
+        if (two && y2) store_dry(a, oh, oqx, oqy, d2);
+        w = __shfl_sync(0xffffffffu, w, 0);
+        if (q1) queue_leaf(a, w + __popc(m1 & below), p1, d1.iC, r1, stamp);
+        if (q2) queue_leaf(a, w + __popc(m1) + __popc(m2 & below), p2, d2.iC, r2, stamp);
     }
 }
 template <typename T>
