@@ -1126,6 +1126,30 @@ class EngineT final : public Engine {
         P.dyL = (T)std::ldexp(spec_.ly, -L_);
         return P;
     }
+    // The traversal and the FV1 update of a step: with quiescent tiles the
+    // listing and the dry pass are one kernel.  A profiled step runs the
+    // kernels of the phases (hwfv1_traverse, hwfv1_step), to time each.
+    void launch_traverse_fv1(bool onfly) {
+        if (!quiet_on_ || prof_) {
+            launch_traverse(false, onfly);
+            launch_fv1();
+            return;
+        }
+        const SigSrc sg = sig_src(onfly);
+        const StepArgs<T> a = step_args();
+        const uint32_t cap = (uint32_t)nsm_ * 8u;
+        if (4u * ntiles_ <= (uint32_t)nsm_) {
+            lk(k_trav_dry<T, kTravQuarters>, 4u * ntiles_, 256, sg, kt_, ntiles_, quiet(), scount_, dlist_, work_, a);
+        } else if (ntiles_ <= cap) {
+            lk(k_trav_dry<T, kTravTiles>, ntiles_, 256, sg, kt_, ntiles_, quiet(), scount_, dlist_, work_, a);
+        } else {
+            lk(k_trav_classify, (ntiles_ + 255) / 256, 256, sg, L_, kt_, ntiles_, st_, quiet(), scount_, work_, dlist_,
+               leaves_);
+            lk(k_trav_dry<T, kTravListed>, resident(k_trav_dry<T, kTravListed>, 256), 256, sg, kt_, ntiles_, quiet(),
+               scount_, dlist_, work_, a);
+        }
+        launch_wet(a);
+    }
     void launch_fv1(const uint32_t* leaves = nullptr) {
         StepArgs<T> a = step_args();
         if (leaves) {
@@ -1189,8 +1213,7 @@ class EngineT final : public Engine {
         const bool onfly = onfly_flags();
         launch_encode();
         if (!onfly) launch_flag();
-        launch_traverse(false, onfly);
-        launch_fv1();
+        launch_traverse_fv1(onfly);
         launch_decode(onfly);
         sb_valid_ = !onfly;
     }
@@ -1332,8 +1355,7 @@ class EngineT final : public Engine {
         launch_encode();
         if (predict_next) fork_predict();
         if (!onfly) launch_flag();
-        launch_traverse(false, onfly);
-        launch_fv1();
+        launch_traverse_fv1(onfly);
         if (predict_next) join_predict();
         launch_decode(onfly);
         sb_valid_ = !onfly;

@@ -2317,6 +2317,197 @@ static __global__ void __launch_bounds__(256) k_fv1_dry(StepArgs<T> a) {
     fv1_dry_body<T>(a, this_blk());
 }
 
+// The rest of the traversal and FV1's first kernel in one: a CTA forms a tile's
+// leaves (a thread per group of four finest cells, k_trav_list) and takes each
+// through fv1_dry_body's decision on the spot, without the list between them.
+// kTravListed: the tiles are those of k_trav_classify's work list, and the
+// leaves that it listed itself (those that cover a tile) are taken from its
+// list.  Otherwise a CTA classifies its tile as well: nothing in the decision
+// needs another tile's outcome, and a grid of at most eight tiles an SM has no
+// use for a launch that thins them out.  kTravQuarters, where four CTAs a tile
+// still leave SMs free: a thread per cell instead of four in turn (64 x 64 cells:
+// 6.2 us, 7.1 with a CTA per tile, 9.2 as three kernels with their gaps).  Not
+// beyond: a CTA's leaves sit together in the queue, which the faces read
+// neighbours from, and quarters of 256 tiles cost the matched 512 x 512 basin 12 %.
+// 32 steps against classify, list and dry pass as kernels of their own: 64 x 64
+// dam break 1453 -> 1297 us, matched basin 3330 -> 3070, 1024 bumps 4183 -> 4084,
+// 2048 columns 1954 -> 1919, 4096 flood 2254 -> 2230, 2048 flood float32 749 -> 735.
+enum { kTravTiles, kTravListed, kTravQuarters };
+template <typename T, int MODE>
+static __global__ void __launch_bounds__(256, 6) k_trav_dry(SigSrc Sb, int kt, uint32_t ntiles, Quiet q,
+                                                            const uint32_t* __restrict__ scount,
+                                                            uint32_t* __restrict__ dlist,
+                                                            const uint32_t* __restrict__ work,
+                                                            const __grid_constant__ StepArgs<T> a) {
+    pdl_wait();
+    DevState* st = a.st;
+    const uint32_t active = now(&st->active), cur = now(&st->cur), epoch = now(&st->epoch);
+    constexpr bool LISTED = MODE == kTravListed;
+    const uint32_t n = LISTED ? now(&st->nact) : MODE == kTravQuarters ? 4u * ntiles : ntiles;
+    const uint32_t nlist = LISTED ? now(&st->M) : 0u;
+    if (!active) return;
+    __shared__ TileBits tb;
+    __shared__ uint32_t red[2][8], lists[8][128], cnt[8], base;
+    uint32_t* const list = lists[threadIdx.x >> 5];
+    const int L = a.L, Lr = L - kt;
+    const uint32_t lm = (1u << (2 * Lr)) - 1u;
+    const uint8_t* X = cur ? q.zf[1] : q.zf[0];
+    uint8_t* Y = cur ? q.zf[0] : q.zf[1];
+    const int par = (int)cur, nxt = par ^ 1;
+    CellSrc<T> src;
+    src.h = par ? a.f[1][0] : a.f[0][0];
+    src.qx = par ? a.f[1][1] : a.f[0][1];
+    src.qy = par ? a.f[1][2] : a.f[0][2];
+    src.z = a.z;
+    const unsigned long long stamp = (unsigned long long)(epoch + 1u) << 32;
+    T* const oh = nxt ? a.f[1][0] : a.f[0][0];
+    T* const oqx = nxt ? a.f[1][1] : a.f[0][1];
+    T* const oqy = nxt ? a.f[1][2] : a.f[0][2];
+    const uint32_t t = threadIdx.x, lane = t & 31u;
+    const uint32_t ngroups = 1u << (2 * (kt - 1));
+    // whether a leaf takes the full update; a dry one is stored
+    auto wet = [&](uint32_t pk) {
+        const DryProbe d = dry_probe(pk);
+        bool y = dry5(src.h, d);
+        if (a.fm) y = y && !refined_nbr(a.Sb, d, L);
+        if (a.inflow_side >= 0) {
+            int64_t lo, hi;
+            y = y && !inlet_range(a, d.n, compact16(d.code), compact16(d.code >> 1), (1u << d.n) - 1u, lo, hi);
+        }
+        if (y) store_dry(a, oh, oqx, oqy, d);
+        return !y;
+    };
+    // the wet ones of each lane's cells (a bit each of pk, pk + 1, ...) to the
+    // queue: the CTA's in a row, by one addition to the queue's length, and a
+    // lane per leaf whichever found it
+    auto queue = [&](uint32_t bits, uint32_t pk) {
+        const uint32_t c = __popc(bits), before = warp_excl(c);
+        __syncthreads();                          // cnt read by all of the last call
+        if (lane == 31u) cnt[t >> 5] = before + c;
+        __syncthreads();
+        uint32_t w = 0u, total = 0u, every = 0u;
+        for (uint32_t j = 0u; j < 8u; ++j) {
+            const uint32_t k = cnt[j];
+            w += j < t >> 5 ? k : 0u;
+            total = j == t >> 5 ? k : total;
+            every += k;
+        }
+        if (every == 0u) return;                  // uniform over the CTA
+        if (t == 0u) base = atomicAdd(&st->nwet, every);
+        for (uint32_t k = 0u, o = before; k < 4u; ++k)
+            if (bits >> k & 1u) list[o++] = pk + k;
+        __syncwarp();
+        uint32_t i = lane;
+        uint32_t p = i < total ? list[i] : 0u;
+        uint64_t iC = lvl_off((int)(p >> kLeafShift)) + (p & kCodeMask);
+        LeafPre<T> r = {};
+        if (i < total) r = leaf_pre(a, src, iC);
+        __syncthreads();                          // base
+        w += base;
+        while (i < total) {
+            queue_leaf(a, w + i, p, iC, r, stamp);
+            i += 32u;
+            if (i < total) {
+                p = list[i];
+                iC = lvl_off((int)(p >> kLeafShift)) + (p & kCodeMask);
+                r = leaf_pre(a, src, iC);
+            }
+        }
+    };
+    uint32_t all = 0u, own = 0u;                  // leaves; those outside skipped tiles
+    for (uint32_t e = blockIdx.x; e < n; e += gridDim.x) {
+        uint32_t tile = MODE == kTravQuarters ? e >> 2 : e;
+        const uint32_t part = MODE == kTravQuarters ? e & 3u : 0u;
+        bool skip = false, ok = true;
+        if (LISTED) {
+            const uint32_t item = __ldg(work + e);
+            tile = item & 0x7FFFFFFFu;
+            skip = (item >> 31) != 0u;            // listed for its count
+        } else if (t < 7u) {
+            // the seven marks of the decision, one a thread, read together
+            const uint32_t xs = tile & kXBits & lm, ys = tile & kYBits & lm;
+            if (t == 0u) ok = X[tile] != 0;
+            else if (t == 1u) ok = Y[tile] != 0;
+            else if (t == 2u) ok = q.inlet[tile] == 0;
+            else if (t == 3u) ok = xs == 0u || X[mort_xm(tile)] != 0;
+            else if (t == 4u) ok = xs == (kXBits & lm) || X[mort_xp(tile)] != 0;
+            else if (t == 5u) ok = ys == 0u || X[mort_ym(tile)] != 0;
+            else ok = ys == (kYBits & lm) || X[mort_yp(tile)] != 0;
+        }
+        __syncthreads();                          // tb reused across tiles
+        load_tile_bits(Sb, L, kt, tile, tb);
+        const int l0 = tb.l0;
+        const bool whole = l0 <= Lr;              // one leaf covers the tile
+        if (!LISTED) {
+            const bool covered = l0 < Lr;
+            skip = __syncthreads_and(ok ? 1 : 0) != 0 && !covered;
+            if (t == 0u && part == 0u) q.act[tile] = skip ? 0 : (covered ? kActCovered : kActOwn);
+            if (t == 1u && part == 0u && !skip && !covered && ok) Y[tile] = 0;     // the step writes into it
+            if (skip && scount) {                 // uniform over the CTA
+                if (t == 0u && part == 0u) all += whole ? 1u : __ldg(scount + tile);
+                continue;
+            }
+        }
+        // the thread's group of four finest cells (in quarters: one cell of it)
+        const uint32_t g = MODE == kTravQuarters ? part * 64u + (t >> 2) : t;
+        const uint32_t cell = MODE == kTravQuarters ? t & 3u : 0u;
+        int l = L;
+        uint32_t c = 0u;
+        const uint32_t m0 = (tile << (2 * kt)) + 4u * g;
+        if (g < ngroups) {
+            l = group_level(tb, L, kt, g);
+            c = l == L ? 4u : ((m0 & ((1u << (2 * (L - l))) - 1u)) == 0u ? 1u : 0u);
+            if (MODE == kTravQuarters) c = cell < c ? 1u : 0u;
+        }
+        all += c;
+        if (skip) continue;
+        own += c;
+        if (part == 0u) {                         // uniform over the CTA
+            const bool big = t < ngroups && needs_decode_kernel(MODE == kTravQuarters ? group_level(tb, L, kt, t) : l, L);
+            if (__syncthreads_or(big ? 1 : 0) && t == 0u)
+                dlist[atomicAdd(&st->ndec, 1u)] = whole ? tile | ((uint32_t)(l0 + 1) << kWholeShift) : tile;
+        }
+        const uint32_t pk = ((uint32_t)l << kLeafShift | m0 >> (2 * (L - l))) + (l == L ? cell : 0u);
+        uint32_t bits = 0u;
+        bool deep = false;                        // four finest cells with water in each
+        if (c == 4u) {
+            T h0, h1, h2, h3;
+            Vec4<T>::load(src.h + lvl_off(L) + m0, h0, h1, h2, h3);
+            deep = !is_zero(h0) && !is_zero(h1) && !is_zero(h2) && !is_zero(h3);
+            bits = deep ? 15u : 0u;
+        }
+        if (c != 0u && !deep) {
+            bits = wet(pk) ? 1u : 0u;
+            if (c == 4u) {
+#pragma unroll
+                for (uint32_t k = 1u; k < 4u; ++k) bits |= wet(pk + k) ? 1u << k : 0u;
+            }
+        }
+        queue(bits, pk);
+    }
+    // the classify kernel's leaves, from the CTAs without a tile on
+    for (uint32_t b = (gridDim.x - 1u - blockIdx.x) * blockDim.x; b < nlist; b += gridDim.x * blockDim.x) {
+        const bool on = b + t < nlist;
+        const uint32_t pk = on ? __ldg(a.leaves + b + t) : 0u;
+        queue(on && wet(pk) ? 1u : 0u, pk);
+    }
+    all = warp_sum(all);
+    own = warp_sum(own);
+    if (lane == 0u) {
+        red[0][t >> 5] = all;
+        red[1][t >> 5] = own;
+    }
+    __syncthreads();
+    if (t < 2u) {
+        uint32_t s = 0u;
+        for (int w = 0; w < 8; ++w) s += red[t][w];
+        if (s != 0u) {
+            if (t == 0u) atomicAdd(&st->Mall, s);
+            else atomicAdd(&st->act_updates, (unsigned long long)s);
+        }
+    }
+}
+
 // CFL bound, write-back (with the prolongation of leaves of 4 or 16 finest
 // cells) and reductions of one updated wet leaf.
 template <typename T>
