@@ -182,6 +182,11 @@ class ClockSampler:
 # velocities x 3, 4 HLL faces x 56, bed source 8, update 20, friction 18,
 # CFL bound 9.
 FV1_WET_FLOP_PER_LEAF = 294
+# Of these the FP64 pipe executes only the sums, 24 a face (two faces a leaf
+# where both others are shared) and 19 in the update: products, roots and
+# reciprocals are integer instructions and a shared face is formed once, so the
+# arithmetic as written can run above the pipe's rate.
+FV1_WET_PIPE_PER_LEAF = 2 * 24 + 19
 # The FP64 pipe issues 2 thread-instructions per cycle per SM (ncu's peak for
 # DFMA); the update may use no FMA (each operation is rounded on its own, as
 # in the oracle), so its peak is one FLOP per instruction: 152 SMs x 2 x
@@ -222,6 +227,8 @@ def roofline(kernel, ms, r, args, pk, src):
                 "unit": "TFLOP/s", "frac": ach / FP64_PEAK_TFLOPS, "traffic": traffic,
                 "measured_fp64_tflops": meas, "frac_of_measured_fp64": (ach / meas) if meas else None,
                 "units_per_launch": r["wet_per_step"], "flop_per_unit": FV1_WET_FLOP_PER_LEAF,
+                "fp64_pipe_per_unit": FV1_WET_PIPE_PER_LEAF,
+                "fp64_pipe_frac": ach / FP64_PEAK_TFLOPS * FV1_WET_PIPE_PER_LEAF / FV1_WET_FLOP_PER_LEAF,
                 "peak_source": "derived: FP64 pipe, 2 instructions/clk/SM x 152 SMs x 2.07 GHz, "
                                "1 FLOP per instruction (no FMA)"}
     return {"kernel": kernel, "bound": None, "achieved": None, "peak": pk["hbm_gbs"], "unit": "GB/s",
