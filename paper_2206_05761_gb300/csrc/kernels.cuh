@@ -2661,18 +2661,18 @@ __device__ __forceinline__ void face_of(const Phys<T>& P, int s, const Cell<T>& 
 }
 
 // The face on side s of the leaf (n, i, j) whose same-level neighbour is
-// refined.  Depth first over the halves (first half: lower j on x faces,
-// lower i on y faces): half r of level m lies between the own-side cell and
-// the neighbour cell of level m that touch it; a finished second half is
-// averaged with the pending first half of its level, one level up, until
-// the face itself is reached.  The walk visits each half face of the finite
-// tree once.
+// refined (m0 = n, r0 = 0), or its part r0 of level m0 > n.  Depth first over
+// the halves (first half: lower j on x faces, lower i on y faces): half r of
+// level m lies between the own-side cell and the neighbour cell of level m
+// that touch it; a finished second half is averaged with the pending first
+// half of its level, one level up, until the part itself is reached.  The walk
+// visits each half face of the finite tree once.
 template <typename T>
 __device__ __noinline__ void matched_face(const StepArgs<T>& a, const CellSrc<T>& src, int s, int n, uint32_t i,
-                                          uint32_t j, T F[3], T& own2) {
+                                          uint32_t j, int m0, uint32_t r0, T F[3], T& own2) {
     T pend[kMaxL][4];                     // pending first halves, by level - n - 1
-    int m = n + 1;
-    uint32_t r = 0u;
+    int m = m0;
+    uint32_t r = r0;
     for (;;) {
         const bool xf = s <= 1;
         uint32_t oi, oj, ni, nj;
@@ -2694,14 +2694,14 @@ __device__ __noinline__ void matched_face(const StepArgs<T>& a, const CellSrc<T>
         const uint64_t base = lvl_off(m);
         T v[4];
         face_of(a.P, s, fetch(src, base + morton2(oi, oj)), fetch(src, base + morton2(ni, nj)), v, v[3]);
-        while (r & 1u) {                          // a second half: close its pair
+        while (m > m0 && (r & 1u)) {              // a second half: close its pair
             const T* p = pend[m - n - 1];
 #pragma unroll
             for (int q = 0; q < 4; ++q) v[q] = half(p[q] + v[q]);
             --m;
             r >>= 1;
         }
-        if (m == n) {
+        if (m == m0) {
             F[0] = v[0];
             F[1] = v[1];
             F[2] = v[2];
@@ -2712,6 +2712,14 @@ __device__ __noinline__ void matched_face(const StepArgs<T>& a, const CellSrc<T>
         for (int q = 0; q < 4; ++q) pend[m - n - 1][q] = v[q];
         r += 1u;                                  // on to its second half
     }
+}
+
+// Whether half r of the face on side s of (n, i, j) meets a refined cell of
+// level n + 1.
+__device__ __forceinline__ bool half_refined(const uint32_t* Sb, int L, int s, int n, uint32_t i, uint32_t j, uint32_t r) {
+    const uint32_t ni = s == 0 ? 2u * i - 1u : (s == 1 ? 2u * i + 2u : 2u * i + r);
+    const uint32_t nj = s == 2 ? 2u * j - 1u : (s == 3 ? 2u * j + 2u : 2u * j + r);
+    return n + 1 < L && sig_bit(Sb, n + 1, morton2(ni, nj));
 }
 
 // One face of a queued leaf: the ghost at the domain edge, the matched face
@@ -2729,7 +2737,7 @@ __device__ __forceinline__ void leaf_face(const StepArgs<T>& a, const CellSrc<T>
     const uint32_t nj = s == 2 ? j - 1u : (s == 3 ? j + 1u : j);
     const uint32_t nc = morton2(ni, nj);
     if (n < a.L && sig_bit(a.Sb, n, nc)) {
-        matched_face(a, src, s, n, i, j, F, own2);
+        matched_face(a, src, s, n, i, j, n, 0u, F, own2);
         return;
     }
     face_of(a.P, s, C, fetch(src, lvl_off(n) + nc), F, own2);
@@ -2823,67 +2831,66 @@ __device__ __forceinline__ AxisProbe axis_probe(uint32_t pk, bool y) {
     return d;
 }
 
-// Face s (0 W, 1 E, 2 S, 3 N) of queued leaf w into the face buffer.
-template <typename T, bool FM>
+// A face of queued leaf w into the face buffer (its other side's squared depth
+// aside); which arrays it took.
+template <typename T>
+__device__ __forceinline__ int store_face(T* face, size_t cap, int s, uint32_t w, const T F[3], T own2) {
+    const int k = s == 0 ? kFaceW : (s == 1 ? kFaceE : (s == 2 ? kFaceS : kFaceN));
+    *pair_at(face, cap, k, w) = make_pair2(F[0], F[1]);
+    *pair_at(face, cap, k + 2, w) = make_pair2(F[2], own2);
+    return k;
+}
+// Face s (0 W, 1 E, 2 S, 3 N) of queued leaf w, not toward a refined cell, into
+// the face buffer.
+template <typename T>
 __device__ __forceinline__ void queued_face(const StepArgs<T>& a, const CellSrc<T>& src, uint32_t tag, bool ok,
                                             uint32_t w, int s, const AxisProbe& d) {
     const size_t cap = a.fcap;
     const bool yface = s >= 2, right = (s & 1) == 0;      // right: the leaf is the right side
     const bool edge = right ? d.endM : d.endP;
     const uint32_t iX = edge ? d.iC : (right ? d.iM : d.iP);
-    T F[3], own2, other2 = T(0);
-    if (FM && !edge && d.n < a.L && sig_bit(a.Sb, d.n, iX - (uint32_t)lvl_off(d.n))) {
-        // toward a refined neighbour: the walk over the finer halves (the
-        // face's other side belongs to no leaf)
-        matched_face(a, src, s, d.n, compact16(d.code), compact16(d.code >> 1), F, own2);
-    } else {
-        // the two sides' records by queue slot: normal and tangential
-        // velocity, free surface and bed (the sides' order is a choice of
-        // slots, not of values)
-        const unsigned long long m = __ldg(a.mark + iX), mc = __ldg(a.mark + d.iC);
-        const bool queued = (uint32_t)(m >> 32) == tag;   // (at an edge: the leaf itself)
-        const uint32_t wx = queued ? (uint32_t)m & ~kUnsafe : w;
-        const uint32_t wL = right ? wx : w, wR = right ? w : wx;
-        const T* const rec = a.face + kLeafUV * cap;
-        const uint32_t on = yface ? 1u : 0u;
-        T nL = rec[2 * (size_t)wL + on], tL = rec[2 * (size_t)wL + (on ^ 1u)];
-        T nR = rec[2 * (size_t)wR + on], tR = rec[2 * (size_t)wR + (on ^ 1u)];
-        typename Pair2<T>::V ezL = *pair_at(a.face, cap, kLeafEZ, wL), ezR = *pair_at(a.face, cap, kLeafEZ, wR);
-        bool safe = ok && !(((uint32_t)mc | (queued ? (uint32_t)m : 0u)) & kUnsafe);
-        if (!queued) {
-            const Cell<T> X = fetch(src, iX);
-            T u, v;
-            velocity(X, a.P.tol, u, v);
-            safe = safe && cell_window(X.h, X.z, u, v);
-            const T xn = yface ? v : u, xt = yface ? u : v;
-            if (right) {
-                nL = xn;
-                tL = xt;
-                ezL = make_pair2(eta_of(X.h, X.z), X.z);
-            } else {
-                nR = xn;
-                tR = xt;
-                ezR = make_pair2(eta_of(X.h, X.z), X.z);
-            }
-        } else if (edge) {
-            // the ghost's velocity is the leaf's, the normal part reversed at
-            // a wall (a dry leaf's is +0 either way)
-            const int wall = s == 0 ? a.bc_ref[0] : (s == 1 ? a.bc_ref[1] : (s == 2 ? a.bc_ref[2] : a.bc_ref[3]));
-            if (wall && ge_nonneg(__ldg(src.h + d.iC), a.P.tol)) {
-                if (right) nL = -nL;
-                else nR = -nR;
-            }
+    // the two sides' records by queue slot: normal and tangential
+    // velocity, free surface and bed (the sides' order is a choice of
+    // slots, not of values)
+    const unsigned long long m = __ldg(a.mark + iX), mc = __ldg(a.mark + d.iC);
+    const bool queued = (uint32_t)(m >> 32) == tag;   // (at an edge: the leaf itself)
+    const uint32_t wx = queued ? (uint32_t)m & ~kUnsafe : w;
+    const uint32_t wL = right ? wx : w, wR = right ? w : wx;
+    const T* const rec = a.face + kLeafUV * cap;
+    const uint32_t on = yface ? 1u : 0u;
+    T nL = rec[2 * (size_t)wL + on], tL = rec[2 * (size_t)wL + (on ^ 1u)];
+    T nR = rec[2 * (size_t)wR + on], tR = rec[2 * (size_t)wR + (on ^ 1u)];
+    typename Pair2<T>::V ezL = *pair_at(a.face, cap, kLeafEZ, wL), ezR = *pair_at(a.face, cap, kLeafEZ, wR);
+    bool safe = ok && !(((uint32_t)mc | (queued ? (uint32_t)m : 0u)) & kUnsafe);
+    if (!queued) {
+        const Cell<T> X = fetch(src, iX);
+        T u, v;
+        velocity(X, a.P.tol, u, v);
+        safe = safe && cell_window(X.h, X.z, u, v);
+        const T xn = yface ? v : u, xt = yface ? u : v;
+        if (right) {
+            nL = xn;
+            tL = xt;
+            ezL = make_pair2(eta_of(X.h, X.z), X.z);
+        } else {
+            nR = xn;
+            tR = xt;
+            ezR = make_pair2(eta_of(X.h, X.z), X.z);
         }
-        T hl, hr;
-        hll_face(a.P.g, a.P.hg, a.P.tol, ezL.x, ezL.y, nL, tL, ezR.x, ezR.y, nR, tR, safe, F, hl, hr);
-        const T l2 = prod(hl, hl), r2 = prod(hr, hr);
-        own2 = right ? r2 : l2;
-        other2 = r2;
+    } else if (edge) {
+        // the ghost's velocity is the leaf's, the normal part reversed at
+        // a wall (a dry leaf's is +0 either way)
+        const int wall = s == 0 ? a.bc_ref[0] : (s == 1 ? a.bc_ref[1] : (s == 2 ? a.bc_ref[2] : a.bc_ref[3]));
+        if (wall && ge_nonneg(__ldg(src.h + d.iC), a.P.tol)) {
+            if (right) nL = -nL;
+            else nR = -nR;
+        }
     }
-    const int k = s == 0 ? kFaceW : (s == 1 ? kFaceE : (s == 2 ? kFaceS : kFaceN));
-    *pair_at(a.face, cap, k, w) = make_pair2(F[0], F[1]);
-    *pair_at(a.face, cap, k + 2, w) = make_pair2(F[2], own2);
-    if (!right) a.face[(k + 4) * cap + w] = other2;
+    T F[3], hl, hr;
+    hll_face(a.P.g, a.P.hg, a.P.tol, ezL.x, ezL.y, nL, tL, ezR.x, ezR.y, nR, tR, safe, F, hl, hr);
+    const T l2 = prod(hl, hl), r2 = prod(hr, hr);
+    const int k = store_face(a.face, cap, s, w, F, right ? r2 : l2);
+    if (!right) a.face[(k + 4) * cap + w] = r2;
 }
 
 // A warp takes 32 leaves (16 where the queue is too short to give every warp
@@ -2898,6 +2905,13 @@ __device__ __forceinline__ void queued_face(const StepArgs<T>& a, const CellSrc<
 // FV1, L=10) take 133 us, in which the FP64 pipe's 24 sums a face fill 78 %
 // of the cycles and 780 integer instructions 66 %; 321 us with every operation
 // on the FP64 pipe and two faces per thread.
+//
+// FM: faces toward a refined neighbour are gathered too (all four sides; their
+// neighbour is no leaf, so nobody shares them) and taken last, four lanes a
+// face: a lane walks a quarter of it, or where a half meets no finer cell the
+// even lane takes the half; the lanes' values are averaged in the order of the
+// whole walk.  A warp's every round had waited for the longest walk of one of
+// its lanes: closed 512 x 512 basin, 48 steps 3288 -> 2704 us.
 template <typename T, bool FM = false>
 __device__ __forceinline__ void fv1_faces_body(const StepArgs<T>& a, Blk B) {
     DevState* st = a.st;
@@ -2916,9 +2930,11 @@ __device__ __forceinline__ void fv1_faces_body(const StepArgs<T>& a, Blk B) {
     src.z = a.z;
     const bool ok = const_window(a.P.g, a.P.tol);
     __shared__ uint8_t lists[8][64];              // (blocks of up to 8 warps)
+    __shared__ uint8_t walks[FM ? 8 : 1][128];
     uint8_t* const list = lists[warp];
+    uint8_t* const walk = walks[FM ? warp : 0u];
     for (uint32_t base = (B.id * wpb + warp) * per; base < nq; base += warps * per) {
-        uint32_t n = 0u;                          // faces gathered
+        uint32_t n = 0u, nwalk = 0u;              // faces gathered
 #pragma unroll 1
         for (uint32_t t0 = 0u; t0 < 2u * per + n; t0 += 32u) {
             const uint32_t t = t0 + lane;
@@ -2942,12 +2958,55 @@ __device__ __forceinline__ void fv1_faces_body(const StepArgs<T>& a, Blk B) {
                 if (on)
                     slots_at(a.face, a.fcap, base + l)[s == 1 ? 0 : 1] =
                         miss ? base + l : ((uint32_t)mm & ~kUnsafe) | kShared;
-                const uint32_t m = __ballot_sync(0xffffffffu, miss);
-                if (miss) list[n + __popc(m & below)] = (uint8_t)(s == 1 ? l : l | 32u);
+                bool own = miss;
+                if constexpr (FM) {
+                    // toward a refined cell: this lane's face, the opposite one
+                    const uint32_t base_n = (uint32_t)lvl_off(d.n);
+                    const bool fine = on && d.n < a.L;
+                    const bool rp = fine && !d.endP && sig_bit(a.Sb, d.n, d.iP - base_n);
+                    const bool rm = fine && !d.endM && sig_bit(a.Sb, d.n, d.iM - base_n);
+                    const uint32_t mp = __ballot_sync(0xffffffffu, rp), mr = __ballot_sync(0xffffffffu, rm);
+                    if (rp) walk[nwalk + __popc(mp & below)] = (uint8_t)(l | (uint32_t)s << 5);
+                    nwalk += __popc(mp);
+                    if (rm) walk[nwalk + __popc(mr & below)] = (uint8_t)(l | (uint32_t)(s - 1) << 5);
+                    nwalk += __popc(mr);
+                    own = miss && !rm;
+                    on = on && !rp;
+                }
+                const uint32_t m = __ballot_sync(0xffffffffu, own);
+                if (own) list[n + __popc(m & below)] = (uint8_t)(s == 1 ? l : l | 32u);
                 n += __popc(m);
             }
-            if (on) queued_face<T, FM>(a, src, tag, ok, base + l, s, d);
+            if (on) queued_face<T>(a, src, tag, ok, base + l, s, d);
             __syncwarp();                         // the list before its readers and the next writers
+        }
+        if constexpr (FM) {
+#pragma unroll 1
+            for (uint32_t t0 = 0u; t0 < 4u * nwalk; t0 += 32u) {
+                const uint32_t k = (t0 + lane) >> 2, q = lane & 3u;
+                const bool on = k < nwalk;
+                const uint32_t e = on ? walk[k] : 0u, w = base + (e & 31u);
+                const int s = (int)(e >> 5);
+                bool quarter = false;                 // this half is in quarters
+                T F[4] = {T(0), T(0), T(0), T(0)};
+                if (on) {
+                    const uint32_t pk = a.wet[w], code = pk & kCodeMask;
+                    const int ln = (int)(pk >> kLeafShift);
+                    const uint32_t i = compact16(code), j = compact16(code >> 1);
+                    quarter = half_refined(a.Sb, a.L, s, ln, i, j, q >> 1);
+                    if (quarter || !(q & 1u))
+                        matched_face(a, src, s, ln, i, j, ln + (quarter ? 2 : 1), quarter ? q : q >> 1, F, F[3]);
+                }
+#pragma unroll
+                for (int c = 0; c < 4; ++c) {
+                    const T f = __shfl_xor_sync(0xffffffffu, F[c], 1);
+                    if (quarter) F[c] = half(F[c] + f);
+                    const T g = __shfl_xor_sync(0xffffffffu, F[c], 2);
+                    F[c] = half(F[c] + g);
+                }
+                if (on && q == 0u) store_face(a.face, (size_t)a.fcap, s, w, F, F[3]);
+            }
+            __syncwarp();
         }
     }
 }
