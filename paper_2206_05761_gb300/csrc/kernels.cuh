@@ -650,6 +650,7 @@ __device__ __forceinline__ void encode_tile(const EncodeArgs<T, NF>& a, int ls, 
     }
     // bit j NF + q: a detail of 0 passes the threshold of level ls-1-j, quantity q
     const uint32_t zbits = __ballot_sync(0xffffffffu, zp);
+    __syncwarp();                                     // sthr before its readers (a vote orders no memory)
     bool nz = false, same = true;                     // same: the warp's cells have held one value so far
     T one[NF];
 #pragma unroll
