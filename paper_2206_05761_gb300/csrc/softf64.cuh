@@ -154,7 +154,7 @@ __host__ __device__ __forceinline__ uint64_t mul_bits(uint32_t al, uint32_t ah, 
 #ifdef __CUDA_ARCH__
     asm("{.reg .u32 t; shl.b32 t, %2, 31; add.cc.u32 t, t, t; addc.cc.u32 t, %4, 0x7fffffff; addc.cc.u32 %0, %2, 0; "
         "addc.u32 %1, %3, %5;}"
-        : "=r"(rl), "=r"(rh) : "r"(kl), "r"(kh), "r"(f), "r"(e));
+        : "=&r"(rl), "=r"(rh) : "r"(kl), "r"(kh), "r"(f), "r"(e));   // (%0 is written before kh and e are read)
 #else
     const uint64_t r = (uint64_t)f + 0x7FFFFFFFu + (kl & 1u);
     const uint64_t k = ((uint64_t)(kh + e) << 32 | kl) + (r >> 32);

@@ -29,3 +29,58 @@ def test_the_encode_orders_its_thresholds_before_they_are_read():
     read = b.index("sthr[w][0]", write)
     between = b[write:read]
     assert "__syncwarp(" in between or "__syncthreads(" in between
+
+
+def asm_statements(src):
+    """(text, outputs, inputs) of every asm statement: operands as constraint
+    strings in order."""
+    out = []
+    for m in re.finditer(r"\basm\b(?:\s+volatile)?\s*\(", src):
+        k, depth, quote = m.end(), 1, False
+        while depth:
+            c = src[k]
+            if c == '"':
+                quote = not quote
+            elif not quote:
+                depth += {"(": 1, ")": -1}.get(c, 0)
+            k += 1
+        stmt = src[m.end():k - 1]
+        # outside of strings, colons separate text, outputs, inputs, clobbers
+        parts, cur, quote = [], "", False
+        for c in stmt:
+            if c == '"':
+                quote = not quote
+            if c == ":" and not quote:
+                parts.append(cur)
+                cur = ""
+            else:
+                cur += c
+        parts.append(cur)
+        strings = [re.findall(r'"([^"]*)"', x) for x in parts]
+        strings += [[]] * (3 - len(strings))
+        out.append(("".join(strings[0]), strings[1], strings[2]))
+    return out
+
+
+def test_outputs_written_before_an_input_is_read_share_no_register():
+    checked = 0
+    for name in sorted(os.listdir(CSRC)):
+        if not name.endswith((".cuh", ".cu", ".h")):
+            continue
+        for text, outs, ins in asm_statements(source(name)):
+            stmts = [re.sub(r"\.reg[^;]*", "", t) for t in text.replace("\\n", "").replace("\\t", "").split(";")]
+            uses = [[int(x) for x in re.findall(r"%(\d+)", t)] for t in stmts]
+            inputs = range(len(outs), len(outs) + len(ins))
+            for o, mark in enumerate(outs):
+                first = [i for i, u in enumerate(uses) if o in u]
+                later = [x for u in uses[first[0] + 1:] for x in u if x in inputs]
+                checked += 1
+                if later:
+                    assert "&" in mark, (name, text, o, mark)
+    assert checked > 10
+
+
+def test_the_reader_of_asm_statements_sees_the_fault():
+    bad = 'asm("add.cc.u32 %0, %2, 0; addc.u32 %1, %3, 0;" : "=r"(a), "=r"(b) : "r"(c), "r"(d));'
+    (text, outs, ins), = asm_statements(bad)
+    assert outs == ["=r", "=r"] and ins == ["r", "r"] and text.count(";") == 2
