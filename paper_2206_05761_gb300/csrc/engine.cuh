@@ -165,7 +165,6 @@ class EngineT final : public Engine {
                 cudaMemsetAsync(f_[0][q], 0, lvl_off(L_) * sizeof(T), stream_);
                 cudaMemsetAsync(f_[1][q], 0, H_ * sizeof(T), stream_);
             }
-        pdl_ = std::getenv("HWFV1_NO_PDL") == nullptr;
         {
             std::vector<uint8_t> inl(ntiles_, 0);
             const int side = step_args().inflow_side;
@@ -225,6 +224,10 @@ class EngineT final : public Engine {
         }
         lk(k_flag, grid_for(words_), 256, Tz_, Cz_, nullptr, Sz_, L_, predict(), close(),
            (const DevState*)nullptr, (uint32_t*)nullptr);
+        // The bed's kernels read from addresses that do not rest on a word read
+        // after pdl_wait, so that nothing but the launch order keeps their loads
+        // behind the kernel ahead: programmatic launches begin with the steps.
+        pdl_ = std::getenv("HWFV1_NO_PDL") == nullptr;
         // leaf count of each tile holding the bed's flags alone (skipped tiles)
         if (!alloc(&scount_, (size_t)ntiles_ * sizeof(uint32_t))) return oom();
         k_static_counts<<<(ntiles_ + kTilesPerCta - 1) / kTilesPerCta, 256, 0, stream_>>>(Sz_, L_, kt_, ntiles_,
@@ -1026,8 +1029,8 @@ class EngineT final : public Engine {
     // the last step formed it on the spot
     void ensure_sig_words() {
         if (sb_valid_) return;
-        lk(k_flag, grid_for(words_), 256, Tb_, Cb_, Sz_, Sb_, L_, predict(), close(),
-           (const DevState*)nullptr, (uint32_t*)nullptr);
+        // (an ordinary launch: without a state to read first, see init)
+        k_flag<<<grid_for(words_), 256, 0, stream_>>>(Tb_, Cb_, Sz_, Sb_, L_, predict(), close(), nullptr, nullptr);
         sb_valid_ = true;
     }
     // `learned`: the flags come from the learned look-ahead, whose skipped
@@ -1615,7 +1618,7 @@ class EngineT final : public Engine {
     uint32_t* scount_ = nullptr;        // per tile: leaves when it holds the bed's flags alone
     uint32_t* work_ = nullptr;          // the traversal's list of tiles to treat one warp each
     bool quiet_on_ = false;
-    bool pdl_ = true;             // programmatic dependent launch in the step chain
+    bool pdl_ = false;            // programmatic dependent launch in the step chain
     bool sb_valid_ = true;        // Sb_ holds the S of the last step (else formed on the spot)
     std::vector<std::pair<const char*, cudaEvent_t>>* prof_ = nullptr;   // profile_step's events
     bool prof_external_ = false;          // events recorded as graph nodes (under capture)

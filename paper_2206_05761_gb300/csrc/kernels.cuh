@@ -21,11 +21,11 @@ template <typename T> struct Vec4;
 // pass takes half the load and store instructions of 128-bit ones.  Every
 // level starts on a multiple of 64 elements and the groups on multiples of
 // four, so p is 32-byte aligned.  Decode of water columns at L=11 (100 MB
-// written): 38 to 29 us.
+// written): 38 to 29 us.  (volatile: no load moves above pdl_wait.)
 template <> struct Vec4<double> {
     static __device__ __forceinline__ void load(const double* p, double& a, double& b, double& c,
                                                 double& d) {
-        asm("ld.global.nc.v4.f64 {%0, %1, %2, %3}, [%4];" : "=d"(a), "=d"(b), "=d"(c), "=d"(d) : "l"(p));
+        asm volatile("ld.global.nc.v4.f64 {%0, %1, %2, %3}, [%4];" : "=d"(a), "=d"(b), "=d"(c), "=d"(d) : "l"(p));
     }
     static __device__ __forceinline__ void store(double* p, double a, double b, double c, double d) {
         asm volatile("st.global.v4.f64 [%0], {%1, %2, %3, %4};" ::"l"(p), "d"(a), "d"(b), "d"(c), "d"(d) : "memory");

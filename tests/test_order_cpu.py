@@ -84,3 +84,22 @@ def test_the_reader_of_asm_statements_sees_the_fault():
     bad = 'asm("add.cc.u32 %0, %2, 0; addc.u32 %1, %3, 0;" : "=r"(a), "=r"(b) : "r"(c), "r"(d));'
     (text, outs, ins), = asm_statements(bad)
     assert outs == ["=r", "=r"] and ins == ["r", "r"] and text.count(";") == 2
+
+
+def test_no_load_can_move_above_the_wait_for_the_kernel_ahead():
+    # an asm statement that loads is volatile, as the wait is: the compiler
+    # keeps volatile statements in order
+    loads = 0
+    for name in ("common.cuh", "kernels.cuh", "skip.cuh"):
+        for m in re.finditer(r"\basm\b\s*(volatile)?\s*\(\s*\"(?:ld\.|\{?\s*ld\.)", source(name)):
+            loads += 1
+            assert m.group(1), (name, source(name)[m.start():m.start() + 80])
+    assert loads >= 4
+    # a launch whose kernel gets no state to read first is an ordinary one: the
+    # bed's encode and flags while the handle is made, the flags on demand
+    src = source("engine.cuh")
+    assert re.search(r"bool pdl_ = false;", src)
+    init = body_of(src, "hwfv1_status init(")
+    assert init.index("pdl_ = ") > max(init.index("encode_passes("), init.index("lk(k_flag"))
+    assert "lk(" not in init[init.index("pdl_ = "):]
+    assert "lk(" not in body_of(src, "void ensure_sig_words(")
