@@ -296,7 +296,9 @@ struct DevState {
     unsigned long long leaf_updates;  // leaves updated, summed over the steps taken
     unsigned long long wet_updates;   // of them, leaves that took the full FV1 update
     unsigned long long act_updates;   // of them, leaves outside skipped (quiescent) tiles
-    uint32_t epoch;                   // completed steps (never reset; tags the face stamps)
+    uint32_t epoch;                   // number of the queue of full updates: counts up whenever the queue
+                                      // is emptied (never reset; tags the face stamps, so that none of an
+                                      // earlier queue's is taken, a step's that was never completed included)
     uint32_t enc_ticket;              // finished CTAs of the fused last encode passes
     uint32_t dec_ticket;              // finished CTAs of the fused decode + finish
     unsigned long long in_bits[3];    // max |h|, |qx|, |qy| of fields coming in (set_fields; 0 between calls)

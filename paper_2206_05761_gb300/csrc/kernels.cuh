@@ -3275,10 +3275,12 @@ __device__ inline double inflow_Q(const FinishArgs& a, double t) {
 __device__ __forceinline__ double thr4_of(double t) { return ge_nonneg(t, 0x1p-1020) ? t * 4.0 : -1.0; }
 __device__ __forceinline__ float thr4_of(float t) { return t >= 0x1p-124f ? t * 4.0f : -1.0f; }
 
-// With t, t_end, dt, s_max and the inflow at t given (no reload of what the
-// caller holds).
+// With t, t_end, dt, s_max, the inflow at t and the new queue's number given (no
+// reload of what the caller holds).  Every way to a step that may take place
+// passes here, also the ones that leave a step half done (a new state or end
+// time after the update of leaves), so the queue is emptied and numbered here.
 __device__ inline void prepare_vals(DevState* st, const FinishArgs& a, double t, double t_end, double dt,
-                                    const double (&smax)[3], double Q) {
+                                    const double (&smax)[3], double Q, uint32_t epoch) {
     for (int k = threadIdx.x; k < 3 * a.L; k += blockDim.x) {
         const int n = k / 3, q = k - 3 * n;
         const double sm = q == 0 ? smax[0] : (q == 1 ? smax[1] : smax[2]);
@@ -3316,6 +3318,7 @@ __device__ inline void prepare_vals(DevState* st, const FinishArgs& a, double t,
             st->rx0f = (float)dt_use / (float)a.lx;
             st->ry0f = (float)dt_use / (float)a.ly;
             st->nwet = 0u;
+            st->epoch = epoch;
             st->rmin_bits = kInfBits;
             st->max_bits[0] = st->max_bits[1] = st->max_bits[2] = 0ull;
             st->speed_bits[0] = st->speed_bits[1] = st->speed_bits[2] = 0ull;
@@ -3324,7 +3327,9 @@ __device__ inline void prepare_vals(DevState* st, const FinishArgs& a, double t,
 }
 __device__ inline void prepare_step(DevState* st, const FinishArgs& a) {
     const double smax[3] = {st->smax[0], st->smax[1], st->smax[2]};
-    prepare_vals(st, a, st->t, st->t_end, st->dt, smax, inflow_Q(a, st->t));
+    const uint32_t epoch = st->epoch + 1u;
+    __syncthreads();                 // read by every thread before one writes it
+    prepare_vals(st, a, st->t, st->t_end, st->dt, smax, inflow_Q(a, st->t), epoch);
 }
 
 // next timestep: CFL * (min CFL bound), capped at dt_max (+inf when dry)
@@ -3359,6 +3364,7 @@ __device__ __forceinline__ void finish_body(DevState* st, const FinishArgs& a) {
     const unsigned long long rmin = __ldcg(&st->rmin_bits);
     const unsigned long long mb[3] = {__ldcg(&st->max_bits[0]), __ldcg(&st->max_bits[1]), __ldcg(&st->max_bits[2])};
     const double t = __ldcg(&st->t) + __ldcg(&st->dt_use), t_end = __ldcg(&st->t_end);
+    const uint32_t epoch = __ldcg(&st->epoch) + 1u;
     if (!active) return;
     __shared__ double s_q[2], s_Q;
     const int warp = (int)(threadIdx.x >> 5), nw = (int)((blockDim.x + 31u) >> 5);
@@ -3367,13 +3373,12 @@ __device__ __forceinline__ void finish_body(DevState* st, const FinishArgs& a) {
     const bool counts = threadIdx.x == (nw > 1 ? 32u : 0u);
     unsigned long long lu = 0ull, au = 0ull, wu = 0ull;
     long long step = 0;
-    uint32_t epoch = 0u, cur = 0u;
+    uint32_t cur = 0u;
     if (counts) {
         lu = __ldcg(&st->leaf_updates) + __ldcg(&st->Mall);
         au = __ldcg(&st->act_updates) + __ldcg(&st->M);
         wu = __ldcg(&st->wet_updates) + __ldcg(&st->nwet);
         step = __ldcg(&st->step) + 1;
-        epoch = __ldcg(&st->epoch) + 1u;
         cur = __ldcg(&st->cur) ^ 1u;
     }
     if ((threadIdx.x & 31u) == 0u) {
@@ -3392,7 +3397,6 @@ __device__ __forceinline__ void finish_body(DevState* st, const FinishArgs& a) {
         st->t = t;
         st->cur = cur;
         st->step = step;
-        st->epoch = epoch;
         st->leaf_updates = lu;
         st->act_updates = au;
         st->wet_updates = wu;
@@ -3412,7 +3416,7 @@ __device__ __forceinline__ void finish_body(DevState* st, const FinishArgs& a) {
         if (!(finite_bits(dt) && finite_bits(smax[0]) && finite_bits(smax[1]) && finite_bits(smax[2])))
             st->err |= kErrNonFinite;
     }
-    prepare_vals(st, a, t, t_end, dt, smax, s_Q);
+    prepare_vals(st, a, t, t_end, dt, smax, s_Q, epoch);
 }
 
 // Decode-back followed, in its last CTA to finish, by the time advance (one

@@ -1,0 +1,64 @@
+"""A step begun by its phases and left before its decode must leave nothing
+behind: whatever replaces the state or starts the next step, the result is
+that of a handle that never saw the abandoned step, bit for bit."""
+import numpy as np
+import pytest
+
+import synth
+
+pytestmark = pytest.mark.gpu
+
+L = 7
+
+
+def _begin(sim):
+    """Every phase up to the update."""
+    sim.encode()
+    sim.flag()
+    sim.traverse()
+    sim.fv1()
+
+
+def _equal(a, b, leaves=True):
+    ga, gb = a.fields(), b.fields()
+    for q in ("h", "qx", "qy"):
+        assert np.array_equal(ga[q], gb[q]), q
+    if leaves:
+        assert np.array_equal(a.leaves(), b.leaves())
+    assert a.time()[:2] == b.time()[:2]
+
+
+@pytest.mark.parametrize("matched", [False, True])
+@pytest.mark.parametrize("how", ["set_fields", "load", "uniform"])
+@pytest.mark.parametrize("precision", [64, 32])
+def test_a_new_state_after_an_abandoned_step(matched, how, precision):
+    from paper_2206_05761_gb300.sim import Simulation
+    p, f = synth.bumpy_dam_break(L=L, eps=1e-3, seed=5)
+    g = synth.bumpy_dam_break(L=L, eps=1e-3, seed=9)[1]
+    # the first state is rough, every finest cell a leaf; the second is coarse in part
+    p = dict(p, flux_match=matched)
+    rough = dict(f)
+    rng = np.random.default_rng(1)
+    rough["h"] = rng.uniform(0.5, 1.0, f["h"].shape)
+    if precision == 32:
+        g = {k: v.astype(np.float32).astype(np.float64) for k, v in g.items()}
+    other = dict(h=g["h"], qx=g["qx"], qy=g["qy"], z=f["z"])
+    a = Simulation(p, dict(rough, z=f["z"]), precision)
+    b = Simulation(p, other, precision)
+    _begin(a)
+    if how == "load":
+        a.load(b.save())
+    else:
+        a.set_fields(other)
+    a.set_time(0.0, 1e-3)
+    b.set_time(0.0, 1e-3)
+    for s in (a, b):
+        if how == "uniform":
+            s.advance_uniform(max_steps=2)
+        else:
+            s.advance(max_steps=2)
+    if how != "uniform":
+        assert 4 ** L > len(b.leaves()) > 0
+    _equal(a, b, leaves=how != "uniform")
+    a.close()
+    b.close()
