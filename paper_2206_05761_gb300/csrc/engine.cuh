@@ -288,6 +288,7 @@ class EngineT final : public Engine {
     }
     hwfv1_status step() override {
         if (hwfv1_status r = phase_guard("step"); r != HWFV1_OK) return r;
+        new_queue();
         launch_fv1();
         return check("step");
     }
@@ -631,6 +632,7 @@ class EngineT final : public Engine {
         cudaEvent_t e0;
         if (cudaEventCreate(&e0) != cudaSuccess) return fail(HWFV1_ERR_CUDA, "event");
         const bool use_graph = std::getenv("HWFV1_NO_GRAPH") == nullptr;
+        new_queue();
         // the step the schedule takes next (the plain step outside the skip)
         const int pkind = skipmode_ ? skip_kind(lstep_++) : kStepPlain;
         hwfv1_status r = HWFV1_OK;
@@ -689,6 +691,7 @@ class EngineT final : public Engine {
         if (reps < 1 || !ms) return fail(HWFV1_ERR_INVALID_SPEC, "profile_update: reps >= 1 and ms");
         if (hwfv1_status r = phase_guard("profile_update"); r != HWFV1_OK) return r;
         const bool onfly = onfly_flags();
+        new_queue();
         launch_encode();
         if (!onfly) launch_flag();
         launch_traverse(false, onfly);
@@ -1513,6 +1516,8 @@ class EngineT final : public Engine {
         }
         k_init_state<<<1, 64, 0, stream_>>>(st_, fin_args(), set_dt);
     }
+
+    void new_queue() { k_new_queue<<<1, 1, 0, stream_>>>(st_); }
 
     hwfv1_status read_state(DevState* s) {
         if (cudaMemcpyAsync(s, st_, sizeof *s, cudaMemcpyDeviceToHost, stream_) != cudaSuccess ||

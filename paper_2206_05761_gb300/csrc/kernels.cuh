@@ -3455,6 +3455,15 @@ static __global__ void k_set_tend(DevState* st, FinishArgs a, double t_end) {
     set_tend_body(st, a, t_end);
 }
 
+// An empty queue of full updates with a number of its own, for a dry pass that
+// no time advance or new end time comes before (the phase call repeated, a
+// profiled step after an abandoned one): appended to the last queue, its leaves
+// would run past the end of the list.
+static __global__ void k_new_queue(DevState* st) {
+    st->nwet = 0u;
+    st->epoch += 1u;
+}
+
 // State from the reductions of the initial (or reloaded) fields: s_max from
 // their maxima, and, if set_dt, dt from rmin_bits.
 __device__ __forceinline__ void init_state_body(DevState* st, const FinishArgs& a, const unsigned long long* max_bits,

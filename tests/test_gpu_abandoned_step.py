@@ -62,3 +62,35 @@ def test_a_new_state_after_an_abandoned_step(matched, how, precision):
     _equal(a, b, leaves=how != "uniform")
     a.close()
     b.close()
+
+
+@pytest.mark.parametrize("matched", [False, True])
+@pytest.mark.parametrize("what", ["step twice", "phases again", "advance", "profile_step", "profile_update"])
+@pytest.mark.parametrize("precision", [64, 32])
+def test_a_step_begun_again(matched, what, precision):
+    # every finest cell is a wet leaf, so that two queues do not fit one list
+    import paper_2206_05761_gb300.hwfv1 as H
+    from paper_2206_05761_gb300.sim import Simulation
+    p, f = synth.bumpy_dam_break(L=L, eps=0.0, seed=5)
+    p = dict(p, flux_match=matched)
+    f = dict(f, h=np.random.default_rng(1).uniform(0.5, 1.0, f["h"].shape))
+    a, b = Simulation(p, f, precision), Simulation(p, f, precision)
+    _begin(a)
+    if what == "step twice":
+        a.fv1()
+        a.decode()
+    elif what == "phases again":
+        a.step()
+    elif what == "advance":
+        a.advance(max_steps=1)
+    elif what == "profile_step":
+        H.hwfv1_profile_step(a.hd)
+    else:
+        H.hwfv1_profile_update(a.hd, 3)
+    b.step()
+    _equal(a, b)
+    ca, cb = a.counters(), b.counters()
+    assert ca[0] == cb[0] == 1 and ca[1] == cb[1] == 4 ** L
+    assert ca[3] == cb[3] == 4 ** L                # full updates: the list's length
+    a.close()
+    b.close()

@@ -103,3 +103,17 @@ def test_no_load_can_move_above_the_wait_for_the_kernel_ahead():
     assert init.index("pdl_ = ") > max(init.index("encode_passes("), init.index("lk(k_flag"))
     assert "lk(" not in init[init.index("pdl_ = "):]
     assert "lk(" not in body_of(src, "void ensure_sig_words(")
+
+
+def test_a_dry_pass_starts_with_an_empty_queue():
+    # every host function that launches the dry pass or a step outside a graph
+    # empties the queue first: by a new end time (advance, uniform steps) or on
+    # its own; appended to an earlier queue, the leaves would leave the list
+    src = source("engine.cuh")
+    for head, start in (("hwfv1_status step()", "launch_fv1("), ("hwfv1_status profile_step(", "launch_step("),
+                        ("hwfv1_status profile_update(", "launch_encode("),
+                        ("hwfv1_status advance(", "launch_step("),
+                        ("hwfv1_status advance_uniform(", "launch_step_uniform(")):
+        b = body_of(src, head)
+        first = min(b.find(x) for x in ("new_queue(", "k_set_tend<<<") if x in b)
+        assert -1 < first < b.index(start), head
