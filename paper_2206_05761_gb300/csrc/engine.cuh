@@ -366,6 +366,10 @@ class EngineT final : public Engine {
                 launch_step_uniform();
             }
         }
+        // the steps set M to the length of their own list; the adaptive one holds
+        // no leaves until the next traversal (hwfv1_step before it would read M
+        // entries that nothing wrote)
+        cudaMemsetAsync(&st_->M, 0, sizeof(uint32_t), stream_);
         return check("advance_uniform");
     }
 

@@ -94,3 +94,21 @@ def test_a_step_begun_again(matched, what, precision):
     assert ca[3] == cb[3] == 4 ** L                # full updates: the list's length
     a.close()
     b.close()
+
+
+@pytest.mark.parametrize("precision", [64, 32])
+def test_the_update_after_uniform_steps_has_no_leaves(precision):
+    # before any traversal: nothing is listed, so nothing is updated or queued
+    from paper_2206_05761_gb300.sim import Simulation
+    p, f = synth.bumpy_dam_break(L=L, eps=1e-3, seed=5)
+    a, b = Simulation(p, f, precision), Simulation(p, f, precision)
+    for s in (a, b):
+        s.advance_uniform(max_steps=2)
+    a.fv1()
+    _equal(a, b, leaves=False)
+    for s in (a, b):
+        s.advance(max_steps=2)
+    _equal(a, b)
+    assert a.counters()[:4] == b.counters()[:4]
+    a.close()
+    b.close()

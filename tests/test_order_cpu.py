@@ -117,3 +117,10 @@ def test_a_dry_pass_starts_with_an_empty_queue():
         b = body_of(src, head)
         first = min(b.find(x) for x in ("new_queue(", "k_set_tend<<<") if x in b)
         assert -1 < first < b.index(start), head
+
+
+def test_uniform_steps_leave_no_length_to_the_adaptive_list():
+    # the uniform steps' M counts a list of their own; hwfv1_step reads M entries
+    # of the adaptive list, of which a handle without a traversal has none
+    b = body_of(source("engine.cuh"), "hwfv1_status advance_uniform(")
+    assert re.search(r"cudaMemsetAsync\(&st_->M, 0, sizeof\(uint32_t\)", b[b.rindex("launch_step_uniform("):])
