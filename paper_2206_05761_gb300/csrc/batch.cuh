@@ -199,27 +199,51 @@ class BatchT final : public Batch {
         cudaGetDevice(&dev);
         cudaDeviceGetAttribute(&nsm_, cudaDevAttrMultiProcessorCount, dev);
         const int D = (int)specs_.size();
+        // out of memory: the members take half of their face buffers
+        bool half = false;
+        auto shrink = [&]() {
+            if (half) return false;
+            half = true;
+            for (auto* e : doms_) e->shrink_faces();
+            return true;
+        };
         for (int d = 0; d < D; ++d) {
             // the batched kernels update every tile (no quiescence bookkeeping),
             // so a member never skips tiles, whichever path advances it
             hwfv1_problem sd = specs_[d];
             sd.flags |= HWFV1_FULL_SWEEP;
-            auto* e = new EngineT<T>(sd, stream_, /*batched=*/true);
-            doms_.push_back(e);
-            const hwfv1_status s = e->init(z[d], h[d], qx[d], qy[d]);
-            if (s != HWFV1_OK) return fail(s, "domain " + std::to_string(d) + ": " + e->err);
+            for (;;) {
+                auto* e = new EngineT<T>(sd, stream_, /*batched=*/true, half);
+                const hwfv1_status s = e->init(z[d], h[d], qx[d], qy[d]);
+                if (s == HWFV1_OK) {
+                    doms_.push_back(e);
+                    break;
+                }
+                const std::string why = e->err;
+                delete e;
+                if (s != HWFV1_ERR_OOM || !shrink()) return fail(s, "domain " + std::to_string(d) + ": " + why);
+            }
         }
-        if (cudaMalloc(&d_plans_, sizeof(DomainPlan<T>) * D) != cudaSuccess ||
-            cudaMalloc(&d_bases_, sizeof(uint32_t) * (D + 1) * BK_KINDS) != cudaSuccess) {
-            cudaGetLastError();
+        auto table = [&](auto** p, size_t bytes) {
+            while (cudaMalloc(p, bytes) != cudaSuccess) {
+                cudaGetLastError();
+                if (!shrink()) return false;
+            }
+            return true;
+        };
+        if (!table(&d_plans_, sizeof(DomainPlan<T>) * D) || !table(&d_bases_, sizeof(uint32_t) * (D + 1) * BK_KINDS))
             return fail(HWFV1_ERR_OOM, "batch tables");
-        }
         return replan(enc_k_, fv1_cells_);
     }
 
     hwfv1_status advance(double t_end, int64_t max_steps) override {
         if (max_steps < 0) return fail(HWFV1_ERR_INVALID_SPEC, "max_steps < 0");
         const int D = (int)doms_.size();
+        // a member gave part of its face buffer up: the plans hold its address
+        bool moved = false;
+        for (auto* e : doms_) moved = e->faces_moved() || moved;
+        if (moved)
+            if (const hwfv1_status s = replan(enc_k_, fv1_cells_); s != HWFV1_OK) return s;
         kb_set_tend<T><<<D, 64, 0, stream_>>>(d_plans_, D, t_end);
         if (!exec_) {
             cudaGraph_t g = nullptr;

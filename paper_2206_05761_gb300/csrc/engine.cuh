@@ -34,10 +34,10 @@ inline int64_t count_kernel_nodes(cudaGraph_t g) {
 template <typename T>
 class EngineT final : public Engine {
    public:
-    // batched: a member of a BatchT, whose own kernels run its steps (no
-    // shared-face buffers)
-    EngineT(const hwfv1_problem& s, cudaStream_t stream, bool batched = false)
-        : spec_(s), stream_(stream), batched_(batched) {
+    // batched: a member of a BatchT, whose own kernels run its steps;
+    // half_faces: half of the face buffer from the start
+    EngineT(const hwfv1_problem& s, cudaStream_t stream, bool batched = false, bool half_faces = false)
+        : spec_(s), stream_(stream), batched_(batched), half_faces_(half_faces) {
         L_ = s.L;
         N_ = 1ull << (2 * L_);
         H_ = hier_size(L_);
@@ -143,10 +143,16 @@ class EngineT final : public Engine {
         dlist_ = counts_ + 2 * ntiles_ + 1;
         // shared faces of the wet-leaf update and a stamp per hierarchy cell.  Float64 only: in
         // float32 the arithmetic saved costs less than the extra launch and
-        // face traffic.
+        // face traffic.  Where the device does not hold the whole buffer, half
+        // of it: 96 bytes a leaf of the full queue, the rest in one pass.
         if (sizeof(T) == 8) {
-            fcap_ = (uint32_t)std::min<uint64_t>(N_, 1ull << 22);
-            if (!alloc(&face_, (size_t)fcap_ * kFaceArrays * sizeof(T))) return oom();
+            fcap_ = (uint32_t)std::min<uint64_t>(N_, 1ull << 22) / (half_faces_ ? 2u : 1u);
+            if (!alloc(&face_, face_bytes())) {
+                if (half_faces_) return oom();
+                half_faces_ = true;
+                fcap_ /= 2u;
+                if (!alloc(&face_, face_bytes())) return oom();
+            }
             if (!alloc(&mark_, H_ * sizeof(unsigned long long))) return oom();
             cudaMemsetAsync(mark_, 0, H_ * sizeof(unsigned long long), stream_);
         }
@@ -391,7 +397,8 @@ class EngineT final : public Engine {
         margin_ = margin;
         const uint64_t npx = 1ull << (2 * (L_ - 4));
         if (!feat_ && !alloc(&feat_, npx * 4 * sizeof(__nv_bfloat16))) return oom();
-        if (!skipwork_reserve(&skw_, (int64_t)npx)) return oom();
+        if (!skipwork_reserve(&skw_, (int64_t)npx) && !(shrink_faces() && skipwork_reserve(&skw_, (int64_t)npx)))
+            return oom();
         if (!side_ && (cudaStreamCreateWithFlags(&side_, cudaStreamNonBlocking) != cudaSuccess ||
                        cudaEventCreateWithFlags(&ev_fork_, cudaEventDisableTiming) != cudaSuccess ||
                        cudaEventCreateWithFlags(&ev_join_, cudaEventDisableTiming) != cudaSuccess))
@@ -1547,16 +1554,56 @@ class EngineT final : public Engine {
     }
     template <typename P>
     bool alloc(P** p, size_t bytes) {
-        void* v = nullptr;
-        keep_pool_memory();
-        if (cudaMallocAsync(&v, bytes, stream_) != cudaSuccess) {
-            cudaGetLastError();
-            return false;
-        }
+        void* const v = pool_alloc(bytes);
+        if (!v) return false;
         allocs_.push_back(v);
         *p = static_cast<P*>(v);
         return true;
     }
+    // device memory, if need be that of half the face buffer (NULL: none)
+    void* pool_alloc(size_t bytes) {
+        void* v = nullptr;
+        keep_pool_memory();
+        while (cudaMallocAsync(&v, bytes, stream_) != cudaSuccess) {
+            cudaGetLastError();
+            if (!shrink_faces()) return nullptr;
+        }
+        return v;
+    }
+    size_t face_bytes() const { return (size_t)fcap_ * kFaceArrays * sizeof(T); }
+
+   public:
+    // Give half of the face buffer back to the pool, for what is allocated
+    // after it: the captured graphs, which hold its address, are captured again
+    // (a batch makes new plans: faces_moved).  The step's results do not depend
+    // on the buffer's size.
+    bool shrink_faces() {
+        if (!face_ || half_faces_) return false;
+        half_faces_ = true;
+        cudaStreamSynchronize(stream_);
+        for (cudaGraphExec_t* g : {&exec_, &exec_multi_, &exec_uniform_})
+            if (*g) {
+                cudaGraphExecDestroy(*g);
+                *g = nullptr;
+            }
+        drop_skip_graphs();
+        allocs_.erase(std::find(allocs_.begin(), allocs_.end(), static_cast<void*>(face_)));
+        cudaFreeAsync(face_, stream_);
+        cudaStreamSynchronize(stream_);
+        face_ = nullptr;
+        fcap_ /= 2u;
+        if (!alloc(&face_, face_bytes())) fcap_ = 0;     // (taken by someone else since: no shared faces)
+        moved_ = true;
+        return true;
+    }
+    // whether the face buffer has moved since the last call
+    bool faces_moved() {
+        const bool m = moved_;
+        moved_ = false;
+        return m;
+    }
+
+   private:
     hwfv1_status oom() { return fail(HWFV1_ERR_OOM, "device allocation failed"); }
     hwfv1_status fail(hwfv1_status s, const std::string& m) {
         err = m;
@@ -1583,12 +1630,8 @@ class EngineT final : public Engine {
     // staging for host transfers: two field slots, stream-ordered on stream_
     // and handed to the copy stream (event 8), freed by the caller on stream_
     hwfv1_status stage_alloc(double** p) {
-        void* v = nullptr;
-        keep_pool_memory();
-        if (cudaMallocAsync(&v, 2 * N_ * sizeof(double), stream_) != cudaSuccess) {
-            cudaGetLastError();
-            return oom();
-        }
+        void* const v = pool_alloc(2 * N_ * sizeof(double));
+        if (!v) return oom();
         *p = static_cast<double*>(v);
         cudaEventRecord(hev_[8], stream_);
         cudaStreamWaitEvent(cstream_, hev_[8], 0);
@@ -1623,6 +1666,8 @@ class EngineT final : public Engine {
     T* face_ = nullptr;                 // shared faces and velocities (kFaceArrays x fcap_)
     std::unordered_map<const void*, int> occ_;   // resident blocks per kernel
     uint32_t fcap_ = 0;
+    bool half_faces_ = false;           // the face buffer is half its full size
+    bool moved_ = false;
     unsigned long long* mark_ = nullptr;   // per hierarchy cell: (epoch + 1) << 32 | queue slot
     uint32_t* scount_ = nullptr;        // per tile: leaves when it holds the bed's flags alone
     uint32_t* work_ = nullptr;          // the traversal's list of tiles to treat one warp each
