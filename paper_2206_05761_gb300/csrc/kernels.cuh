@@ -2250,16 +2250,20 @@ __device__ __forceinline__ void queue_leaf(const StepArgs<T>& a, uint32_t w, uin
 // FV1, first kernel: every leaf whose own and four same-level neighbour
 // depths are exactly zero and that has no inflow gets (+0, +0, +0) -- what
 // the full update computes for it -- decided on the depth bits alone.  Every
-// other leaf is queued for the full update.  Two leaves a thread, so many
-// independent loads are in flight.
+// other leaf is queued for the full update.  Two leaves a thread, a grid stride
+// apart, so many independent loads are in flight.
 //
-// A warp takes 64 leaves in a row (an 8 x 8 patch where they are of one size)
-// and appends its wet ones with one addition to the queue's length, whose
-// latency passes while it forms what the faces read of them.  With an addition
-// for each 32 leaves, all on one word, 1 M wet leaves took 34 us, now 24, and the
-// faces and the update of 1024 x 1024 bumps gain 3 % by the queue's order.  One
-// addition a block would want two barriers: slower where most leaves are dry
-// (2048 x 2048 float32 flood, 32 steps: 780 us, 763 with one per 32, now 745).
+// Bound by the latency of those loads: six blocks of 256 an SM (40 registers),
+// and lanes with dry leaves go on without waiting for the warp's wet ones.  Where
+// a warp formed its 64 leaves' votes and appended them together, at 48 registers
+// and five blocks, a uniform step over dry ground took 145 us at L=12 (now 128;
+// 137 with an addition to the queue's length for each 32 leaves), over the flood
+// at its peak 210 us (191; 190), its full sweep 362 us (348; 355).
+//
+// The wet leaves of a warp's two are appended by one addition to the queue's
+// length, whose latency passes while it forms what the faces read of the first.
+// With an addition for each 32 leaves, all on one word, 1 M wet leaves took 34 us,
+// now 24.
 template <typename T>
 __device__ __forceinline__ void fv1_dry_body(const StepArgs<T>& a, Blk B) {
     DevState* st = a.st;
@@ -2275,14 +2279,12 @@ __device__ __forceinline__ void fv1_dry_body(const StepArgs<T>& a, Blk B) {
     T* const oh = nxt ? a.f[1][0] : a.f[0][0];
     T* const oqx = nxt ? a.f[1][1] : a.f[0][1];
     T* const oqy = nxt ? a.f[1][2] : a.f[0][2];
-    const uint32_t lane = threadIdx.x & 31u, below = (1u << lane) - 1u;
-    const uint32_t warps = B.n * (blockDim.x / 32u);
-    // a list that leaves warps idle at that: 32 leaves a warp
-    const uint32_t per = M > warps * 32u ? 64u : 32u;
-    for (uint32_t b = (B.id * (blockDim.x / 32u) + threadIdx.x / 32u) * per; b < M; b += warps * per) {
-        const uint32_t k = b + lane, k2 = k + 32u;
-        const bool one = k < M, two = k2 < M && per == 64u;
-        const uint32_t p1 = one ? __ldg(a.leaves + k) : 0u, p2 = two ? __ldg(a.leaves + k2) : 0u;
+    const uint32_t lane = threadIdx.x & 31u;
+    const uint32_t stride = B.n * blockDim.x;
+    for (uint32_t k = B.id * blockDim.x + threadIdx.x; k < M; k += 2u * stride) {
+        const uint32_t k2 = k + stride;
+        const bool two = k2 < M;
+        const uint32_t p1 = __ldg(a.leaves + k), p2 = two ? __ldg(a.leaves + k2) : 0u;
         const DryProbe d1 = dry_probe(p1);
         const DryProbe d2 = dry_probe(p2);
         bool y1 = dry5(src.h, d1);
@@ -2298,22 +2300,25 @@ __device__ __forceinline__ void fv1_dry_body(const StepArgs<T>& a, Blk B) {
             y1 = y1 && !inlet_range(a, d1.n, compact16(d1.code), compact16(d1.code >> 1), (1u << d1.n) - 1u, lo, hi);
             y2 = y2 && !inlet_range(a, d2.n, compact16(d2.code), compact16(d2.code >> 1), (1u << d2.n) - 1u, lo, hi);
         }
-        const bool q1 = one && !y1, q2 = two && !y2;
-        const uint32_t m1 = __ballot_sync(0xffffffffu, q1), m2 = __ballot_sync(0xffffffffu, q2);
-        uint32_t w = 0;
-        if (lane == 0 && (m1 | m2) != 0u) w = atomicAdd(&st->nwet, (uint32_t)(__popc(m1) + __popc(m2)));
-        LeafPre<T> r1 = {}, r2 = {};
-        if (q1) r1 = leaf_pre(a, src, d1.iC);
-        if (q2) r2 = leaf_pre(a, src, d2.iC);
-        if (one && y1) store_dry(a, oh, oqx, oqy, d1);
-        if (two && y2) store_dry(a, oh, oqx, oqy, d2);
-        w = __shfl_sync(0xffffffffu, w, 0);
-        if (q1) queue_leaf(a, w + __popc(m1 & below), p1, d1.iC, r1, stamp);
-        if (q2) queue_leaf(a, w + __popc(m1) + __popc(m2 & below), p2, d2.iC, r2, stamp);
+        if (y1) store_dry(a, oh, oqx, oqy, d1);
+        if (y2) store_dry(a, oh, oqx, oqy, d2);
+        const bool q1 = !y1, q2 = two && !y2;
+        if (q1 || q2) {
+            // (the lanes that came here together)
+            const uint32_t m = __activemask(), below = (1u << lane) - 1u, leader = __ffs(m) - 1u;
+            const uint32_t m1 = __ballot_sync(m, q1), m2 = __ballot_sync(m, q2);
+            uint32_t w = 0;
+            if (lane == leader) w = atomicAdd(&st->nwet, (uint32_t)(__popc(m1) + __popc(m2)));
+            LeafPre<T> r = {};
+            if (q1) r = leaf_pre(a, src, d1.iC);
+            w = __shfl_sync(m, w, leader);
+            if (q1) queue_leaf(a, w + __popc(m1 & below), p1, d1.iC, r, stamp);
+            if (q2) queue_leaf(a, w + __popc(m1) + __popc(m2 & below), p2, d2.iC, leaf_pre(a, src, d2.iC), stamp);
+        }
     }
 }
 template <typename T>
-static __global__ void __launch_bounds__(256) k_fv1_dry(StepArgs<T> a) {
+static __global__ void __launch_bounds__(256, 6) k_fv1_dry(StepArgs<T> a) {
     pdl_wait();
     fv1_dry_body<T>(a, this_blk());
 }
