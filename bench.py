@@ -195,7 +195,7 @@ FP64_PEAK_TFLOPS = 152 * 2 * 2.07e9 / 1e12
 # DRAM traffic of the wet-leaf update (k_fv1_faces + k_fv1_update) of one
 # step in the timed window: mean over the launches of the window's ncu
 # launch list (the committed summary under profiles/), valid while
-# kernels.cuh and common.cuh (in that order) have this SHA-256.
+# kernels.cuh, softf64.cuh and common.cuh (in that order) have this SHA-256.
 FV1_WET_TRAFFIC = {"kernels_sha256": "f7425a497b256c00097eabcfed7c4552b54cbb38f3e42b7f2847d38de9446e59",
                    "bytes_per_launch": 7260160 + 17082496 + 1024}
 
@@ -203,7 +203,7 @@ FV1_WET_TRAFFIC = {"kernels_sha256": "f7425a497b256c00097eabcfed7c4552b54cbb38f3
 def kernels_sha256():
     import hashlib
     h = hashlib.sha256()
-    for name in ("kernels.cuh", "common.cuh"):
+    for name in ("kernels.cuh", "softf64.cuh", "common.cuh"):
         with open(os.path.join(ROOT, "paper_2206_05761_gb300", "csrc", name), "rb") as fh:
             h.update(fh.read())
     return h.hexdigest()
@@ -229,6 +229,8 @@ def roofline(kernel, ms, r, args, pk, src):
                 "units_per_launch": r["wet_per_step"], "flop_per_unit": FV1_WET_FLOP_PER_LEAF,
                 "fp64_pipe_per_unit": FV1_WET_PIPE_PER_LEAF,
                 "fp64_pipe_frac": ach / FP64_PEAK_TFLOPS * FV1_WET_PIPE_PER_LEAF / FV1_WET_FLOP_PER_LEAF,
+                "note": "frac and frac_of_measured_fp64 count the operations as written, most of which run as "
+                        "integer instructions; fp64_pipe_frac is the share of the pipe's rate that is used",
                 "peak_source": "derived: FP64 pipe, 2 instructions/clk/SM x 152 SMs x 2.07 GHz, "
                                "1 FLOP per instruction (no FMA)"}
     return {"kernel": kernel, "bound": None, "achieved": None, "peak": pk["hbm_gbs"], "unit": "GB/s",
