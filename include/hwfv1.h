@@ -231,7 +231,12 @@ hwfv1_status hwfv1_get_stats(hwfv1_handle* hd, int64_t* num_leaves, double* smax
  * plain step outside the learned skip) with a CUDA event recorded after
  * every kernel: the step is captured as a graph
  * whose kernels are separated by event-record nodes (HWFV1_NO_GRAPH set:
- * ordinary launches on the handle's stream).  Writes the duration in ms of
+ * ordinary launches on the handle's stream).  The results are the ordinary
+ * step's bit for bit; the kernels are those of the phase calls: where the
+ * plain step's traversal and dry pass are one kernel (k_trav_dry, not with
+ * HWFV1_FULL_SWEEP), a profiled step runs k_trav_classify, k_trav_list and
+ * k_fv1_dry, so that each phase has a time of its own, and their sum lies
+ * above what the ordinary step takes.  Writes the duration in ms of
  * each kernel (from the previous event) to ms[0..cap) and its name (static
  * strings owned by the library) to names[0..cap); either may be NULL;
  * *n = number of kernels.  Advances the simulation by one step and

@@ -3425,8 +3425,9 @@ __device__ __forceinline__ void finish_body(DevState* st, const FinishArgs& a) {
 }
 
 // Decode-back followed, in its last CTA to finish, by the time advance (one
-// launch instead of two).  decode_body reads the state through L2 only, so
-// the last CTA sees every other CTA's reductions after the fence.
+// launch instead of two).  finish_body reads the state through L2 (__ldcg), so
+// the last CTA sees every other CTA's reductions after the fence, whatever
+// lines decode_body left in L1.
 //
 // Only the first min(ndec, grid) CTAs (at least one) take part: the others
 // have no tile to decode (decode_body strides over the list by the grid)
